@@ -64,6 +64,7 @@ void free_plan_memory(sht_plan_s* p) {
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (p->split) split_tables_destroy(p);
+    if (p->slice) slice64_destroy(p);
     if (p->ragged) {
         ragged_free(p->ragged);
         p->ragged = nullptr;
@@ -280,6 +281,7 @@ extern "C" int sht_plan_create_grid(int N, int J, int I, int nfields, int precis
         if (e == cudaSuccess) e = build_pnm_table(p, s);
         if (e == cudaSuccess) e = build_twiddles(p, s);
         if (e == cudaSuccess && !fp64) e = split_tables_create(p, s);
+        if (e == cudaSuccess && fp64) e = slice64_create(p, s);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e != cudaSuccess) {
             if (e == cudaErrorNotSupported) {

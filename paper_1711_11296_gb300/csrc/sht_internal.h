@@ -78,6 +78,7 @@ struct InvScale {
 };
 
 struct SplitTables;   // tensor-core operand tables (split plans)
+struct Slice64;       // tensor-core operand slices (FP64 plans)
 
 // Reduced grid: latitude j carries its own number I_j of longitudes.  The
 // distinct half-lengths L = I_j/2 each have an FFT shape and tables; their
@@ -190,6 +191,8 @@ struct sht_plan_s {
     int* d_jmin;               // FP64 plans with the reduced transform: [2(N+1)]
                                // first node with some |P~| >= 1e-16 (null: off)
     sht::SplitTables* split;   // null for FP64 plans
+    sht::Slice64* slice;       // FP64 plans whose contractions run on the tensor
+                               // cores (else null)
     unsigned* d_colmax;        // FP16 split plans: [2][2F] column maxima (float bits)
                                // of the forward and inverse GEMMs' FP32 operand
     sht::Profiler* prof;       // per-launch timing, off by default
@@ -305,6 +308,14 @@ cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,
                                      double* spec, cudaStream_t s);
 cudaError_t launch_legendre_inv_fp64(const sht_plan_s* p, const double* spec,
                                      double* work, cudaStream_t s);
+
+// FP64 contractions on the tensor cores (sht_slice64.cu): plan tables (none
+// where the FP64 pipe is faster) and the launches launch_legendre_*_fp64
+// hand over to when the plan has them.
+cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s);
+void slice64_destroy(sht_plan_s* p);
+cudaError_t launch_legendre_slice64(const sht_plan_s* p, bool inverse, const double* in,
+                                    double* out, cudaStream_t s);
 
 __host__ __device__ inline size_t coef_offset(int N, int m) {
     return (size_t)m * (N + 1) - (size_t)m * (m - 1) / 2;

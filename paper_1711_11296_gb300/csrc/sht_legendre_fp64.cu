@@ -185,6 +185,20 @@ __global__ void __launch_bounds__(NT) legendre_inv_fp64_group_kernel(
 cudaError_t launch_legendre_fp64_group(sht_plan_s* const* plans, int n, bool inverse,
                                        const void* const* in, void* const* out,
                                        const int4* tiles, int ntiles, cudaStream_t s) {
+    // a plan with tensor-core tables fills the GPU by itself: per-plan launches
+    bool sliced = false;
+    for (int q = 0; q < n; ++q) sliced = sliced || plans[q]->slice;
+    if (sliced) {
+        for (int q = 0; q < n; ++q) {
+            const cudaError_t e =
+                inverse ? launch_legendre_inv_fp64(plans[q], static_cast<const double*>(in[q]),
+                                                   static_cast<double*>(out[q]), s)
+                        : launch_legendre_fwd_fp64(plans[q], static_cast<const double*>(in[q]),
+                                                   static_cast<double*>(out[q]), s);
+            if (e) return e;
+        }
+        return cudaSuccess;
+    }
     LegGroup G;
     G.n = n;
     for (int q = 0; q < n; ++q) {
@@ -227,6 +241,7 @@ void build_legendre_tiles(int N, int Jh, int C, std::vector<int4>& fwd,
 
 cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,
                                      double* spec, cudaStream_t s) {
+    if (p->slice) return launch_legendre_slice64(p, false, work, spec, s);
     if (p->ntiles_fwd == 0) return cudaSuccess;
     legendre_fwd_fp64_kernel<<<p->ntiles_fwd, NT, 0, s>>>(
         p->d_pnm, p->ldp, work, spec, p->d_tiles_fwd, p->N, p->Jh, 2 * p->F, p->d_jmin);
@@ -236,6 +251,7 @@ cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,
 
 cudaError_t launch_legendre_inv_fp64(const sht_plan_s* p, const double* spec,
                                      double* work, cudaStream_t s) {
+    if (p->slice) return launch_legendre_slice64(p, true, spec, work, s);
     if (p->ntiles_inv == 0) return cudaSuccess;
     legendre_inv_fp64_kernel<<<p->ntiles_inv, NT, 0, s>>>(
         p->d_pnm, p->ldp, spec, work, p->d_tiles_inv, p->N, p->Jh, 2 * p->F, p->d_jmin);

@@ -1,0 +1,767 @@
+// FP64 Legendre contractions on the 5th-generation tensor cores, by an
+// error-free split of both operands into 8-bit slices (Ozaki's scheme for
+// matrix products, with balanced base-256 digits).
+//
+// The FP64 pipe of GB300 does 2 multiply-adds per clock and SM, so the
+// 2.7e11 flops of a T639 x 256 pair take 241 ms on it at its full rate
+// (sht_legendre_fp64.cu).  The tensor cores do about 1700 times as many
+// BF16 products, and BF16 holds every integer up to 256 exactly.  Measured
+// (us, forward / inverse contraction, FP64 pipe -> slices): T639 x 256
+// 120600 / 117800 -> 6650 / 6570; T319 x 100 8530 / 8090 -> 673 / 952;
+// T159 x 256 2721 / 2411 -> 310 / 327.
+//
+// Every row r of A (the P~ table) and every column c of B (the Fourier data
+// or the spectrum) is scaled by a power of two to an integer of at most
+// 2^sh (sh = 53..55, more bits than the 53 of the input for all but the
+// entries far below their row's or column's largest), written with seven
+// digits d_0 .. d_6 in [-128, 128], value = sum_a d_a 256^(6 - a).  Digit a
+// is stored as the BF16 number d_a 2^(-8a) in slice a.  A product of two
+// slices sums integers below 2^24 in the FP32 accumulators, which is exact;
+// the products of equal a + b share an accumulator:
+//   a + b = 0, 1, 2, 3, 4 | 5, 6, 7 together,
+// 34 products of the 49 (the 15 left out are below 2^-60 of row times
+// column maximum, under the rounding of the operands).  The last
+// accumulator rounds at 2^-24 of its leading term, 2^-62 of the maxima.
+// The epilogue adds the six sums as a 64-bit integer, converts it once and
+// scales it back, so an output carries the operands' rounding (2^-56 of the
+// row and column maxima) and one final rounding: less than the sum of K
+// FP64 products accumulates (T319 synthesis against 113-bit sums over the
+// same table: 3.6e-16, FP64 pipe 6.6e-16).
+//
+// Per transform: slice_b_kernel reads the K x C operand of each (m, parity)
+// problem once, finds the column exponents and writes the slices in the
+// K-major core-matrix layout; slice_gemm_kernel multiplies, both operands
+// arriving by bulk copies.  The slices of A are made once per plan.
+#include <limits.h>
+
+#include <algorithm>
+#include <new>
+#include <vector>
+
+#include "sht_internal.h"
+#include "sht_tc.h"
+
+namespace sht {
+
+constexpr int kSlices = 7;
+
+struct S64Prob {
+    long long a_off;     // byte offset of the problem's A slices in the table
+    long long b_off;     // byte offset of its B slices in the slice buffer
+    long long src_off;   // double offset of B row 0 in the operand
+    long long o_off;     // double offset of output row 0
+    int R, R16;          // rows of A, rounded up to 16
+    int K, nkt;          // depth, and its K slabs of 16
+    int src_stride, o_stride;
+    int ea_off;          // first row in the exponent table
+    int sh;              // operands are scaled below 2^sh
+    int wide;            // the sum of the accumulators may need more than 63 bits
+};
+
+// One pass of slice_b + GEMM: problems [p0, p1), tiles [t0, t1).
+struct S64Chunk { int p0, p1, t0, t1; };
+
+struct S64Dir {
+    bool mcols = true;              // the MMA's 128-wide M side holds columns (else rows)
+    unsigned char* table = nullptr; // A slices: per problem [K slab][slice][R16][16]
+    int* ea = nullptr;              // exponent of every row of A
+    S64Prob* d_probs = nullptr;
+    int4* d_tiles = nullptr;        // {problem, m0, n0, -}
+    std::vector<S64Chunk> chunks;
+    int maxK = 0;
+};
+
+struct Slice64 {
+    S64Dir dir[2];                  // forward, inverse
+    unsigned char* bbuf = nullptr;  // B slices of one chunk: [K slab][slice][C16][16]
+    int* eb = nullptr;              // [problem][C16] column exponents
+    int C16 = 0;
+};
+
+namespace {
+
+constexpr int TM = 128, TN = 64, TK = 16;   // MMA tile: M x N, K slab
+constexpr int NSTAGE = 5;
+constexpr int M_SLICE = TM * TK * 2, N_SLICE = TN * TK * 2;   // bytes
+constexpr int STAGE = kSlices * (M_SLICE + N_SLICE);          // 43 KB
+constexpr int NACC = 6;                     // accumulators of TN TMEM columns
+constexpr int TMEM_COLS = 512;
+constexpr int NBAR = 2 * NSTAGE + 3;
+constexpr int SMEM = NSTAGE * STAGE + 256;
+static_assert(SMEM <= 227 * 1024 && 8 * NBAR + 16 <= 256, "one CTA's shared memory");
+constexpr int NEPI = 256;                   // epilogue threads (8 warps)
+constexpr int NT = NEPI + 64;               // + copy warp + MMA warp
+constexpr int kNonFinite = INT_MAX;         // column exponent of Inf / NaN columns
+
+// ---- slicing -------------------------------------------------------------
+
+// |v| < 2^e for v with biased exponent field eb: e = max(eb, 1) - 1022.
+__device__ __forceinline__ int exp_field(double v) {
+    return (int)((__double_as_longlong(v) >> 52) & 0x7ff);
+}
+
+// v 2^(sh - e), e = exponent of the row or column maximum (biased field
+// emax), rounded to nearest; |result| <= 2^sh.  Integer arithmetic: the FP64
+// pipe would take longer than the memory traffic.
+__device__ __forceinline__ long long to_fixed(double v, int emax, int sh) {
+    const long long bits = __double_as_longlong(v);
+    const int ex = (int)((bits >> 52) & 0x7ff);
+    long long man = bits & 0xfffffffffffffll;
+    if (ex) man |= 0x10000000000000ll;
+    man <<= sh - 53;
+    const int d = min(max(emax, 1) - max(ex, 1), 62);
+    man = (man + ((1ll << d) >> 1)) >> d;
+    return bits < 0 ? -man : man;
+}
+
+// The 16 bytes (one core-matrix row: 8 K values) of slice a of the
+// integers x, biased by 128 in every digit so that digit a is
+// (x >> 8 (6 - a)) & 0xff, minus 128 (the top digit has 9 bits).
+__device__ __forceinline__ uint4 slice8(const long long (&x)[8], int a) {
+    const float w = __uint_as_float((unsigned)(127 - 8 * a) << 23);   // 2^(-8a)
+    unsigned h[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const unsigned dig = a == 0 ? (unsigned)(x[e] >> 48) & 0x1ffu
+                                    : (unsigned)(x[e] >> (8 * (6 - a))) & 0xffu;
+        // 2^23 + digit + 128, less 2^23 + 128; exact, as is the scaling, and
+        // the 8 significant bits fill the upper half of the FP32 word
+        h[e] = __float_as_uint((__uint_as_float(0x4B000000u | dig) - 8388736.f) * w);
+    }
+    return make_uint4(__byte_perm(h[0], h[1], 0x7632), __byte_perm(h[2], h[3], 0x7632),
+                      __byte_perm(h[4], h[5], 0x7632), __byte_perm(h[6], h[7], 0x7632));
+}
+
+__device__ __forceinline__ long long bias(long long x) { return x + 0x80808080808080ll; }
+
+// Byte offset of (row, K group k8 of the slab) within one slice.
+__device__ __forceinline__ int core_off(int row, int k8) {
+    return ((row >> 3) * 2 + k8) * 128 + (row & 7) * 16;
+}
+
+// Slices of the operand B of problems p0 + blockIdx.x, columns 32
+// blockIdx.y + lane; warp w takes the groups of 8 K rows w, w + 16, ....
+// NG > 0: at most NG groups per warp, held in registers between the
+// exponent pass and the slicing (one read of B, which bounds the kernel
+// together with the 14 bytes written per value); NG = 0: any K, read twice.
+// Inverse: the Equator row (node Jh - 1), which the tiles leave out so that
+// they cover J - 1 nodes in whole tiles, is summed here in FP64 (odd parity:
+// P~(0) = 0).
+template <int NG, bool INV>
+__global__ void __launch_bounds__(512)
+    slice_b_kernel(const double* __restrict__ B, const S64Prob* __restrict__ probs, int p0, int C,
+                   int C16, unsigned char* __restrict__ out, int* __restrict__ eb,
+                   const double* __restrict__ pnm, int ldp, int N, int Jh,
+                   double* __restrict__ O) {
+    __shared__ int red[16][32];
+    __shared__ double redq[16][32];
+    const int p = p0 + blockIdx.x;
+    const S64Prob pr = probs[p];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c = blockIdx.y * 32 + lane;
+    const bool cin = c < C;
+    const double* col = B + pr.src_off + c;
+    auto load = [&](int k) -> double {
+        return (k < pr.K && cin) ? __ldg(col + (long long)k * pr.src_stride) : 0.0;
+    };
+    const int ng = 2 * pr.nkt;
+    double v[NG > 0 ? 8 * NG : 8];
+    int ex = 0;
+    if constexpr (NG > 0) {
+#pragma unroll
+        for (int i = 0; i < NG; ++i)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[8 * i + e] = load((w + 16 * i) * 8 + e);
+#pragma unroll
+        for (int i = 0; i < 8 * NG; ++i) ex = max(ex, exp_field(v[i]));
+    } else {
+        for (int g = w; g < ng; g += 16) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = load(g * 8 + e);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) ex = max(ex, exp_field(v[e]));
+        }
+    }
+    if (INV) {
+        double acc = 0.0;
+        if ((p & 1) == 0) {
+            const double* pe = pnm + coef_offset(N, p >> 1) * ldp + (Jh - 1);
+            if constexpr (NG > 0) {
+#pragma unroll
+                for (int i = 0; i < NG; ++i)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int k = (w + 16 * i) * 8 + e;
+                        if (k < pr.K) acc = fma(__ldg(pe + 2 * (size_t)k * ldp), v[8 * i + e], acc);
+                    }
+            } else {
+                for (int g = w; g < ng; g += 16)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int k = g * 8 + e;
+                        if (k < pr.K) acc = fma(__ldg(pe + 2 * (size_t)k * ldp), load(k), acc);
+                    }
+            }
+        }
+        redq[w][lane] = acc;
+    }
+    red[w][lane] = ex;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) ex = max(ex, red[i][lane]);
+    if (w == 0 && c < C16)
+        eb[(size_t)p * C16 + c] = ex == 0x7ff ? kNonFinite : max(ex, 1) - 1022;
+    if (INV && w == 1 && cin) {
+        double acc = redq[0][lane];
+#pragma unroll
+        for (int i = 1; i < 16; ++i) acc += redq[i][lane];
+        O[pr.o_off + (long long)(Jh - 1) * pr.o_stride + c] = acc;
+    }
+    if (c >= C16) return;
+    unsigned char* dst = out + pr.b_off;
+    auto put = [&](int g, const double* x8) {
+        long long x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = bias(to_fixed(x8[e], ex, pr.sh));
+        unsigned char* d = dst + (long long)(g >> 1) * kSlices * C16 * 32 + core_off(c, g & 1);
+#pragma unroll
+        for (int a = 0; a < kSlices; ++a)
+            *reinterpret_cast<uint4*>(d + (long long)a * C16 * 32) = slice8(x, a);
+    };
+    if constexpr (NG > 0) {
+#pragma unroll
+        for (int i = 0; i < NG; ++i)
+            if (w + 16 * i < ng) put(w + 16 * i, v + 8 * i);
+    } else {
+        for (int g = w; g < ng; g += 16) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = load(g * 8 + e);
+            put(g, v);
+        }
+    }
+}
+
+// Row exponents (biased fields) of the table A of every problem.  Forward:
+// rows n, K = nodes (a warp per row); inverse: rows = nodes, K = degrees (a
+// thread per row).
+__global__ void table_exp_kernel(const double* __restrict__ pnm, int ldp, int N,
+                                 const S64Prob* __restrict__ probs, int inverse, int* ea) {
+    const int p = blockIdx.x;
+    const S64Prob pr = probs[p];
+    const double* P = pnm + (coef_offset(N, p >> 1) + (p & 1)) * ldp;
+    if (!inverse) {
+        const int lane = threadIdx.x & 31;
+        for (int r = threadIdx.x >> 5; r < pr.R16; r += blockDim.x >> 5) {
+            int ex = 0;
+            if (r < pr.R)
+                for (int k = lane; k < pr.K; k += 32) ex = max(ex, exp_field(P[2 * (size_t)r * ldp + k]));
+            ex = __reduce_max_sync(0xffffffffu, ex);
+            if (lane == 0) ea[pr.ea_off + r] = ex;
+        }
+    } else {
+        for (int r = threadIdx.x; r < pr.R16; r += blockDim.x) {
+            int ex = 0;
+            if (r < pr.R)
+                for (int k = 0; k < pr.K; ++k) ex = max(ex, exp_field(P[2 * (size_t)k * ldp + r]));
+            ea[pr.ea_off + r] = ex;
+        }
+    }
+}
+
+// Slices of A, one thread per (row, group of 8 K values).
+__global__ void table_slice_kernel(const double* __restrict__ pnm, int ldp, int N,
+                                   const S64Prob* __restrict__ probs, int inverse,
+                                   const int* __restrict__ ea, unsigned char* __restrict__ out) {
+    const int p = blockIdx.x;
+    const S64Prob pr = probs[p];
+    const double* P = pnm + (coef_offset(N, p >> 1) + (p & 1)) * ldp;
+    const int ng = 2 * pr.nkt;
+    const long long units = (long long)ng * pr.R16;
+    for (long long u = (long long)blockIdx.y * blockDim.x + threadIdx.x; u < units;
+         u += (long long)gridDim.y * blockDim.x) {
+        // neighbouring threads: neighbouring K groups (forward, rows of the
+        // table contiguous in K) or neighbouring rows (inverse)
+        const int r = inverse ? (int)(u % pr.R16) : (int)(u / ng);
+        const int g = inverse ? (int)(u / pr.R16) : (int)(u % ng);
+        const int ex = ea[pr.ea_off + r];
+        long long x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int k = g * 8 + e;
+            const double v = (r < pr.R && k < pr.K)
+                                 ? (inverse ? P[2 * (size_t)k * ldp + r] : P[2 * (size_t)r * ldp + k])
+                                 : 0.0;
+            x[e] = bias(to_fixed(v, ex, pr.sh));
+        }
+        unsigned char* d =
+            out + pr.a_off + (long long)(g >> 1) * kSlices * pr.R16 * 32 + core_off(r, g & 1);
+#pragma unroll
+        for (int a = 0; a < kSlices; ++a)
+            *reinterpret_cast<uint4*>(d + (long long)a * pr.R16 * 32) = slice8(x, a);
+    }
+}
+
+// ---- the product ------------------------------------------------------------
+
+struct S64Args {
+    const unsigned char* table;
+    const unsigned char* bbuf;
+    const S64Prob* probs;
+    const int4* tiles;
+    int ntiles;
+    double* O;
+    const int* ea;
+    const int* eb;
+    const int* jmin;   // reduced transform (Sec. 4.1): first significant node per problem
+    int inverse;
+    int C, C16;
+    int* status;
+};
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// d 2^k for an integer-valued d (0 or 2^0 <= |d| < 2^63).
+__device__ __forceinline__ double scale2(double d, int k) {
+    const long long bits = __double_as_longlong(d);
+    const int e = (int)((bits >> 52) & 0x7ff) + k;
+    if (d == 0.0) return 0.0;
+    if (e > 0 && e < 0x7ff) return __longlong_as_double(bits + ((long long)k << 52));
+    return scalbn(d, k);
+}
+
+// Persistent CTAs, one per SM: 128 x 64 tiles (M x N) with six FP32
+// accumulators (384 of the 512 TMEM columns), K slabs of 16 through a ring
+// of 5 stages of 43 KB (14 slices).  Warps 0-7 the epilogue, warp 8 the bulk
+// copies (a lane per slice), one thread of warp 9 the 34 MMAs of a stage.
+// The ring runs on across tiles, so the next tile's operands load during
+// the epilogue.
+// Per stage the MMAs read 34 x 6 KB of shared memory (48 cycles each at 128
+// bytes per clock, against 32 at the tensor rate): that port bounds the
+// main loop.
+template <bool MCOLS>
+__global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant__ S64Args g) {
+    extern __shared__ __align__(1024) unsigned char s64_smem[];
+    unsigned char* smem = s64_smem;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NSTAGE * STAGE);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + NSTAGE * STAGE + 8 * NBAR);
+    volatile int* abort_flag =
+        reinterpret_cast<volatile int*>(smem + NSTAGE * STAGE + 8 * NBAR + 8);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t bar0 = smem_u32(bars);
+    auto full = [&](int s) { return bar0 + 8u * s; };
+    auto empty = [&](int s) { return bar0 + 8u * (NSTAGE + s); };
+    const uint32_t done = bar0 + 8u * (2 * NSTAGE);   // a tile's accumulators complete
+    const uint32_t acc_empty = done + 8u;             // read out by the epilogue
+    const uint32_t fin = done + 16u;                  // every MMA of the CTA complete
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NSTAGE; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        mbar_init(done, 1);
+        mbar_init(acc_empty, NEPI);
+        mbar_init(fin, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+
+    // first K slab and number of slabs of a tile (the reduced transform skips
+    // forward slabs, and inverse tiles whose outputs are then zero, of nodes
+    // before the first significant one)
+    auto range = [&](const S64Prob& pr, const int4& t, int& kb) -> int {
+        kb = 0;
+        if (!g.jmin) return pr.nkt;
+        const int j0 = g.jmin[t.x];
+        if (g.inverse) {
+            const int last = MCOLS ? t.z + TN : t.y + TM;
+            return last <= j0 ? 0 : pr.nkt;
+        }
+        kb = min(j0 / TK, pr.nkt);
+        return pr.nkt - kb;
+    };
+    auto aborted = [&]() { return __any_sync(0xffffffffu, *abort_flag != 0) != 0; };
+
+    if (warp == NEPI / 32) {
+        // ---- bulk copies: lane a < 7 slice a of M, lane 7 + a slice a of N ----
+        uint32_t q = 0, issued = 0;
+        bool ok = true;
+        for (int tt = blockIdx.x; tt < g.ntiles && ok && !aborted(); tt += gridDim.x) {
+            const int4 t = g.tiles[tt];
+            const S64Prob pr = g.probs[t.x];
+            int kb;
+            const int nst = range(pr, t, kb);
+            const int mrows = MCOLS ? g.C16 : pr.R16, nrows = MCOLS ? pr.R16 : g.C16;
+            const int hm = min(TM, mrows - t.y), hn = min(TN, nrows - t.z);
+            const unsigned char* mb =
+                (MCOLS ? g.bbuf + pr.b_off : g.table + pr.a_off) + (long long)t.y * 32;
+            const unsigned char* nb =
+                (MCOLS ? g.table + pr.a_off : g.bbuf + pr.b_off) + (long long)t.z * 32;
+            for (int li = 0; li < nst; ++li, ++q) {
+                const int s = q % NSTAGE;
+                if (lane == 0) {
+                    ok = mbar_wait(empty(s), ((q / NSTAGE) & 1u) ^ 1u, abort_flag);
+                    if (ok) mbar_expect_tx(full(s), (uint32_t)(kSlices * 32 * (hm + hn)));
+                }
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (!ok) break;
+                issued = q + 1;
+                const long long kt = kb + li;
+                const uint32_t st = smem_u32(smem + s * STAGE);
+                if (lane < kSlices) {
+                    bulk_g2s(st + lane * M_SLICE, mb + (kt * kSlices + lane) * mrows * 32,
+                             (uint32_t)hm * 32, full(s));
+                } else if (lane < 2 * kSlices) {
+                    const int a = lane - kSlices;
+                    bulk_g2s(st + kSlices * M_SLICE + a * N_SLICE,
+                             nb + (kt * kSlices + a) * nrows * 32, (uint32_t)hn * 32, full(s));
+                }
+                __syncwarp();
+            }
+        }
+        // after an abort, let the copies in flight land (bounded)
+        if (lane == 0 && *abort_flag) {
+            for (uint32_t j = issued > (uint32_t)NSTAGE ? issued - NSTAGE : 0u; j < issued; ++j) {
+                const long long t0 = clock64();
+                while (!mbar_try(full(j % NSTAGE), (j / NSTAGE) & 1u) &&
+                       clock64() - t0 < kWaitCycles) {
+                }
+            }
+        }
+    } else if (warp == NEPI / 32 + 1) {
+        if (lane == 0) {
+            uint32_t q = 0, nacc = 0;
+            bool ok = true;
+            for (int tt = blockIdx.x; tt < g.ntiles && ok && !*abort_flag; tt += gridDim.x) {
+                const int4 t = g.tiles[tt];
+                const S64Prob pr = g.probs[t.x];
+                int kb;
+                const int nst = range(pr, t, kb);
+                if (nst == 0) continue;
+                const int hn = min(TN, (MCOLS ? pr.R16 : g.C16) - t.z);
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
+                                       ((uint32_t)(hn >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+                if (nacc > 0 && !(ok = mbar_wait(acc_empty, (nacc - 1) & 1u, abort_flag))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (int li = 0; li < nst; ++li, ++q) {
+                    const int s = q % NSTAGE;
+                    if (!(ok = mbar_wait(full(s), (q / NSTAGE) & 1u, abort_flag))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t st = smem_u32(smem + s * STAGE);
+                    const uint64_t md = sdesc(st, 128, 256);
+                    const uint64_t nd = sdesc(st + kSlices * M_SLICE, 128, 256);
+#pragma unroll
+                    for (int a = 0; a < kSlices; ++a) {
+#pragma unroll
+                        for (int b = 0; b < kSlices; ++b) {
+                            if (a + b > 7) continue;
+                            const int acc = a + b < NACC ? a + b : NACC - 1;
+                            // (0, b) opens accumulator b
+                            const uint32_t add = (li > 0 || !(a == 0 && b < NACC)) ? 1u : 0u;
+                            mma_f16_rt(tmem + acc * TN, md + (uint64_t)(a * M_SLICE / 16),
+                                       nd + (uint64_t)(b * N_SLICE / 16), idesc, add);
+                        }
+                    }
+                    mma_commit(empty(s));
+                }
+                if (!ok) break;
+                mma_commit(done);
+                ++nacc;
+            }
+            mma_commit(fin);
+        }
+    } else {
+        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (the M
+        // side), N columns 32 (w / 4) .. +31 ----
+        uint32_t nacc = 0;
+        bool ok = true;
+        const int lq = warp & 3, half = warp >> 2;
+        for (int tt = blockIdx.x; tt < g.ntiles && ok && !aborted(); tt += gridDim.x) {
+            const int4 t = g.tiles[tt];
+            const S64Prob pr = g.probs[t.x];
+            int kb;
+            const int nst = range(pr, t, kb);
+            const bool have = nst > 0;
+            if (have) ok = mbar_wait(done, nacc & 1u, abort_flag);
+            ok = __all_sync(0xffffffffu, ok) != 0;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int im = t.y + 32 * lq + lane;           // this lane's M index
+            const int mv = MCOLS ? g.C : pr.R, nv = MCOLS ? pr.R : g.C;
+            const bool mok = im < mv && ok;
+            const int* ebp = g.eb + (size_t)t.x * g.C16;
+            const int* eap = g.ea + pr.ea_off;
+            auto row_exp = [&](int r) { return max(__ldg(eap + r), 1) - 1022; };
+            const int em = mok ? (MCOLS ? __ldg(ebp + im) : row_exp(im)) : 0;
+            double* om = g.O + pr.o_off + (MCOLS ? (long long)im : (long long)im * pr.o_stride);
+            const long long on = MCOLS ? pr.o_stride : 1;
+            const int k0 = 56 - 2 * pr.sh;
+            for (int i0 = half * 32; i0 < half * 32 + 32; i0 += 8) {
+                const int n0 = t.z + i0;
+                if (n0 >= nv || !ok) break;   // uniform over the warp
+                uint32_t r[NACC][8];
+                if (have) {
+#pragma unroll
+                    for (int s = 0; s < NACC; ++s)
+                        tmem_ld8(tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(s * TN + i0), r[s]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int in = n0 + i;
+                    if (!mok || in >= nv) continue;
+                    double d = 0.0;
+                    if (have) {
+                        const int en = MCOLS ? row_exp(in) : __ldg(ebp + in);
+                        // sum of the accumulators in units of 2^-40 (the first
+                        // apart where 64 bits may not hold it)
+                        const int lead = __float2int_rn(__uint_as_float(r[0][i]));
+                        long long T = pr.wide ? 0 : lead;
+#pragma unroll
+                        for (int s = 1; s < NACC; ++s)
+                            T = (T << 8) + __float2int_rn(__uint_as_float(r[s][i]) *
+                                                          (float)(1ull << (8 * s)));
+                        double sum = (double)T;
+                        if (pr.wide) sum = fma((double)lead, 1099511627776.0, sum);
+                        const int ec = MCOLS ? em : en;
+                        d = ec == kNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                             : scale2(sum, em + en + k0);
+                    }
+                    om[in * on] = d;
+                }
+            }
+            if (have && ok) {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                mbar_arrive(acc_empty);
+                ++nacc;
+            }
+        }
+    }
+    if (*abort_flag && threadIdx.x == 0 && g.status) atomicOr(g.status, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        const long long t0 = clock64();
+        while (!mbar_try(fin, 0) && clock64() - t0 < kWaitCycles) {
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(TMEM_COLS)
+                     : "memory");
+    }
+}
+
+// ---- host ---------------------------------------------------------------------
+
+constexpr size_t kChunkBytes = 1ull << 30;   // B slices of one pass
+
+struct HostDir {
+    std::vector<S64Prob> probs;
+    std::vector<int4> tiles;
+    long long table_bytes = 0, ea_rows = 0;
+    size_t bbytes = 0;   // the largest chunk's B slices
+};
+
+void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
+    const int nprob = 2 * (N + 1), C16 = (C + 15) / 16 * 16;
+    h.probs.assign(nprob, S64Prob{});
+    long long mac_cols = 0, mac_rows = 0;   // padded MMA work of either orientation
+    for (int p = 0; p < nprob; ++p) {
+        const int m = p >> 1, q = p & 1, dd = N - m - q;
+        const int Rn = dd >= 0 ? dd / 2 + 1 : 0;   // degrees of this parity
+        const long long row0 = (long long)coef_offset(N, m) + q;
+        S64Prob& s = h.probs[p];
+        s.R = inverse ? Jh - 1 : Rn;
+        s.K = inverse ? Rn : Jh;
+        s.R16 = (s.R + 15) / 16 * 16;
+        s.nkt = (s.K + TK - 1) / TK;
+        // K products of the leading digits (up to 2^(sh - 48)) fit the 24
+        // bits that FP32 adds exactly; the six accumulators fit one 64-bit
+        // integer (K 2^14 2^40 and the rest below 2^63) up to K = 480
+        s.sh = s.K <= 1024 ? 55 : 54;
+        s.wide = s.K > 480;
+        s.src_off = inverse ? row0 * C : (long long)p * Jh * C;
+        s.src_stride = inverse ? 2 * C : C;
+        s.o_off = inverse ? (long long)p * Jh * C : row0 * C;
+        s.o_stride = inverse ? C : 2 * C;
+        s.a_off = h.table_bytes;
+        h.table_bytes += (long long)s.nkt * kSlices * s.R16 * 32;
+        s.ea_off = (int)h.ea_rows;
+        h.ea_rows += s.R16;
+        d.maxK = std::max(d.maxK, s.K);
+        mac_cols += (long long)s.nkt * ((C16 + TM - 1) / TM * TM) * s.R16;
+        mac_rows += (long long)s.nkt * ((s.R16 + TM - 1) / TM * TM) * C16;
+    }
+    d.mcols = mac_cols <= mac_rows;
+    S64Chunk ch{0, 0, 0, 0};
+    size_t used = 0;
+    for (int p = 0; p < nprob; ++p) {
+        S64Prob& s = h.probs[p];
+        const size_t need = (size_t)s.nkt * kSlices * C16 * 32;
+        if (used > 0 && used + need > kChunkBytes) {
+            ch.p1 = p;
+            ch.t1 = (int)h.tiles.size();
+            d.chunks.push_back(ch);
+            ch = S64Chunk{p, p, ch.t1, ch.t1};
+            used = 0;
+        }
+        s.b_off = (long long)used;
+        used += need;
+        h.bbytes = std::max(h.bbytes, used);
+        const int mr = d.mcols ? C16 : s.R16, nr = d.mcols ? s.R16 : C16;
+        for (int m0 = 0; m0 < mr; m0 += TM)
+            for (int n0 = 0; n0 < nr; n0 += TN) h.tiles.push_back(make_int4(p, m0, n0, 0));
+    }
+    ch.p1 = nprob;
+    ch.t1 = (int)h.tiles.size();
+    d.chunks.push_back(ch);
+}
+
+template <bool INV>
+void launch_slice_b(int maxK, dim3 grid, cudaStream_t s, const double* B, const S64Prob* probs,
+                    int p0, int C, int C16, unsigned char* out, int* eb, const double* pnm,
+                    int ldp, int N, int Jh, double* O) {
+    using Fn = void (*)(const double*, const S64Prob*, int, int, int, unsigned char*, int*,
+                        const double*, int, int, int, double*);
+    static const Fn tab[7] = {slice_b_kernel<0, INV>, slice_b_kernel<1, INV>,
+                              slice_b_kernel<2, INV>, slice_b_kernel<3, INV>,
+                              slice_b_kernel<4, INV>, slice_b_kernel<5, INV>,
+                              slice_b_kernel<6, INV>};
+    const int ng = (maxK + 127) / 128;
+    tab[ng <= 6 ? ng : 0]<<<grid, 512, 0, s>>>(B, probs, p0, C, C16, out, eb, pnm, ldp, N, Jh, O);
+}
+
+cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, double* O,
+                       cudaStream_t s) {
+    const Slice64* sl = p->slice;
+    const S64Dir& d = sl->dir[inverse ? 1 : 0];
+    const int C = 2 * p->F;
+    const void* fn = d.mcols ? (const void*)slice_gemm_kernel<true>
+                             : (const void*)slice_gemm_kernel<false>;
+    cudaError_t e = ensure_smem(fn, SMEM);
+    if (e) return e;
+    for (const S64Chunk& c : d.chunks) {
+        const dim3 grid(c.p1 - c.p0, (sl->C16 + 31) / 32);
+        if (inverse)
+            launch_slice_b<true>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
+                                 sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
+        else
+            launch_slice_b<false>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
+                                  sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
+        note_launch();
+        if ((e = cudaGetLastError())) return e;
+        S64Args g;
+        g.table = d.table;
+        g.bbuf = sl->bbuf;
+        g.probs = d.d_probs;
+        g.tiles = d.d_tiles + c.t0;
+        g.ntiles = c.t1 - c.t0;
+        g.O = O;
+        g.ea = d.ea;
+        g.eb = sl->eb;
+        g.jmin = p->d_jmin;
+        g.inverse = inverse ? 1 : 0;
+        g.C = C;
+        g.C16 = sl->C16;
+        g.status = p->d_status;
+        if (g.ntiles == 0) continue;
+        const int ctas = std::min(g.ntiles, p->num_sms);
+        if (d.mcols)
+            slice_gemm_kernel<true><<<ctas, NT, SMEM, s>>>(g);
+        else
+            slice_gemm_kernel<false><<<ctas, NT, SMEM, s>>>(g);
+        note_launch();
+        if ((e = cudaGetLastError())) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace
+
+// The tensor cores are the faster way from about 4e5 flops per transform
+// (us of the forward + inverse stages, FP64 pipe -> slices: T31 x 1 45 -> 34,
+// one launch more; T31 x 16 46 -> 43; T63 x 1 95 -> 34; T127 x 1 406 -> 58;
+// T639 x 256 238400 -> 13200).  Below, a transform is one small wave either
+// way and the single launch is kept.
+static bool slice64_wanted(const sht_plan_s* p) {
+    return 4.0 * (double)p->ncoef * p->Jh * p->F > 4e5 && p->Jh <= 4096;
+}
+
+// The slice tables of an FP64 plan; without the memory for them the plan
+// stays on the FP64 pipe.
+cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
+    if (!slice64_wanted(p)) return cudaSuccess;
+    Slice64* sl = new (std::nothrow) Slice64();
+    if (!sl) return cudaSuccess;
+    p->slice = sl;
+    const int C = 2 * p->F, nprob = 2 * (p->N + 1);
+    sl->C16 = (C + 15) / 16 * 16;
+    HostDir h[2];
+    for (int i = 0; i < 2; ++i) build_dir(p->N, p->Jh, C, i == 1, sl->dir[i], h[i]);
+    cudaError_t e = cudaMalloc(&sl->bbuf, std::max(h[0].bbytes, h[1].bbytes));
+    if (e == cudaSuccess) e = cudaMalloc(&sl->eb, (size_t)nprob * sl->C16 * sizeof(int));
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+        S64Dir& d = sl->dir[i];
+        e = cudaMalloc(&d.table, (size_t)h[i].table_bytes + 16);
+        if (e == cudaSuccess) e = cudaMalloc(&d.ea, (size_t)(h[i].ea_rows + 1) * sizeof(int));
+        if (e == cudaSuccess) e = cudaMalloc(&d.d_probs, nprob * sizeof(S64Prob));
+        if (e == cudaSuccess) e = cudaMalloc(&d.d_tiles, (h[i].tiles.size() + 1) * sizeof(int4));
+    }
+    if (e != cudaSuccess) {
+        slice64_destroy(p);
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+        S64Dir& d = sl->dir[i];
+        e = cudaMemcpyAsync(d.d_probs, h[i].probs.data(), nprob * sizeof(S64Prob),
+                            cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(d.d_tiles, h[i].tiles.data(), h[i].tiles.size() * sizeof(int4),
+                                cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) break;
+        table_exp_kernel<<<nprob, 256, 0, s>>>(p->d_pnm, p->ldp, p->N, d.d_probs, i, d.ea);
+        table_slice_kernel<<<dim3(nprob, 8), 256, 0, s>>>(p->d_pnm, p->ldp, p->N, d.d_probs, i,
+                                                         d.ea, d.table);
+        e = cudaGetLastError();
+    }
+    // (the host lists above must outlive the copies)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e;
+}
+
+void slice64_destroy(sht_plan_s* p) {
+    Slice64* sl = p->slice;
+    if (!sl) return;
+    if (sl->bbuf) cudaFree(sl->bbuf);
+    if (sl->eb) cudaFree(sl->eb);
+    for (S64Dir& d : sl->dir) {
+        void* ptrs[] = {d.table, d.ea, d.d_probs, d.d_tiles};
+        for (void* q : ptrs)
+            if (q) cudaFree(q);
+    }
+    delete sl;
+    p->slice = nullptr;
+}
+
+cudaError_t launch_legendre_slice64(const sht_plan_s* p, bool inverse, const double* in,
+                                    double* out, cudaStream_t s) {
+    return launch_dir(p, inverse, in, out, s);
+}
+
+}  // namespace sht

@@ -52,6 +52,7 @@
 #include <vector>
 
 #include "sht_internal.h"
+#include "sht_tc.h"
 
 namespace sht {
 
@@ -103,7 +104,6 @@ constexpr int NTHREADS = NCONV + 96;       // + bulk-copy warp + MMA warp + B-ro
 constexpr int WARP_PRODUCER = NCONV / 32, WARP_MMA = NCONV / 32 + 1, WARP_RAW = NCONV / 32 + 2;
 constexpr int A_TILE_BYTES = TM * TK * 2;   // one term
 constexpr uint32_t kSBO = (TK / 8) * 128;   // stride between 8-row core groups
-constexpr long long kWaitCycles = 4LL << 30;   // ~2 s at 2 GHz
 
 // Per column-tile width TN: one 16-bit B tile (TK x TN), the FP32 staging of
 // B (TK rows of TN) and the tensor memory of the two TN-column accumulators.
@@ -182,59 +182,6 @@ __device__ __forceinline__ float col_unscale(unsigned maxbits) {
     return __uint_as_float((eb + 1u) << 23);
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                 "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait: true when the phase completed, false on timeout or abort.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
-                                          volatile int* abort_flag) {
-    const long long t0 = clock64();
-    while (!mbar_try(bar, parity)) {
-        if (*abort_flag) return false;
-        if (clock64() - t0 > kWaitCycles) {
-            *abort_flag = 1;
-            return false;
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
-                                         uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
-        "[%0], [%1], %2, [%3];" ::"r"(dst),
-        "l"(src), "r"(bytes), "r"(bar)
-        : "memory");
-}
-
 // One TK x TN box of the tensor map at column x, row y (x * 4 bytes is a
 // multiple of 16: x is a multiple of TN).
 __device__ __forceinline__ void tensor_g2s_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
@@ -254,14 +201,6 @@ __device__ __forceinline__ void tensor_prefetch_l2_2d(const CUtensorMap* map, in
                  : "memory");
 }
 
-// Shared-memory matrix descriptor, no swizzle: start address, leading
-// (K-direction core stride) and stride (M/N-direction 8-row-group stride)
-// byte offsets, descriptor version 1 at bit 46.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
-}
-
 // Instruction descriptor, kind::f16: FP32 accumulator (bit 4), A and B
 // BF16 (format 1 at bits 7 and 10) or FP16 (format 0), both K-major,
 // N = TN (N/8 at bit 17), M = 128 (M/16 at bit 24).
@@ -269,16 +208,6 @@ template <bool F16, int TN>
 constexpr uint32_t idesc_f16() {
     return (1u << 4) | (F16 ? 0u : ((1u << 7) | (1u << 10))) | ((uint32_t)(TN >> 3) << 17) |
            ((uint32_t)(TM >> 4) << 24);
-}
-
-// The same MMA with the instruction descriptor in a register (N chosen per tile).
-__device__ __forceinline__ void mma_f16_rt(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                           uint32_t accum) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum));
 }
 
 template <bool F16, int TN>
@@ -324,13 +253,6 @@ __device__ __forceinline__ uint4 split_term8(float (&x)[8]) {
         }
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            bar)
-        : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {

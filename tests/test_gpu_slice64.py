@@ -1,0 +1,88 @@
+"""FP64 contractions on the tensor cores (sliced operands) against the CPU
+oracle and the FP64-pipe kernels, at the edges of their tiles: one more and
+one fewer row, node or column than a multiple of 16, 64 or 128, both
+orientations of the product, column ranges of 1e-300 .. 1e300, and
+non-finite columns.
+
+Tolerance: a slice carries its operand to 2^-55 of the row or column
+maximum, so a sum of K products is within 2 K 2^-55 of (row maximum x column
+maximum) besides the final rounding; with K <= 322 and |P~| <= 26 that is
+below 5e-13 of the largest column, and the FP64 tolerance of the other tests
+(1e-12) covers it."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_1711_11296_gb300 import workloads as W
+from sht_testutil import assert_fp64_close, built_lib, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+# (N, J, I, F): columns are 2 F, parity rows at most N / 2 + 1, nodes J / 2
+CASES = [
+    (63, 129, 256, 1),     # 2 columns, 64 nodes + the Equator
+    (63, 127, 256, 8),     # 16 columns, 63 nodes
+    (62, 131, 128, 9),     # 18 columns, 65 nodes
+    (127, 257, 512, 31),   # 62 columns, 128 nodes, rows up to 64
+    (129, 263, 288, 33),   # 66 columns
+    (31, 65, 128, 64),     # 128 columns, 16 rows
+    (33, 69, 72, 65),      # 130 columns, 17 rows
+    (40, 71, 96, 129),     # 258 columns, inexact grid (J < 2 N + 1)
+]
+
+
+@pytest.fixture(scope="module")
+def sht():
+    built_lib()
+    from paper_1711_11296_gb300 import sht as S
+    return S
+
+
+@pytest.mark.parametrize("N,J,I,F", CASES)
+def test_matches_oracle(sht, N, J, I, F):
+    p = sht.Plan(N, J, I, F, "fp64")
+    x = W.random_grid(F, J, I, seed=2100 + N)
+    a = W.random_spectrum(N, F, "flat", seed=2200 + N)
+    assert_fp64_close(p.forward(to_cuda(x, torch.float64)).cpu().numpy(), O.analysis(x, N))
+    assert_fp64_close(p.inverse(to_cuda(a, torch.complex128)).cpu().numpy(),
+                      O.synthesis(a, N, J, I))
+    p.status()
+
+
+def test_columns_are_scaled_alone(sht):
+    # columns at the ends of the FP64 range, and an all-zero one: each
+    # field's result is that of the field alone, scaled (powers of two)
+    N, J, I, F = 63, 129, 256, 6
+    p = sht.Plan(N, J, I, F, "fp64")
+    a = W.random_spectrum(N, 1, "flat", seed=2300)
+    scale = np.array([1.0, 2.0 ** -990, 2.0 ** 990, 0.0, 2.0 ** 40, 2.0 ** -40])
+    t = p.inverse(to_cuda(a * scale, torch.complex128)).cpu().numpy()
+    for f, s in enumerate(scale):
+        ref = t[0] * s
+        assert np.abs(t[f] - ref).max() <= 1e-14 * np.abs(ref).max()
+    s0 = p.forward(to_cuda(t, torch.float64)).cpu().numpy()
+    for f, s in enumerate(scale):
+        ref = s0[:, 0] * s
+        assert np.abs(s0[:, f] - ref).max() <= 1e-14 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_non_finite_fields_stay_apart(sht, bad):
+    N, J, I, F = 63, 129, 256, 5
+    p = sht.Plan(N, J, I, F, "fp64")
+    x = W.random_grid(F, J, I, seed=2400)
+    y = x.copy()
+    y[3, 17, 40] = bad
+    good = p.forward(to_cuda(x, torch.float64)).cpu().numpy()
+    got = p.forward(to_cuda(y, torch.float64)).cpu().numpy()
+    keep = [0, 1, 2, 4]
+    np.testing.assert_array_equal(got[:, keep], good[:, keep])
+    assert not np.isfinite(got[:, 3]).any()
+    a = W.random_spectrum(N, F, "flat", seed=2401)
+    b = a.copy()
+    b[100, 2] = bad
+    good = p.inverse(to_cuda(a, torch.complex128)).cpu().numpy()
+    got = p.inverse(to_cuda(b, torch.complex128)).cpu().numpy()
+    np.testing.assert_array_equal(got[[0, 1, 3, 4]], good[[0, 1, 3, 4]])
+    assert not np.isfinite(got[2]).any()
