@@ -41,12 +41,13 @@
 #include <mutex>
 #include <type_traits>
 
+#include "sht_fft_common.h"
 #include "sht_internal.h"
 
 namespace sht {
 namespace {
 
-constexpr int NT = 256;   // threads per FFT CTA (two CTAs per SM for FP32)
+constexpr int NT = kFftThreads;
 
 // Paired FP32 arithmetic (add/sub/mul.f32x2): one instruction on both
 // components of a complex value.
@@ -103,45 +104,10 @@ template <typename T> struct C2 {
     static __device__ __forceinline__ V mul_pi(V a) { return make(-a.y, a.x); }
 };
 
-// The plan's factorisation as a compile-time constant.
-template <int L, bool FP64> struct FacOf {
-    static constexpr FftShape v = fft_factor(L, FP64);
-};
-
 // W_N^e = exp(-2 pi i e/N) for the composite register DFT sizes, written
 // once per device by fft_constants_init (offsets per N below).
 constexpr int kTw10 = 0, kTw16 = 10, kTw20 = 26, kTw32 = 46, kTw40 = 78, kTwTotal = 118;
 __constant__ float2 c_twf[kTwTotal];
-__constant__ double2 c_twd[kTwTotal];
-
-template <typename T>
-__device__ __forceinline__ typename Vec2<T>::type twc(int idx) {
-    if constexpr (sizeof(T) == 4)
-        return c_twf[idx];
-    else
-        return c_twd[idx];
-}
-
-// Asynchronous global -> shared copy of one element (cp.async, no register
-// staging, so all of a thread's copies are in flight at once).
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* dst, const void* src) {
-    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-    if constexpr (BYTES == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES)
-                     : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
-
-template <typename T>
-__device__ __forceinline__ int ph(int pos) {
-    return pos + (pos >> PadShift<T>::value);
-}
 
 // ---- radix-R DFTs (forward sign) ---------------------------------------
 template <typename T, int R> struct Dft;
@@ -262,7 +228,7 @@ struct DftComposite {
 #pragma unroll
             for (int k1 = 0; k1 < A; ++k1)
                 x[b + B * k1] =
-                    (b * k1 == 0) ? t[k1] : K::mul(t[k1], twc<T>(TWOFF + (b * k1) % N));
+                    (b * k1 == 0) ? t[k1] : K::mul(t[k1], c_twf[TWOFF + (b * k1) % N]);
         }
 #pragma unroll
         for (int k1 = 0; k1 < A; ++k1) {
@@ -433,79 +399,6 @@ __host__ __device__ constexpr bool inverse_stores_from_last_pass() {
     }
 }
 
-// Digit-reversed position of frequency k.
-template <typename T, int L>
-__device__ __forceinline__ int rev_fixed(int k) {
-    constexpr FftShape F = FacOf<L, sizeof(T) == 8>::v;
-    int pos = 0;
-#pragma unroll
-    for (int q = 0; q < F.npass; ++q) {
-        pos += (k % F.radix[q]) * F.span[q];
-        k /= F.radix[q];
-    }
-    return pos;
-}
-
-template <typename T>
-struct FwdArgs {
-    using V = typename Vec2<T>::type;
-    const T* grid;
-    RowSource src;
-    V* work;
-    const V* twp;      // per-pass twiddle tables
-    const V* twpost;
-    const int* rev;
-    const double* rowscale;
-    double mscale0, mscale1;
-    unsigned* colmax;   // FP16 split plans: max |output| per real column (float bits)
-    const long long* rowoff;   // reduced grid: first point of each row (null: regular)
-    const int* jh_list;        // latitude pair of each CTA row (null: blockIdx.y)
-    const V* shiftph;          // rows shifted by half a spacing: e^{-i pi m / I_j} (else null)
-    const V* chirp;            // Bluestein rows: e^{-i pi n^2 / L}
-    const V* dft;              // Bluestein rows: DFT of the conjugate chirp / L2
-    int F, J, Jh, L, LP, N, G;
-    FftShape shape;
-};
-
-template <typename T>
-struct InvArgs {
-    using V = typename Vec2<T>::type;
-    const V* work;
-    T* grid;
-    const V* twp;
-    const V* twpost;
-    const int* rev;
-    const double* rowscale;
-    double mfactor1;
-    const long long* rowoff;   // reduced grid: first point of each row (null: regular)
-    long long fstride;         // reduced grid: points per field
-    const int* jh_list;        // latitude pair of each CTA row (null: blockIdx.y)
-    int accumulate;            // 1: grid += rows (prolongation of a correction);
-                               // 2: products (Sec. 4.2): with w the synthesised
-                               // value, grid holds u and becomes u v, grid2
-                               // holds v and becomes u v w
-    T* grid2;                  // second grid of the products (else null)
-    const V* shiftph;          // rows shifted by half a spacing: e^{-i pi m / I_j} (else null)
-    const V* chirp;            // Bluestein rows: e^{-i pi n^2 / L}
-    const V* dft;              // Bluestein rows: DFT of the conjugate chirp / L2
-    int F, J, Jh, I, L, LP, N, G;
-    FftShape shape;
-};
-
-// Copy the per-pass twiddle tables into shared memory asynchronously, so
-// that they are in flight together with the CTA's data copies (one wait).
-template <typename V>
-__device__ __forceinline__ void load_twiddles_async(V* dst, const V* src, int n) {
-    for (int e = threadIdx.x; e < n; e += NT) cp_async<sizeof(V)>(dst + e, src + e);
-}
-
-// The same by plain loads and stores (measured faster ahead of the inverse
-// kernel's gathered copies).
-template <typename V>
-__device__ __forceinline__ void load_twiddles(V* dst, const V* src, int n) {
-    for (int e = threadIdx.x; e < n; e += NT) dst[e] = src[e];
-}
-
 // LT > 0: the compile-time shape of that half-length; LT = 0: any shape at
 // run time; LT = -1: a run-time shape without the two-pass radices.
 template <typename T, int LT>
@@ -516,16 +409,6 @@ __device__ __forceinline__ void run_passes(typename Vec2<T>::type* rows, int nro
         passes_fixed<T, LT, 0>(rows, nrows, LP, twp);
     else
         passes_runtime<T, LT == 0>(rows, nrows, LP, sh, twp);
-}
-
-template <typename T, int LT>
-__device__ __forceinline__ int rev_of(int k, const int* rev) {
-    if constexpr (LT > 0)
-        return rev_fixed<T, LT>(k);
-    else if constexpr (LT == -2)
-        return k;   // Bluestein rows end in natural order
-    else
-        return rev[k];
 }
 
 // Bluestein's chirp-z DFT of each of nrows padded rows of half-length L (any
@@ -564,32 +447,6 @@ __device__ void bluestein_rows(typename Vec2<T>::type* rows, int nrows, int LP, 
         __syncthreads();
     }
 }
-
-// Padded pitch of a row of n complex values (fft_row_pitch on the device).
-template <typename T>
-__device__ __forceinline__ int row_pitch(int n) {
-    return n + (n >> PadShift<T>::value) + 1;
-}
-
-// Iterates idx = tid, tid + NT, ... as (major, minor) = (idx / d, idx % d)
-// without dividing inside the loop.
-struct Walk2 {
-    int major, minor, step_major, step_minor, d;
-    __device__ __forceinline__ Walk2(int start, int d_) : d(d_) {
-        major = start / d;
-        minor = start - major * d;
-        step_major = NT / d;
-        step_minor = NT - step_major * d;
-    }
-    __device__ __forceinline__ void next() {
-        major += step_major;
-        minor += step_minor;
-        if (minor >= d) {
-            minor -= d;
-            ++major;
-        }
-    }
-};
 
 extern __shared__ __align__(16) unsigned char fft_smem_raw[];
 
@@ -1152,21 +1009,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     inv_body<T, LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
 }
 
-// ---- grouped launches: several plans' rows in one grid ----------------
-template <typename T> struct FwdGroup {
-    int n;
-    int cta_start[kMaxGroup + 1];   // first CTA of each plan
-    int nfg[kMaxGroup];             // field groups per latitude of each plan
-    FwdArgs<T> a[kMaxGroup];
-};
-
-template <typename T> struct InvGroup {
-    int n;
-    int cta_start[kMaxGroup + 1];
-    int nfg[kMaxGroup];
-    InvArgs<T> a[kMaxGroup];
-};
-
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_forward_group_kernel(const __grid_constant__ FwdGroup<T> G) {
@@ -1209,48 +1051,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
         case 1024: inv_body<T, 1024>(A, fg, jh); break;
         case 1280: inv_body<T, 1280>(A, fg, jh); break;
         default: inv_body<T, -1>(A, fg, jh);
-    }
-}
-
-// ---- reduced grids: a half-length per latitude pair -------------------
-// Each CTA takes its latitude pair's FFT shape and the offsets of that
-// shape's tables; rows, shared memory and the row pitch are sized for the
-// longest row of the grid.
-template <typename T> struct RaggedFwd {
-    FwdArgs<T> a;
-    const RShape* shapes;
-    const int* shape_of;
-    const int* shift_of;                       // per latitude pair (null: none shifted)
-    const typename Vec2<T>::type* shiftbase;   // all shapes' shift phases
-    const typename Vec2<T>::type* chirpbase;   // all Bluestein shapes' chirps
-    const typename Vec2<T>::type* dftbase;     // all Bluestein shapes' chirp spectra
-};
-
-template <typename T> struct RaggedInv {
-    InvArgs<T> a;
-    const RShape* shapes;
-    const int* shape_of;
-    const int* shift_of;
-    const typename Vec2<T>::type* shiftbase;
-    const typename Vec2<T>::type* chirpbase;
-    const typename Vec2<T>::type* dftbase;
-};
-
-// Per-CTA arguments of a reduced-grid row class: the latitude pair's shape,
-// its tables, and its shift.
-template <typename Args, typename R>
-__device__ __forceinline__ void apply_shape(Args& A, const R& Rg, int jh) {
-    const RShape& rs = Rg.shapes[Rg.shape_of[jh]];
-    A.shape = rs.sh;
-    A.L = rs.L;
-    A.twp += rs.tw_off;
-    A.twpost += rs.post_off;
-    A.rev += rs.rev_off;
-    A.shiftph = (Rg.shift_of && Rg.shift_of[jh] && rs.shift_off >= 0)
-                    ? Rg.shiftbase + rs.shift_off : nullptr;
-    if (rs.bluestein) {
-        A.chirp = Rg.chirpbase + rs.chirp_off;
-        A.dft = Rg.dftbase + rs.dft_off;
     }
 }
 
@@ -1373,9 +1173,13 @@ cudaError_t fwd_impl(const sht_plan_s* p, const void* grid, const RowSource& src
     const dim3 g((p->F + p->G - 1) / p->G, p->Jh);
     const bool strided = src.elem_stride != 1;
     if (!fft_has_fixed_kernel(p->fft.L) && !small_radices(p->fft)) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 8) {
+        return fx_forward(A, strided, g, p->fft_smem, s);
+    } else {
 #define SHT_FWD(LV) fwd_launch<T, LV>(A, strided, g, p->fft_smem, s)
-    SHT_FFT_DISPATCH(p->fft.L, SHT_FWD)
+        SHT_FFT_DISPATCH(p->fft.L, SHT_FWD)
 #undef SHT_FWD
+    }
 }
 
 template <typename T>
@@ -1409,9 +1213,13 @@ cudaError_t inv_impl(const sht_plan_s* p, const void* work, const InvScale& sc,
     const InvArgs<T> A = make_inv_args<T>(p, work, sc, grid);
     const dim3 g((p->F + p->G - 1) / p->G, p->Jh);
     if (!fft_has_fixed_kernel(p->fft.L) && !small_radices(p->fft)) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 8) {
+        return fx_inverse(A, g, p->fft_smem, s);
+    } else {
 #define SHT_INV(LV) inv_launch<T, LV>(A, g, p->fft_smem, s)
-    SHT_FFT_DISPATCH(p->fft.L, SHT_INV)
+        SHT_FFT_DISPATCH(p->fft.L, SHT_INV)
 #undef SHT_INV
+    }
 }
 
 // Dispatch of a compile-time length (the lengths of fft_has_fixed_kernel).
@@ -1444,16 +1252,24 @@ void set_class(Args& A, const RaggedGrid* rg, const RShape& r, int off, size_t v
 
 template <typename T>
 cudaError_t fwd_ragged_class(const FwdArgs<T>& A, dim3 g, size_t smem, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+        return fx_forward(A, false, g, smem, s);
+    } else {
 #define SHT_FWDC(LV) fwd_launch<T, LV>(A, false, g, smem, s)
-    SHT_FFT_FIXED(A.L, SHT_FWDC)
+        SHT_FFT_FIXED(A.L, SHT_FWDC)
 #undef SHT_FWDC
+    }
 }
 
 template <typename T>
 cudaError_t inv_ragged_class(const InvArgs<T>& A, dim3 g, size_t smem, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+        return fx_inverse(A, g, smem, s);
+    } else {
 #define SHT_INVC(LV) inv_launch<T, LV>(A, g, smem, s)
-    SHT_FFT_FIXED(A.L, SHT_INVC)
+        SHT_FFT_FIXED(A.L, SHT_INVC)
 #undef SHT_INVC
+    }
 }
 
 // Reduced grid: one launch of the compile-time kernel per length class that
@@ -1498,11 +1314,17 @@ cudaError_t fwd_ragged_impl(const sht_plan_s* p, const void* grid, const FwdScal
     cudaError_t e;
     if (rg->generic_count > 0) {
         R.a.jh_list = rg->d_jh + rg->generic_off;
-        e = ensure_smem((const void*)fft_forward_ragged_kernel<T>, p->fft_smem);
-        if (e) return e;
-        fft_forward_ragged_kernel<T><<<dim3(nfg, rg->generic_count), NT, p->fft_smem, s>>>(R);
-        note_launch();
-        if ((e = cudaGetLastError())) return e;
+        const dim3 g(nfg, rg->generic_count);
+        if constexpr (sizeof(T) == 8) {
+            e = fx_forward_ragged(R, g, p->fft_smem, s);
+            if (e) return e;
+        } else {
+            e = ensure_smem((const void*)fft_forward_ragged_kernel<T>, p->fft_smem);
+            if (e) return e;
+            fft_forward_ragged_kernel<T><<<g, NT, p->fft_smem, s>>>(R);
+            note_launch();
+            if ((e = cudaGetLastError())) return e;
+        }
     }
     if (rg->blue_count > 0) {
         R.a.jh_list = rg->d_jh + rg->blue_off;
@@ -1548,11 +1370,17 @@ cudaError_t inv_ragged_impl(const sht_plan_s* p, const void* work, const InvScal
     cudaError_t e;
     if (rg->generic_count > 0) {
         R.a.jh_list = rg->d_jh + rg->generic_off;
-        e = ensure_smem((const void*)fft_inverse_ragged_kernel<T>, p->fft_smem);
-        if (e) return e;
-        fft_inverse_ragged_kernel<T><<<dim3(nfg, rg->generic_count), NT, p->fft_smem, s>>>(R);
-        note_launch();
-        if ((e = cudaGetLastError())) return e;
+        const dim3 g(nfg, rg->generic_count);
+        if constexpr (sizeof(T) == 8) {
+            e = fx_inverse_ragged(R, g, p->fft_smem, s);
+            if (e) return e;
+        } else {
+            e = ensure_smem((const void*)fft_inverse_ragged_kernel<T>, p->fft_smem);
+            if (e) return e;
+            fft_inverse_ragged_kernel<T><<<g, NT, p->fft_smem, s>>>(R);
+            note_launch();
+            if ((e = cudaGetLastError())) return e;
+        }
     }
     if (rg->blue_count > 0) {
         R.a.jh_list = rg->d_jh + rg->blue_off;
@@ -1592,11 +1420,15 @@ cudaError_t fwd_group_impl(sht_plan_s* const* plans, int n, const void* const* g
         G.cta_start[q + 1] = G.cta_start[q] + G.nfg[q] * p->Jh;
         if (p->fft_smem > smem) smem = p->fft_smem;
     }
-    cudaError_t e = ensure_smem((const void*)fft_forward_group_kernel<T>, smem);
-    if (e) return e;
-    fft_forward_group_kernel<T><<<G.cta_start[n], NT, smem, s>>>(G);
-    note_launch();
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        return fx_forward_group(G, G.cta_start[n], smem, s);
+    } else {
+        cudaError_t e = ensure_smem((const void*)fft_forward_group_kernel<T>, smem);
+        if (e) return e;
+        fft_forward_group_kernel<T><<<G.cta_start[n], NT, smem, s>>>(G);
+        note_launch();
+        return cudaGetLastError();
+    }
 }
 
 template <typename T>
@@ -1614,11 +1446,15 @@ cudaError_t inv_group_impl(sht_plan_s* const* plans, int n, void* const* grids,
         G.cta_start[q + 1] = G.cta_start[q] + G.nfg[q] * p->Jh;
         if (p->fft_smem > smem) smem = p->fft_smem;
     }
-    cudaError_t e = ensure_smem((const void*)fft_inverse_group_kernel<T>, smem);
-    if (e) return e;
-    fft_inverse_group_kernel<T><<<G.cta_start[n], NT, smem, s>>>(G);
-    note_launch();
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        return fx_inverse_group(G, G.cta_start[n], smem, s);
+    } else {
+        cudaError_t e = ensure_smem((const void*)fft_inverse_group_kernel<T>, smem);
+        if (e) return e;
+        fft_inverse_group_kernel<T><<<G.cta_start[n], NT, smem, s>>>(G);
+        note_launch();
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace
@@ -1632,7 +1468,6 @@ cudaError_t fft_constants_init() {
     std::lock_guard<std::mutex> lk(mu);
     if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
     float2 hf[kTwTotal];
-    double2 hd[kTwTotal];
     const int sizes[5] = {10, 16, 20, 32, 40};
     const int offs[5] = {kTw10, kTw16, kTw20, kTw32, kTw40};
     const long double pi = 3.14159265358979323846264338327950288L;
@@ -1640,11 +1475,9 @@ cudaError_t fft_constants_init() {
         for (int k = 0; k < sizes[q]; ++k) {
             const long double ang = 2.0L * pi * (long double)k / (long double)sizes[q];
             const double c = (double)cosl(ang), sn = -(double)sinl(ang);
-            hd[offs[q] + k] = make_double2(c, sn);
             hf[offs[q] + k] = make_float2((float)c, (float)sn);
         }
     e = cudaMemcpyToSymbol(c_twf, hf, sizeof(hf));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_twd, hd, sizeof(hd));
     if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
     return e;
 }
@@ -1674,7 +1507,8 @@ size_t fft_smem_bytes(int I, int G, bool fp64) {
     const size_t v = fp64 ? sizeof(double2) : sizeof(float2);
     // padded rows + per-pass twiddle tables (fewer than L entries) + the
     // column maxima of the forward kernel's output (2 words per field)
-    return (2 * (size_t)G * fft_row_pitch((int)L, fp64) + L) * v + 8 * (size_t)G;
+    // or, FP64, the fields' scales (32 bytes each)
+    return (2 * (size_t)G * fft_row_pitch((int)L, fp64) + L) * v + (fp64 ? 32 : 8) * (size_t)G;
 }
 
 cudaError_t launch_fft_forward(const sht_plan_s* p, const void* grid,

@@ -225,8 +225,11 @@ cudaError_t build_node_tables(sht_plan_s* p, cudaStream_t s);
 cudaError_t build_pnm_table(sht_plan_s* p, cudaStream_t s);
 cudaError_t build_twiddles(sht_plan_s* p, cudaStream_t s);
 cudaError_t launch_twpass(const sht_plan_s* p, cudaStream_t s);
-cudaError_t build_fft_tables(const FftShape& sh, bool fp64, void* twpass, void* twpost,
-                             int* rev, void* tmp, cudaStream_t s);
+cudaError_t build_fft_tables(const FftShape& sh, bool fp64, bool fixed, void* twpass,
+                             void* twpost, int* rev, void* tmp, cudaStream_t s);
+// FP64 twiddle tables to the fixed-point form that the FP64 FFT kernels
+// read (in place, the same 16 bytes an entry).
+cudaError_t launch_fixed_twiddles(void* table, int n, cudaStream_t s);
 // Tables of a Bluestein shape (rows of half-length L, passes sh2 of length
 // L2 >= 2L - 1): the passes' twiddles and digit reversal, the row's
 // real-spectrum twiddles e^{-2 pi i q / 2L}, the chirp e^{-pi i n^2 / L}

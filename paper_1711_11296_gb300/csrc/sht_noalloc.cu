@@ -244,6 +244,8 @@ extern "C" int sht_forward_noalloc(int N, int J, int I, int nfields,
     if (e == cudaSuccess) e = launch_pnm_recurrence(&t, s);
     if (e == cudaSuccess) e = launch_twiddles_fp64(&t, s);
     if (e == cudaSuccess) e = launch_twpass(&t, s);
+    if (e == cudaSuccess) e = launch_fixed_twiddles(t.d_twpass, shape.twtotal, s);
+    if (e == cudaSuccess) e = launch_fixed_twiddles(t.d_twpost, shape.L, s);
     if (e == cudaSuccess) {
         rev_kernel<<<(shape.L + th - 1) / th, th, 0, s>>>(shape, t.d_rev);
         e = cudaGetLastError();

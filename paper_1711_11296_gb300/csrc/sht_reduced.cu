@@ -235,7 +235,7 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
                                        static_cast<char*>(rg->d_chirp) + r.chirp_off * vb,
                                        static_cast<char*>(rg->d_dft) + r.dft_off * vb, tmp, s);
         else
-            e = build_fft_tables(r.sh, fp64, tw, post, rg->d_rev + r.rev_off, tmp, s);
+            e = build_fft_tables(r.sh, fp64, fp64, tw, post, rg->d_rev + r.rev_off, tmp, s);
         if (e == cudaSuccess && r.shift_off >= 0)
             e = build_shift_table(r.L, 2 * r.L, fp64,
                                   static_cast<char*>(rg->d_shiftph) + r.shift_off * vb, s);

@@ -211,6 +211,10 @@ cudaError_t build_twiddles(sht_plan_s* p, cudaStream_t s) {
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     err = launch_twpass(p, s);
+    if (p->prec == SHT_FP64) {
+        if (err == cudaSuccess) err = launch_fixed_twiddles(p->d_twpass, p->fft.twtotal, s);
+        if (err == cudaSuccess) err = launch_fixed_twiddles(p->d_twpost, L, s);
+    }
     if (err != cudaSuccess) return err;
     // digit-reversed output positions of the in-place mixed-radix FFT
     std::vector<int> rev(L);
@@ -232,9 +236,10 @@ cudaError_t build_twiddles(sht_plan_s* p, cudaStream_t s) {
 // device buffers: the per-pass twiddle tables (sh.twtotal entries), the
 // real-spectrum twiddles e^{-2 pi i q / I} (L entries) and the digit-
 // reversed positions (L ints).  tmp holds L complex entries (the length-L
-// table the per-pass tables are gathered from).  Synchronises s.
-cudaError_t build_fft_tables(const FftShape& sh, bool fp64, void* twpass, void* twpost,
-                             int* rev, void* tmp, cudaStream_t s) {
+// table the per-pass tables are gathered from).  fixed (FP64 only): the
+// fixed-point form.  Synchronises s.
+cudaError_t build_fft_tables(const FftShape& sh, bool fp64, bool fixed, void* twpass,
+                             void* twpost, int* rev, void* tmp, cudaStream_t s) {
     const int L = sh.L;
     const int threads = 128;
     const int blocks = (L + threads - 1) / threads;
@@ -253,6 +258,8 @@ cudaError_t build_fft_tables(const FftShape& sh, bool fp64, void* twpass, void* 
         twiddle_kernel<float2><<<blocks, threads, 0, s>>>((float2*)twpost, L, 2 * L);
     }
     cudaError_t err = cudaGetLastError();
+    if (err == cudaSuccess && fixed) err = launch_fixed_twiddles(twpass, sh.twtotal, s);
+    if (err == cudaSuccess && fixed) err = launch_fixed_twiddles(twpost, L, s);
     if (err != cudaSuccess) return err;
     std::vector<int> h(L);
     for (int k = 0; k < L; ++k) {
@@ -342,7 +349,7 @@ cudaError_t build_bluestein_tables(int L, const FftShape& sh2, bool fp64, void* 
     void* post2 = t + L2 * vb;
     double2* c64 = reinterpret_cast<double2*>(t + 2 * L2 * sizeof(double2));
     double* costab = reinterpret_cast<double*>(c64 + L2);
-    cudaError_t e = build_fft_tables(sh2, fp64, twpass, post2, rev, base, s);
+    cudaError_t e = build_fft_tables(sh2, fp64, false, twpass, post2, rev, base, s);
     if (e != cudaSuccess) return e;
     const int bL = (L + threads - 1) / threads, bL2 = (L2 + threads - 1) / threads;
     cos_table_kernel<<<bL2, threads, 0, s>>>(costab, L2);
