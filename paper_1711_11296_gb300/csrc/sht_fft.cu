@@ -1504,11 +1504,12 @@ size_t bluestein_smem_bytes(int Lmax, int L2, int G, bool fp64) {
 
 size_t fft_smem_bytes(int I, int G, bool fp64) {
     const size_t L = (size_t)I / 2;
-    const size_t v = fp64 ? sizeof(double2) : sizeof(float2);
-    // padded rows + per-pass twiddle tables (fewer than L entries) + the
+    const size_t rows = 2 * (size_t)G * fft_row_pitch((int)L, fp64);
+    // FP64: padded rows + the fields' scales
+    if (fp64) return rows * sizeof(double2) + kFxFieldBytes * (size_t)G;
+    // FP32: padded rows + per-pass twiddle tables (fewer than L entries) + the
     // column maxima of the forward kernel's output (2 words per field)
-    // or, FP64, the fields' scales (32 bytes each)
-    return (2 * (size_t)G * fft_row_pitch((int)L, fp64) + L) * v + (fp64 ? 32 : 8) * (size_t)G;
+    return (rows + L) * sizeof(float2) + 8 * (size_t)G;
 }
 
 cudaError_t launch_fft_forward(const sht_plan_s* p, const void* grid,

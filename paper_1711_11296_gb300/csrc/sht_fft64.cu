@@ -32,7 +32,13 @@
 // A CTA owns a latitude pair for G fields, as in sht_fft.cu: rows of
 // 16-byte complex integers in the padded layout, radices 8 first, then 4, 2,
 // 3, 5, each butterfly in registers; the first pass converts the FP64
-// values as it reads them.
+// values as it reads them.  The kernel is bound by its phases' latency and
+// by issue (T639: 14 500 instructions a row, half of the cycles issue one),
+// so four CTAs share an SM: 64 registers, and the twiddle tables (20 KB at
+// L = 1280) are read through L1 rather than copied to shared memory.
+// Measured for 16 fields at T639, forward / inverse: 536 / 454 us with three
+// CTAs and copied tables, 509 / 413 with four; 475 / 415 with the integer
+// conversion.
 #include "sht_fft_common.h"
 #include "sht_internal.h"
 
@@ -52,18 +58,20 @@ __device__ __forceinline__ int lo32(ll x) { return (int)x; }
 __device__ __forceinline__ int hi32(ll x) {
     return (int)(x >> 32) + (int)((unsigned)x >> 31);
 }
-// round(m / 2^32) of m + 2^31
-__device__ __forceinline__ ll top(ll m) { return (ll)(int)(m >> 32); }
-constexpr ll kHalf = 0x80000000ll;
 
 // z w / 2 for a twiddle w = {re hi, re lo, im hi, im lo} in 2^-63 units
-// (|z| < 2^61.5).  The products of the two low halves, at most 1/2 in the
-// last place together, are left out.
+// (|z| < 2^61.5).  Of the products with one low half only the upper words
+// are formed (each rounded down: the four add a bias of -2 to the imaginary
+// part, which is put back; in the real part it cancels), those of two low
+// halves are left out: 0.6 in the last place rms.  64-bit sums of all cross
+// products were more exact (0.3) but took 44 instructions instead of 30, and
+// the input's rounding at 2^-SH is larger than either.
 __device__ __forceinline__ V cmul63(V z, int4 w) {
     const int xl = lo32(z.x), xh = hi32(z.x), yl = lo32(z.y), yh = hi32(z.y);
-    const ll mr = kHalf + wide(xh, w.y) + wide(xl, w.x) - (wide(yh, w.w) + wide(yl, w.z));
-    const ll mi = kHalf + wide(xh, w.w) + wide(xl, w.z) + wide(yh, w.y) + wide(yl, w.x);
-    return mk(top(mr) + wide(xh, w.x) - wide(yh, w.z), top(mi) + wide(xh, w.z) + wide(yh, w.x));
+    const int tr = __mulhi(xh, w.y) + __mulhi(xl, w.x) - (__mulhi(yh, w.w) + __mulhi(yl, w.z));
+    const int ti =
+        __mulhi(xh, w.w) + __mulhi(xl, w.z) + __mulhi(yh, w.y) + __mulhi(yl, w.x) + 2;
+    return mk(wide(xh, w.x) - wide(yh, w.z) + (ll)tr, wide(xh, w.z) + wide(yh, w.x) + (ll)ti);
 }
 
 // x c / 2^64
@@ -71,7 +79,7 @@ template <ll CQ>
 __device__ __forceinline__ ll mulc(ll x) {
     constexpr int cl = (int)CQ, ch = (int)((CQ - (ll)cl) >> 32);
     const int xl = lo32(x), xh = hi32(x);
-    return top(kHalf + wide(xh, cl) + wide(xl, ch)) + wide(xh, ch);
+    return wide(xh, ch) + (ll)(__mulhi(xh, cl) + __mulhi(xl, ch) + 1);
 }
 
 // constants c - 1 in 2^-64 units (c x = x + (c - 1) x)
@@ -156,46 +164,64 @@ template <> struct Dft<8> {
 
 // ---- FP64 <-> fixed point --------------------------------------------------
 
-// Per field of the CTA: exponent field of the largest component (high words
-// while it is gathered), L1 norms of its two rows in units of 2^(e - 13),
-// the conversion shift and the factors of the way back.
+// Per field of the CTA: largest |component| (high word of its FP64 bits)
+// and the warps' shares of the L1 norms of its two rows (added in a fixed
+// order, so that the scale does not depend on timing) while they are
+// gathered, then the exponent shift of the conversion and the factors of
+// the way back.
 struct Field {
-    int emax;
-    unsigned l1[2];
-    int base;        // 61 - SH + emax
+    unsigned hmax;
+    int shift;       // SH - e: integer = round(v 2^shift)
     double sc, sc2;  // integer -> FP64: times sc (times sc2 at the range's end)
+    float l1[2][NT / 32];
+    __device__ __forceinline__ float norm(int row) const {
+        float x = 0.f;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) x += l1[row][w];
+        return x;
+    }
 };
+static_assert(sizeof(Field) <= kFxFieldBytes, "the launches reserve this much per field");
 
 __device__ __forceinline__ unsigned hi_abs(double v) {
     return (unsigned)(__double_as_longlong(v) >> 32) & 0x7fffffffu;
 }
 
-// |v| rounded up, in units of 2^(e - 13) (e: |v| < 2^e, exponent field E)
-__device__ __forceinline__ unsigned l1_units(double v, int E) {
-    const unsigned h = hi_abs(v);
-    const int d = E - max((int)(h >> 20), 1) + 8;
-    return (((h & 0xfffffu) | 0x100000u) >> min(d, 31)) + 1u;
+// |v| truncated to 20 bits of mantissa as FP32, from its high word; below
+// 2^-126 it reads as 0, above 2^128 wrongly (finish_field tells from the
+// maximum).  Integer operations: a conversion would take the FP64 pipe.
+__device__ __forceinline__ float abs_f32(unsigned h) {
+    return __int_as_float(max((int)h - (896 << 20), 0) << 3);
 }
 
-// v 2^(SH - e) rounded (base = 61 - SH + E)
-__device__ __forceinline__ ll to_fx(double v, int base) {
+// round(v 2^shift), |result| <= 2^61.  Integer operations: as a conversion on
+// the FP64 pipe the first pass of the forward took 7 % longer.
+__device__ __forceinline__ ll to_fx(double v, int shift) {
     const ll bits = __double_as_longlong(v);
     const int ex = (int)(bits >> 52) & 0x7ff;
     ll man = bits & 0xfffffffffffffll;
     if (ex) man |= 0x10000000000000ll;
-    const int d = min(base - max(ex, 1), 63);
+    const int d = min(1083 - shift - max(ex, 1), 63);
     const ll t = (ll)(((unsigned long long)(man << 9) >> d) + 1) >> 1;
     return bits < 0 ? -t : t;
 }
 
-// SH and the scales of one field from its gathered maximum and L1 norm.
-// b: largest bound of the modulus over the passes, in units of 2^SH; k: the
-// transform's value is integer * 2^(e - SH + k), times f.
-__device__ __forceinline__ void finish_field(Field& fd, float b, int k, double f) {
-    const int E = max(fd.emax, 1);
+// SH and the scales of one field from its gathered maximum and L1 norm l1 (in
+// units of 2^e: |v| < 2^e).  b(l1): largest bound of the modulus over the
+// passes, in units of 2^SH; k: the transform's value is
+// integer * 2^(e - SH + k), times f.
+template <class Bound>
+__device__ __forceinline__ void finish_field(Field& fd, float l1, Bound bound, double f) {
+    const int E = max((int)(fd.hmax >> 20), 1);   // biased exponent field
+    const int e = E - 1022;
+    // without a usable FP32 sum the maximum alone bounds the growth
+    l1 = (E >= 940 && E <= 1140) ? l1 * 1.0001f * __int_as_float((127 - e) << 23)
+                                 : __int_as_float(0x7f800000);
+    int k;
+    const float b = bound(l1, k);
     const int SH = min(61, (int)floorf(61.4f - log2f(b)));
-    fd.base = 61 - SH + E;
-    const int p2 = E - 1022 - SH + k;
+    fd.shift = SH - e;
+    const int p2 = e - SH + k;
     const bool tiny = p2 < -900;   // 2^p2 would be subnormal
     fd.sc = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
                        : ldexp(f, tiny ? p2 + 200 : p2);
@@ -207,12 +233,19 @@ __device__ __forceinline__ double from_fx(ll x, double sc, double sc2) {
     return sc2 == 1.0 ? d : d * sc2;
 }
 
+// The same for a scale that is a power of two (|sc| in range, or NaN: the
+// exponent is then not a plain one), by an integer addition to the exponent.
+__device__ __forceinline__ double from_fx_pow2(ll x, int p2) {
+    const double d = __ll2double_rn(x);
+    return x == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (p2 << 20), __double2loint(d));
+}
+
 // ---- passes -------------------------------------------------------------------
 
 // One butterfly of radix R over span M (M <= 0: run-time span Mr); FIRST reads
 // FP64 values.  Results with twiddles (span > 1) are halved.
 template <int R, int M, bool FIRST>
-__device__ __forceinline__ void bfly(V* z, int at, int Mr, const int4* tw, int n1, int base) {
+__device__ __forceinline__ void bfly(V* z, int at, int Mr, const int4* tw, int n1, int shift) {
     const int m = M > 0 ? M : Mr;
     V a[R];
 #pragma unroll
@@ -220,7 +253,7 @@ __device__ __forceinline__ void bfly(V* z, int at, int Mr, const int4* tw, int n
         const int i = ph<double>(at + t * m);
         if constexpr (FIRST) {
             const double2 d = reinterpret_cast<const double2*>(z)[i];
-            a[t] = mk(to_fx(d.x, base), to_fx(d.y, base));
+            a[t] = mk(to_fx(d.x, shift), to_fx(d.y, shift));
         } else {
             a[t] = z[i];
         }
@@ -230,7 +263,7 @@ __device__ __forceinline__ void bfly(V* z, int at, int Mr, const int4* tw, int n
         a[0] = mk(a[0].x >> 1, a[0].y >> 1);
         if (n1 != 0) {
 #pragma unroll
-            for (int k1 = 1; k1 < R; ++k1) a[k1] = cmul63(a[k1], tw[(k1 - 1) * m + n1]);
+            for (int k1 = 1; k1 < R; ++k1) a[k1] = cmul63(a[k1], __ldg(tw + (k1 - 1) * m + n1));
         } else {
 #pragma unroll
             for (int k1 = 1; k1 < R; ++k1) a[k1] = mk(a[k1].x >> 1, a[k1].y >> 1);
@@ -250,12 +283,12 @@ __device__ __forceinline__ void pass_rt(V* rows, int nrows, int nf, int LP, cons
         const int blk = b / M, n1 = b - blk * M;
         V* z = rows + (size_t)row * LP;
         const int at = blk * S + n1;
-        const int base = FIRST ? fd[row < nf ? row : row - nf].base : 0;
-        if (r == 8) bfly<8, 0, FIRST>(z, at, M, tw, n1, base);
-        else if (r == 4) bfly<4, 0, FIRST>(z, at, M, tw, n1, base);
-        else if (r == 2) bfly<2, 0, FIRST>(z, at, M, tw, n1, base);
-        else if (r == 5) bfly<5, 0, FIRST>(z, at, M, tw, n1, base);
-        else bfly<3, 0, FIRST>(z, at, M, tw, n1, base);
+        const int shift = FIRST ? fd[row < nf ? row : row - nf].shift : 0;
+        if (r == 8) bfly<8, 0, FIRST>(z, at, M, tw, n1, shift);
+        else if (r == 4) bfly<4, 0, FIRST>(z, at, M, tw, n1, shift);
+        else if (r == 2) bfly<2, 0, FIRST>(z, at, M, tw, n1, shift);
+        else if (r == 5) bfly<5, 0, FIRST>(z, at, M, tw, n1, shift);
+        else bfly<3, 0, FIRST>(z, at, M, tw, n1, shift);
     }
     __syncthreads();
 }
@@ -270,9 +303,9 @@ __device__ __forceinline__ void passes_ct(V* rows, int nrows, int nf, int LP, co
         for (int idx = threadIdx.x; idx < nrows * NB; idx += NT) {
             const int row = idx / NB, b = idx - row * NB;
             const int blk = b / M, n1 = b - blk * M;
-            const int base = FIRST ? fd[row < nf ? row : row - nf].base : 0;
+            const int shift = FIRST ? fd[row < nf ? row : row - nf].shift : 0;
             bfly<R, M, FIRST>(rows + (size_t)row * LP, blk * S + n1, M, twp + F.twoff[P], n1,
-                              base);
+                              shift);
         }
         __syncthreads();
         passes_ct<L, P + 1, CONV>(rows, nrows, nf, LP, twp, fd);
@@ -289,8 +322,8 @@ __device__ __forceinline__ void passes(V* rows, int nrows, int nf, int LP, const
         if (CONV && sh.npass == 0) {   // rows of one complex value
             for (int r = threadIdx.x; r < nrows; r += NT) {
                 const double2 d = reinterpret_cast<const double2*>(rows)[(size_t)r * LP];
-                const int base = fd[r < nf ? r : r - nf].base;
-                rows[(size_t)r * LP] = mk(to_fx(d.x, base), to_fx(d.y, base));
+                const int shift = fd[r < nf ? r : r - nf].shift;
+                rows[(size_t)r * LP] = mk(to_fx(d.x, shift), to_fx(d.y, shift));
             }
             __syncthreads();
         }
@@ -332,6 +365,17 @@ __device__ __forceinline__ float pass_bound(const FftShape& sh, float zmax, floa
     }
 }
 
+// Reduce a thread's share of one row into its field.
+__device__ __forceinline__ void gather_row(Field& fd, int row, unsigned hm, float l1) {
+    hm = __reduce_max_sync(0xffffffffu, hm);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&fd.hmax, hm);
+        fd.l1[row][threadIdx.x >> 5] = l1;
+    }
+}
+
 extern __shared__ __align__(16) unsigned char fx_smem[];
 
 template <int LT, bool STRIDED>
@@ -340,8 +384,8 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<double>& A, int fg, int j
     const int LP = A.LP;
     V* rows = reinterpret_cast<V*>(fx_smem);
     const double2* raw = reinterpret_cast<const double2*>(fx_smem);
-    int4* tws = reinterpret_cast<int4*>(rows + (size_t)2 * A.G * LP);
-    Field* fd = reinterpret_cast<Field*>(tws + L);
+    const int4* tws = reinterpret_cast<const int4*>(A.twp);
+    Field* fd = reinterpret_cast<Field*>(rows + (size_t)2 * A.G * LP);
     const int f0 = fg * A.G;
     const int nf = min(A.G, A.F - f0);
     const bool equator = (jh == A.Jh - 1);
@@ -349,8 +393,8 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<double>& A, int fg, int j
     const int tid = threadIdx.x;
 
     for (int f = tid; f < nf; f += NT) {
-        fd[f].emax = 0;
-        fd[f].l1[0] = fd[f].l1[1] = 0u;
+        fd[f].hmax = 0u;
+        for (int w = 0; w < NT / 32; ++w) fd[f].l1[1][w] = 0.f;   // no southern Equator row
     }
     const int s = A.src.elem_stride;
     for (int r = 0; r < nrows; ++r) {
@@ -369,39 +413,27 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<double>& A, int fg, int j
             }
         }
     }
-    load_twiddles_async(tws, reinterpret_cast<const int4*>(A.twp),
-                        LT > 0 ? FacOf<(LT > 0 ? LT : 2), true>::v.twtotal : A.shape.twtotal);
     cp_async_wait_all();
     __syncthreads();
-    // the largest component of each field, then the L1 norm of each row
+    // the largest component of each field and the L1 norm of each row
     for (int r = 0; r < nrows; ++r) {
-        unsigned h = 0;
+        unsigned hm = 0u;
+        float l1 = 0.f;
         for (int k = tid; k < L; k += NT) {
             const double2 v = raw[(size_t)r * LP + ph<double>(k)];
-            h = max(h, max(hi_abs(v.x), hi_abs(v.y)));
+            const unsigned hx = hi_abs(v.x), hy = hi_abs(v.y);
+            hm = max(hm, max(hx, hy));
+            l1 += abs_f32(hx) + abs_f32(hy);
         }
-        h = __reduce_max_sync(0xffffffffu, h);
-        if ((tid & 31) == 0) atomicMax(&fd[r < nf ? r : r - nf].emax, (int)(h >> 20));
-    }
-    __syncthreads();
-    for (int r = 0; r < nrows; ++r) {
-        const int f = r < nf ? r : r - nf;
-        const int E = max(fd[f].emax, 1);
-        unsigned u = 0;
-        for (int k = tid; k < L; k += NT) {
-            const double2 v = raw[(size_t)r * LP + ph<double>(k)];
-            u += l1_units(v.x, E) + l1_units(v.y, E);
-        }
-        u = __reduce_add_sync(0xffffffffu, u);
-        if ((tid & 31) == 0) atomicAdd(&fd[f].l1[r < nf ? 0 : 1], u);
+        gather_row(fd[r < nf ? r : r - nf], r < nf ? 0 : 1, hm, l1);
     }
     __syncthreads();
     if (tid < nf) {
         Field& q = fd[tid];
-        const float l1 = (float)max(q.l1[0], q.l1[1]) * (1.f / 8192.f);
-        int h;
-        const float b = pass_bound<LT>(A.shape, 1.4142136f, l1, 2.f, h);
-        finish_field(q, b, h, A.rowscale ? A.rowscale[jh] : 1.0);
+        finish_field(
+            q, fmaxf(q.norm(0), q.norm(1)),
+            [&](float l1, int& k) { return pass_bound<LT>(A.shape, 1.4142136f, l1, 2.f, k); },
+            A.rowscale ? A.rowscale[jh] : 1.0);
     }
     __syncthreads();
     passes<LT, true>(rows, nrows, nf, LP, A.shape, tws, fd);
@@ -420,8 +452,8 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<double>& A, int fg, int j
         const int m = w.major, fl = w.minor;
         double2 os = make_double2(0.0, 0.0), oa = os;
         if (m <= kmax) {
-            const int pm = ph<double>(rev_of<double, LT>(m, A.rev));
-            const int pc = ph<double>(rev_of<double, LT>(m == 0 ? 0 : L - m, A.rev));
+            const int pm = ph<double>(__ldg(A.rev + m));
+            const int pc = ph<double>(__ldg(A.rev + (m == 0 ? 0 : L - m)));
             const int4 wt = post[m];
             const V* zn = rows + (size_t)fl * LP;
             const V xn = real_spec(zn[pm], zn[pc], wt, m == 0);
@@ -454,16 +486,16 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
     const int LP = A.LP;
     V* rows = reinterpret_cast<V*>(fx_smem);
     const double2* raw = reinterpret_cast<const double2*>(fx_smem);
-    int4* tws = reinterpret_cast<int4*>(rows + (size_t)2 * A.G * LP);
-    Field* fd = reinterpret_cast<Field*>(tws + L);
+    const int4* tws = reinterpret_cast<const int4*>(A.twp);
+    Field* fd = reinterpret_cast<Field*>(rows + (size_t)2 * A.G * LP);
     const int f0 = fg * A.G;
     const int nf = min(A.G, A.F - f0);
     const bool equator = (jh == A.Jh - 1);
     const int nrows = equator ? nf : 2 * nf;
     const int tid = threadIdx.x;
     for (int f = tid; f < nf; f += NT) {
-        fd[f].emax = 0;
-        fd[f].l1[0] = fd[f].l1[1] = 0u;
+        fd[f].hmax = 0u;
+        for (int w = 0; w < NT / 32; ++w) fd[f].l1[1][w] = 0.f;   // no southern Equator row
     }
     // S lands in the northern row, A in the southern one; a reduced-grid row
     // carries the wavenumbers up to min(N, L - 1)
@@ -475,46 +507,39 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
         cp_async<16>(d, src);
         if (!equator) cp_async<16>(d + (size_t)nf * LP, src + (size_t)A.Jh * A.F);
     }
-    load_twiddles_async(tws, reinterpret_cast<const int4*>(A.twp),
-                        LT > 0 ? FacOf<(LT > 0 ? LT : 2), true>::v.twtotal : A.shape.twtotal);
     cp_async_wait_all();
     __syncthreads();
     // the largest component of S and A of each field and their L1 norms (Im
-    // at m = 0 is not an input)
+    // at m = 0 is not an input; Re there counts twice, as Y_0 may)
     for (int r = 0; r < nrows; ++r) {
-        unsigned h = 0;
+        unsigned hm = 0u;
+        float l1 = 0.f;
         for (int k = tid; k <= kmax; k += NT) {
             const double2 v = raw[(size_t)r * LP + ph<double>(k)];
-            h = max(h, max(hi_abs(v.x), k == 0 ? 0u : hi_abs(v.y)));
+            const unsigned hx = hi_abs(v.x), hy = k == 0 ? hx : hi_abs(v.y);
+            hm = max(hm, max(hx, hy));
+            l1 += abs_f32(hx) + abs_f32(hy);
         }
-        h = __reduce_max_sync(0xffffffffu, h);
-        if ((tid & 31) == 0) atomicMax(&fd[r < nf ? r : r - nf].emax, (int)(h >> 20));
-    }
-    __syncthreads();
-    for (int r = 0; r < nrows; ++r) {
-        const int f = r < nf ? r : r - nf;
-        const int E = max(fd[f].emax, 1);
-        unsigned u = 0;
-        for (int k = tid; k <= kmax; k += NT) {
-            const double2 v = raw[(size_t)r * LP + ph<double>(k)];
-            u += l1_units(v.x, E) + (k == 0 ? l1_units(v.x, E) : l1_units(v.y, E));
-        }
-        u = __reduce_add_sync(0xffffffffu, u);
-        if ((tid & 31) == 0) atomicAdd(&fd[f].l1[r < nf ? 0 : 1], u);
+        gather_row(fd[r < nf ? r : r - nf], r < nf ? 0 : 1, hm, l1);
     }
     __syncthreads();
     // The factor of the m >= 1 terms (1, or 1/2 for an adjoint) goes into the
-    // scale, its inverse into Y_0 (counted twice in the L1 norm above).
+    // scale, its inverse into Y_0.
     const int y0_shift = A.mfactor1 == 0.5 ? 1 : 0;
     if (tid < nf) {
         Field& q = fd[tid];
-        const float l1 = (float)(q.l1[0] + q.l1[1]) * (1.f / 8192.f);
         // packed values: |Z_q| / 2 <= |Y_q| + |Y_{L-q}|, |Y| <= |S| + |A|; the
         // phase of a shifted row may raise a component by sqrt(2)
-        if (A.shiftph && q.emax < 0x7fe) ++q.emax;
-        int h;
-        const float b = pass_bound<LT>(A.shape, 5.656855f, 2.f * l1, 1.f, h);
-        finish_field(q, b, h + 1, A.mfactor1 * (A.rowscale ? A.rowscale[jh] : 1.0));
+        if (A.shiftph && q.hmax < 0x7fe00000u) q.hmax += 0x100000u;
+        finish_field(
+            q, q.norm(0) + q.norm(1),
+            [&](float l1, int& k) {
+                // (two outputs per input: the L1 norm of the packed values)
+                const float b = pass_bound<LT>(A.shape, 5.656855f, 2.f * l1, 1.f, k);
+                ++k;
+                return b;
+            },
+            A.mfactor1 * (A.rowscale ? A.rowscale[jh] : 1.0));
     }
     __syncthreads();
     // One thread owns frequencies q and L - q of all fields and both
@@ -531,7 +556,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
         for (int fl = 0; fl < nf; ++fl) {
             V* zn = rows + (size_t)fl * LP;
             V* zs = zn + (size_t)nf * LP;
-            const int base = fd[fl].base;
+            const int shift = fd[fl].shift;
             auto get = [&](const V* z, int pos, int k) -> V {
                 double2 d = reinterpret_cast<const double2*>(z)[pos];
                 if (A.shiftph) {
@@ -540,7 +565,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
                     if (k == 0) d.y = 0.0;
                     d = make_double2(d.x * p.x + d.y * p.y, d.y * p.x - d.x * p.y);
                 }
-                return mk(to_fx(d.x, base), to_fx(d.y, base));
+                return mk(to_fx(d.x, shift), to_fx(d.y, shift));
             };
             const V zero = mk(0, 0);
             const V Sq = hq ? get(zn, pq, q) : zero, Aq = hq && !equator ? get(zs, pq, q) : zero;
@@ -571,9 +596,17 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
         double2* x2 = A.grid2 ? reinterpret_cast<double2*>(A.grid2 + off) : nullptr;
         const V* z = rows + (size_t)r * LP;
         const double sc = fd[fl].sc, sc2 = fd[fl].sc2;
+        // without row weights the scale is a power of two (exponent p2, far
+        // inside the range unless the field is at its ends)
+        const int p2 = ((__double2hiint(sc) >> 20) & 0x7ff) - 1023;
+        const bool pow2 = A.rowscale == nullptr && sc2 == 1.0 && p2 > -900 && p2 < 900;
         for (int k = tid; k < L; k += NT) {
-            const V v = z[ph<double>(rev_of<double, LT>(k, A.rev))];
-            double2 y = make_double2(from_fx(v.x, sc, sc2), from_fx(-v.y, sc, sc2));
+            const V v = z[ph<double>(__ldg(A.rev + k))];
+            double2 y;
+            if (pow2)
+                y = make_double2(from_fx_pow2(v.x, p2), from_fx_pow2(-v.y, p2));
+            else
+                y = make_double2(from_fx(v.x, sc, sc2), from_fx(-v.y, sc, sc2));
             if (A.accumulate == 1) {
                 const double2 g = xv[k];
                 y = make_double2(g.x + y.x, g.y + y.y);
@@ -589,18 +622,18 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
 }
 
 template <int LT, bool STRIDED>
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, 4)
     fx_forward_kernel(const __grid_constant__ FwdArgs<double> A) {
     fwd_body<LT, STRIDED>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
 }
 
 template <int LT>
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, 4)
     fx_inverse_kernel(const __grid_constant__ InvArgs<double> A) {
     inv_body<LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
 }
 
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, 4)
     fx_forward_ragged_kernel(const __grid_constant__ RaggedFwd<double> R) {
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<double> A = R.a;
@@ -608,7 +641,7 @@ __global__ void __launch_bounds__(NT, 2)
     fwd_body<-1, false>(A, blockIdx.x, jh);
 }
 
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, 4)
     fx_inverse_ragged_kernel(const __grid_constant__ RaggedInv<double> R) {
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<double> A = R.a;
@@ -630,7 +663,7 @@ __global__ void __launch_bounds__(NT, 2)
     }
 
 // the plan's half-length picks its compile-time body (one branch per CTA)
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, 4)
     fx_forward_group_kernel(const __grid_constant__ FwdGroup<double> G) {
     const int b = blockIdx.x;
     int p = 0;
@@ -643,7 +676,7 @@ __global__ void __launch_bounds__(NT, 2)
 #undef SHT_CALL
 }
 
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, 4)
     fx_inverse_group_kernel(const __grid_constant__ InvGroup<double> G) {
     const int b = blockIdx.x;
     int p = 0;

@@ -137,6 +137,9 @@ inline bool fft_has_fixed_kernel(int L) {
            L == 1280;
 }
 
+// Shared memory per field of the FP64 FFT kernels beside the rows.
+constexpr size_t kFxFieldBytes = 96;
+
 enum Stage { kStageFftFwd = 0, kStageLegFwd = 1, kStageLegInv = 2,
              kStageFftInv = 3, kStageSplitConv = 4 };
 
