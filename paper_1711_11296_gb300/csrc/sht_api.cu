@@ -214,16 +214,10 @@ extern "C" int sht_plan_create_grid(int N, int J, int I, int nfields, int precis
     p->fft = shape;
     const bool fp64 = precision == SHT_FP64;
     const size_t vbytes = fp64 ? sizeof(double2) : sizeof(float2);
-    const size_t rowbytes = (size_t)fft_row_pitch(shape.L, fp64) * vbytes;
-    const size_t budget = 110 * 1024;
-    long g = (long)((budget / rowbytes > 1 ? budget / rowbytes - 1 : 0) / 2);
-    if (g < 1) g = 1;
-    if (g > 16) g = 16;
-    if (g > nfields) g = nfields;
-    p->G = (int)g;
+    p->G = fft_default_fields(I, p->Jh, nfields, fp64);
     p->fft_threads = 256;
     p->fft_smem = fft_smem_bytes(I, p->G, fp64);
-    if (p->fft_smem > 227 * 1024) {
+    if (p->G == 0) {
         delete p;
         set_error("I = %d too large for the shared-memory FFT", I);
         return SHT_ERR_UNSUPPORTED;

@@ -1512,6 +1512,25 @@ size_t fft_smem_bytes(int I, int G, bool fp64) {
     return (rows + L) * sizeof(float2) + 8 * (size_t)G;
 }
 
+// The largest power of two that leaves room for the CTAs an SM holds by
+// registers (FP32 two, FP64 four) and keeps the grid at 256 (FP64: 512) CTAs
+// or more.  A power of two: the threads then divide into whole groups of
+// fields and a CTA's workspace pieces into whole sectors (forward / inverse
+// us: T319 x 300 bf16x3, 10 fields 443 / 486, 8 fields 370 / 418; T255 x 256,
+// 12 fields 229 / 241, 8 fields 206 / 216; Tc479 x 64, 6 fields 402 / 497, 4
+// fields 369 / 449).  Small grids (T31 x 32 bf16x3): 16 fields, 66 CTAs
+// 10.0 / 11.4, 4 fields, 264 CTAs 8.4 / 8.0; FP64 T63 x 16: 8 fields, 130
+// CTAs 18.0 / 22.4, 2 fields, 520 CTAs 15.1 / 14.2.
+int fft_default_fields(int I, int Jh, int F, bool fp64) {
+    const size_t budget = (fp64 ? 55 : 112) * 1024;
+    const long ctas = fp64 ? 512 : 256;
+    int g = 16;
+    while (g > 1 && (g > F || fft_smem_bytes(I, g, fp64) > budget ||
+                     (long)Jh * ((F + g - 1) / g) < ctas))
+        g /= 2;
+    return fft_smem_bytes(I, g, fp64) <= 227 * 1024 ? g : 0;
+}
+
 cudaError_t launch_fft_forward(const sht_plan_s* p, const void* grid,
                                const RowSource& src, const FwdScale& sc,
                                void* work, cudaStream_t s) {

@@ -223,8 +223,11 @@ __device__ __forceinline__ void finish_field(Field& fd, float l1, Bound bound, d
     fd.shift = SH - e;
     const int p2 = e - SH + k;
     const bool tiny = p2 < -900;   // 2^p2 would be subnormal
+    // (zero rows give zeros, not the last place's rounding; values that are
+    // all below 2^-1042, whose high words are 0, count as zero)
     fd.sc = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                       : ldexp(f, tiny ? p2 + 200 : p2);
+            : fd.hmax == 0u ? 0.0
+                            : ldexp(f, tiny ? p2 + 200 : p2);
     fd.sc2 = tiny ? 6.223015277861142e-61 : 1.0;   // 2^-200
 }
 
@@ -530,7 +533,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
         Field& q = fd[tid];
         // packed values: |Z_q| / 2 <= |Y_q| + |Y_{L-q}|, |Y| <= |S| + |A|; the
         // phase of a shifted row may raise a component by sqrt(2)
-        if (A.shiftph && q.hmax < 0x7fe00000u) q.hmax += 0x100000u;
+        if (A.shiftph && q.hmax != 0u && q.hmax < 0x7fe00000u) q.hmax += 0x100000u;
         finish_field(
             q, q.norm(0) + q.norm(1),
             [&](float l1, int& k) {

@@ -308,6 +308,8 @@ cudaError_t launch_fft_forward_group(sht_plan_s* const* plans, int n,
 cudaError_t launch_fft_inverse_group(sht_plan_s* const* plans, int n,
                                      void* const* grids, cudaStream_t s);
 size_t fft_smem_bytes(int I, int G, bool fp64);
+// Fields per FFT CTA of a plan before any tuning (0: the rows do not fit).
+int fft_default_fields(int I, int Jh, int F, bool fp64);
 
 // FP64 Legendre launches
 cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,

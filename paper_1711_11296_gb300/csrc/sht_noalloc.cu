@@ -174,14 +174,10 @@ extern "C" int sht_forward_noalloc(int N, int J, int I, int nfields,
     t.ncoef = (size_t)(N + 1) * (N + 2) / 2;
     t.ldp = (t.Jh + 7) / 8 * 8;
     t.fft = shape;
-    const size_t rowbytes = (size_t)fft_row_pitch(shape.L, true) * sizeof(double2);
-    const size_t budget = 110 * 1024;
-    long g = (long)((budget / rowbytes > 1 ? budget / rowbytes - 1 : 0) / 2);
-    g = g < 1 ? 1 : (g > 16 ? 16 : g);
-    t.G = (int)(g > nfields ? nfields : g);
+    t.G = fft_default_fields(I, t.Jh, nfields, true);
     t.fft_threads = 256;
     t.fft_smem = fft_smem_bytes(I, t.G, true);
-    if (t.fft_smem > 227 * 1024) {
+    if (t.G == 0) {
         set_error("I = %d too large for the shared-memory FFT", I);
         return SHT_ERR_UNSUPPORTED;
     }
