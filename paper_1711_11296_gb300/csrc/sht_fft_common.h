@@ -203,6 +203,29 @@ __device__ __forceinline__ void apply_shape(Args& A, const R& Rg, int jh) {
     }
 }
 
+// FP32 launches of the kernels in other translation units, and the upload of
+// their constant twiddles to the current device.
+cudaError_t fft_any_init();
+cudaError_t fft_any_forward(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
+                            cudaStream_t s);
+cudaError_t fft_any_inverse(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s);
+cudaError_t fft_any_forward_ragged(const RaggedFwd<float>& R, dim3 grid, size_t smem,
+                                   cudaStream_t s);
+cudaError_t fft_any_inverse_ragged(const RaggedInv<float>& R, dim3 grid, size_t smem,
+                                   cudaStream_t s);
+cudaError_t fft_bluestein_init();
+cudaError_t fft_bluestein_forward(const RaggedFwd<float>& R, dim3 grid, size_t smem,
+                                  cudaStream_t s);
+cudaError_t fft_bluestein_forward(const RaggedFwd<double>& R, dim3 grid, size_t smem,
+                                  cudaStream_t s);
+cudaError_t fft_bluestein_inverse(const RaggedInv<float>& R, dim3 grid, size_t smem,
+                                  cudaStream_t s);
+cudaError_t fft_bluestein_inverse(const RaggedInv<double>& R, dim3 grid, size_t smem,
+                                  cudaStream_t s);
+cudaError_t fft_group_init();
+cudaError_t fft_group_forward(const FwdGroup<float>& G, int ctas, size_t smem, cudaStream_t s);
+cudaError_t fft_group_inverse(const InvGroup<float>& G, int ctas, size_t smem, cudaStream_t s);
+
 // Fixed-point FFT launches of the FP64 path (sht_fft64.cu); the arguments'
 // twiddle tables are the fixed-point ones (launch_fixed_twiddles).
 cudaError_t fx_forward(const FwdArgs<double>& A, bool strided, dim3 grid, size_t smem,
