@@ -47,7 +47,7 @@ struct DeviceGuard {
 
 bool factor_fft(int L, bool fp64, FftShape& sh) {
     if (!fft_factorable(L)) return false;
-    sh = fft_shape(L, fp64);
+    sh = fft_shape(L, fp64, fft_has_fixed_kernel(L));
     return true;
 }
 

@@ -345,14 +345,14 @@ cudaError_t launch_fft_inverse_group(sht_plan_s* const* plans, int n,
 }
 
 // Factorisation of a half-length for the kernels with run-time shapes.  FP32
-// lengths other than the compile-time ones take the passes, out of every
-// register DFT size, with the least estimated time: per pass and value 14
+// lengths take the passes, out of the register DFT sizes those kernels hold
+// (with_radix), with the least estimated time: per pass and value 14
 // instructions of shared-memory traffic, twiddles and addresses plus the
 // DFT's own, over the share of the CTA's threads that have a butterfly in
 // the rounds of its (nominal) rows.  Two or three passes of large radices
 // then replace up to five of 2 .. 8.
-FftShape fft_shape(int L, bool fp64) {
-    if (fp64 || L == 1 || fft_has_fixed_kernel(L)) return fft_factor(L, fp64);
+FftShape fft_shape(int L, bool fp64, bool compile_time) {
+    if (fp64 || L == 1 || compile_time) return fft_factor(L, fp64);
     struct Size { int r; float work; };   // instructions of the DFT per value
     static const Size sizes[] = {{2, 1.f}, {3, 3.f}, {4, 2.5f}, {5, 6.f}, {6, 5.3f}, {8, 5.f},
                                  {9, 7.8f}, {10, 8.6f}, {12, 7.5f}, {15, 11.f}, {16, 7.3f},

@@ -288,9 +288,10 @@ __host__ __device__ constexpr FftShape fft_factor(int L, bool fp64) {
     return sh;
 }
 
-// The plan-time choice: the above for FP64 and the compile-time lengths, else
-// passes of any register DFT size (2 .. 40).
-FftShape fft_shape(int L, bool fp64);
+// The plan-time choice: the above for FP64 and where the compile-time kernel
+// of the length will run, else passes of the register DFT sizes that the
+// kernels with run-time shapes hold (2 .. 32).
+FftShape fft_shape(int L, bool fp64, bool compile_time);
 
 __host__ __device__ constexpr bool fft_factorable(int L) {
     return L == 1 || fft_factor(L, true).npass > 0;

@@ -144,14 +144,14 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
             r.L = L;
             if (route == kRouteBluestein) {
                 r.bluestein = 1;
-                r.sh = fft_shape(small_radix_ceil(2 * L - 1), fp64);
+                r.sh = fft_shape(small_radix_ceil(2 * L - 1), fp64, false);
                 r.chirp_off = chirp_total;
                 r.dft_off = dft_total;
                 chirp_total += L;
                 dft_total += r.sh.L;
                 L2max = std::max(L2max, r.sh.L);
             } else {
-                r.sh = fft_shape(L, fp64);
+                r.sh = fft_shape(L, fp64, route == kRouteClass);
             }
             r.tw_off = tw_total;
             r.post_off = post_total;

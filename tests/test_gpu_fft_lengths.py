@@ -1,0 +1,81 @@
+"""FP32 FFT shapes read at run time, against the oracle: regular rows of
+lengths without a compile-time kernel (one to three passes of register DFT
+sizes, odd ones among them), reduced-grid rows of compile-time lengths that a
+half-spacing shift sends to the run-time kernel, and rows transformed by
+Bluestein's method with convolution lengths on either side of and equal to
+the compile-time ones.
+
+Tolerance: the split transform's (1e-6, relative L2); the FFT's rounding is
+an order below it."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_1711_11296_gb300 import workloads as W
+from sht_testutil import built_lib, rel_l2, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-6
+N, J = 12, 27
+
+
+@pytest.fixture(scope="module")
+def sht():
+    built_lib()
+    from paper_1711_11296_gb300 import sht as S
+    return S
+
+
+@pytest.mark.parametrize("L", [15, 25, 27, 32, 45, 81, 96, 125, 160, 192, 225, 243, 250, 288,
+                               375, 384, 405, 480, 500, 625, 720, 768, 810, 900, 960, 1000,
+                               1125, 1350, 1536, 1600, 2000, 2048, 4096])
+@pytest.mark.parametrize("F", [1, 5])
+def test_regular_rows(sht, L, F):
+    I = 2 * L
+    p = sht.Plan(N, J, I, F, "bf16x3")
+    x = W.random_grid(F, J, I, seed=2500 + L).astype(np.float32).astype(np.float64)
+    a = W.random_spectrum(N, F, "flat", seed=2600 + L).astype(np.complex64)
+    assert rel_l2(p.forward(to_cuda(x, torch.float32)).cpu().numpy(), O.analysis(x, N)) <= TOL
+    got = p.inverse(torch.from_numpy(a).cuda()).cpu().numpy()
+    assert rel_l2(got, O.synthesis(a.astype(np.complex128), N, J, I)) <= TOL
+    p.status()
+
+
+def _reduced(sht, pts, shift, F):
+    p = sht.Plan(N, J, max(pts), F, "bf16x3", grid="reduced", lat_points=pts, half_shift=shift)
+    x = np.random.default_rng(sum(pts)).standard_normal((F, sum(pts)))
+    x = x.astype(np.float32).astype(np.float64)
+    a = W.random_spectrum(N, F, "flat", seed=2700 + pts[0]).astype(np.complex64)
+    got = p.forward(to_cuda(x, torch.float32)).cpu().numpy()
+    spacings = None if shift is None else [0.5 * v for v in shift]
+    ref = O.analysis_reduced(x, N, J, pts, shifts=spacings)
+    assert rel_l2(got, ref) <= TOL
+    got = p.inverse(torch.from_numpy(a).cuda()).cpu().numpy()
+    ref = O.synthesis_reduced(a.astype(np.complex128), N, J, pts, shifts=spacings)
+    assert rel_l2(got, ref) <= TOL
+    p.status()
+
+
+@pytest.mark.parametrize("L", [64, 128, 256, 320, 512, 640, 1024, 1280])
+def test_shifted_rows_of_compile_time_lengths(sht, L):
+    _reduced(sht, [2 * L] * J, [1] * J, 3)
+
+
+@pytest.mark.parametrize("L2", [64, 256, 320, 512, 640, 1024, 1280, 1350])
+@pytest.mark.parametrize("F", [1, 6])
+def test_bluestein_convolution_lengths(sht, L2, F):
+    # the longest row whose convolution takes L2 points and has a prime factor
+    # above 5, and shorter rows beside it
+    L = max(k for k in range(14, L2 // 2 + 1) if 2 * k - 1 <= L2 and _big_prime(k))
+    pts = [2 * L - 2 * (j % 3) if j != J // 2 else 2 * L for j in range((J + 1) // 2)]
+    pts = pts + pts[-2::-1]
+    _reduced(sht, pts, None, F)
+
+
+def _big_prime(n):
+    for q in (2, 3, 5):
+        while n % q == 0:
+            n //= q
+    return n > 1
