@@ -351,7 +351,8 @@ cudaError_t launch_fft_inverse_group(sht_plan_s* const* plans, int n,
 // DFT's own, over the share of the CTA's threads that have a butterfly in
 // the rounds of its (nominal) rows.  Two or three passes of large radices
 // then replace up to five of 2 .. 8.
-FftShape fft_shape(int L, bool fp64, bool compile_time) {
+FftShape fft_shape(int L, bool fp64, bool compile_time, float* time) {
+    if (time) *time = 0.f;
     if (fp64 || L == 1 || compile_time) return fft_factor(L, fp64);
     struct Size { int r; float work; };   // instructions of the DFT per value
     static const Size sizes[] = {{2, 1.f}, {3, 3.f}, {4, 2.5f}, {5, 6.f}, {6, 5.3f}, {8, 5.f},
@@ -383,6 +384,7 @@ FftShape fft_shape(int L, bool fp64, bool compile_time) {
     };
     search(search, L, 0, 0, 0.f);
     if (nbest == 0) return fft_factor(L, true);
+    if (time) *time = tbest * (float)L;
     FftShape sh{};
     sh.L = L;
     sh.npass = nbest;
@@ -402,12 +404,10 @@ FftShape fft_shape(int L, bool fp64, bool compile_time) {
     return sh;
 }
 
-size_t bluestein_smem_bytes(int Lmax, int L2, int G, bool fp64) {
+size_t bluestein_smem_bytes(int L2, int G, bool fp64) {
     const size_t v = fp64 ? sizeof(double2) : sizeof(float2);
-    // rows | twiddles of length L2 | column maxima (2 G words, rounded up to
-    // whole complex values) | two scratch rows of length L2
-    return (2 * (size_t)G * fft_row_pitch(Lmax, fp64) + L2 + (8 * (size_t)G + v - 1) / v +
-            2 * (size_t)fft_row_pitch(L2, fp64)) * v;
+    // rows of length L2 | twiddles of length L2 | column maxima (2 G words)
+    return (2 * (size_t)G * fft_row_pitch(L2, fp64) + L2) * v + 8 * (size_t)G;
 }
 
 size_t fft_smem_bytes(int I, int G, bool fp64) {

@@ -437,39 +437,73 @@ __device__ __forceinline__ void run_passes(typename Vec2<T>::type* rows, int nro
         passes_runtime<T>(rows, nrows, LP, sh, 0, sh.npass, twp);
 }
 
-// Bluestein's chirp-z DFT of each of nrows padded rows of half-length L (any
-// L; natural order in and out), for the rows of reduced grids whose L has a
-// prime factor above 5.  With c_n = e^{-i pi n^2 / L},
+// Bluestein's chirp-z DFT of rows of half-length L (any L), for the rows of
+// reduced grids whose L has a prime factor above 5.  With
+// c_n = e^{-i pi n^2 / L},
 //   Z_k = sum_n z_n e^{-2 pi i n k / L} = c_k sum_n (z_n c_n) conj(c_{k-n}),
-// a circular convolution of length L2 >= 2L - 1 (sh2.L, 2-3-5-smooth) of
+// a circular convolution of length L2 >= 2L - 1 (sh.L, 2-3-5-smooth) of
 // a_n = z_n c_n (zero-padded) with the conjugate chirp wrapped around L2,
-// whose DFT D (divided by L2) is a table.  Per row: the FFT of a, the
-// pointwise product with D, conjugated and moved to natural order, a second
-// FFT, and Z_k = c_k conj(result at k).  b1, b2: two padded scratch rows of
-// length L2; tws: the per-pass twiddles of length L2; rev2: its digit
-// reversal.
+// whose DFT D (divided by L2) is a table:
+//   Z_k = c_k conj(r_k),  r = DFT(conj(DFT(a) D)).
+// In place on nrows padded rows at once: on entry a, on return r, both in
+// natural order.  The first DFT runs its passes forwards (decimation in
+// frequency) and leaves the digit-reversed order; the second runs the
+// transposed passes backwards (decimation in time), which takes that order
+// back to the natural one, so nothing is permuted.  The last pass of the
+// first and the first of the second work on the same R contiguous values
+// (span 1): one butterfly in registers does both, with the product by D
+// between (D in the order in which the threads read it, see
+// bluestein_dft_kernel).
 template <typename T>
-__device__ void bluestein_rows(typename Vec2<T>::type* rows, int nrows, int LP, int L,
-                               const FftShape& sh2, const typename Vec2<T>::type* tws,
-                               const typename Vec2<T>::type* chirp,
-                               const typename Vec2<T>::type* dft, const int* rev2,
-                               typename Vec2<T>::type* b1, typename Vec2<T>::type* b2) {
+__device__ __noinline__ void bluestein_rows(typename Vec2<T>::type* rows, int nrows, int LP,
+                                            const FftShape& sh,
+                                            const typename Vec2<T>::type* tws,
+                                            const typename Vec2<T>::type* dft) {
     using V = typename Vec2<T>::type;
     using K = C2<T>;
-    const int L2 = sh2.L;
-    const int tid = threadIdx.x;
-    for (int r = 0; r < nrows; ++r) {
-        V* z = rows + (size_t)r * LP;
-        for (int n = tid; n < L2; n += NT)
-            b1[ph<T>(n)] = n < L ? K::mul(z[ph<T>(n)], chirp[n]) : K::make((T)0, (T)0);
-        __syncthreads();
-        passes_runtime<T>(b1, 1, 0, sh2, 0, sh2.npass, tws);
-        for (int k = tid; k < L2; k += NT)
-            b2[ph<T>(k)] = K::conj(K::mul(b1[ph<T>(rev2[k])], dft[k]));
-        __syncthreads();
-        passes_runtime<T>(b2, 1, 0, sh2, 0, sh2.npass, tws);
-        for (int k = tid; k < L; k += NT)
-            z[ph<T>(k)] = K::mul(chirp[k], K::conj(b2[ph<T>(rev2[k])]));
+    const int np = sh.npass;
+    passes_runtime<T>(rows, nrows, LP, sh, 0, np - 1, tws);
+    with_radix<T>(sh.radix[np - 1], [&](auto rc) {
+        constexpr int R = decltype(rc)::value;
+        const int nb = sh.L / R;
+        for (int idx = threadIdx.x; idx < nrows * nb; idx += NT) {
+            const int row = idx / nb, b = idx - row * nb;
+            V* z = rows + (size_t)row * LP;
+            V a[R], y[R];
+#pragma unroll
+            for (int t = 0; t < R; ++t) a[t] = z[ph<T>(b * R + t)];
+            Dft<T, R>::run(a);
+#pragma unroll
+            for (int t = 0; t < R; ++t)
+                y[t] = K::conj(K::mul(a[Dft<T, R>::pos(t)], dft[t * nb + b]));
+            Dft<T, R>::run(y);
+#pragma unroll
+            for (int t = 0; t < R; ++t) z[ph<T>(b * R + t)] = y[Dft<T, R>::pos(t)];
+        }
+    });
+    __syncthreads();
+    for (int p = np - 2; p >= 0; --p) {
+        const int M = sh.span[p];
+        const V* tw = tws + sh.twoff[p];
+        with_radix<T>(sh.radix[p], [&](auto rc) {
+            constexpr int R = decltype(rc)::value;
+            const int nb = sh.L / R, S = R * M;
+            for (int idx = threadIdx.x; idx < nrows * nb; idx += NT) {
+                const int row = idx / nb, b = idx - row * nb;
+                const int blk = b / M, n1 = b - blk * M, at = blk * S + n1;
+                V* z = rows + (size_t)row * LP;
+                V a[R];
+#pragma unroll
+                for (int t = 0; t < R; ++t) a[t] = z[ph<T>(at + t * M)];
+                if (n1 != 0) {
+#pragma unroll
+                    for (int t = 1; t < R; ++t) a[t] = K::mul(a[t], tw[(t - 1) * M + n1]);
+                }
+                Dft<T, R>::run(a);
+#pragma unroll
+                for (int k1 = 0; k1 < R; ++k1) z[ph<T>(at + k1 * M)] = a[Dft<T, R>::pos(k1)];
+            }
+        });
         __syncthreads();
     }
 }
@@ -481,7 +515,7 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
     using V = typename Vec2<T>::type;
     using K = C2<T>;
     const int L = LT > 0 ? LT : A.L;
-    const int LP = A.LP;
+    const int LP = LT == -2 ? row_pitch<T>(A.shape.L) : A.LP;
     V* rows = reinterpret_cast<V*>(fft_smem_raw);
     V* tws = rows + (size_t)2 * A.G * LP;
     const int f0 = fg * A.G;
@@ -577,6 +611,17 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
         });
         __syncthreads();
         passes_runtime<T>(rows, nrows, LP, A.shape, 1, A.shape.npass, tws);
+    } else if constexpr (LT == -2) {
+        load_twiddles_async(tws, A.twp, A.shape.twtotal);
+        for (int r = 0; r < nrows; ++r) {
+            const V* x = reinterpret_cast<const V*>(row_ptr(r));
+            V* d = rows + (size_t)r * LP;
+            for (int n = tid; n < A.shape.L; n += NT)
+                d[ph<T>(n)] = n < L ? K::mul(x[n], A.chirp[n]) : K::make((T)0, (T)0);
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        bluestein_rows<T>(rows, nrows, LP, A.shape, tws, A.dft);
     } else {
         {
             // element k of row r goes to rows[r LP + ph(k)], copied
@@ -599,13 +644,7 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
             cp_async_wait_all();
         }
         __syncthreads();
-        if constexpr (LT == -2) {
-            V* b1 = tws + A.shape.L + (2 * A.G * 4 + sizeof(V) - 1) / sizeof(V);
-            V* b2 = b1 + row_pitch<T>(A.shape.L);
-            bluestein_rows<T>(rows, nrows, LP, L, A.shape, tws, A.chirp, A.dft, A.rev, b1, b2);
-        } else {
-            run_passes<T, LT>(rows, nrows, LP, A.shape, tws);
-        }
+        run_passes<T, LT>(rows, nrows, LP, A.shape, tws);
     }
 
     const int nout = (A.N + 1) * nf;
@@ -672,7 +711,7 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
             const int pcb = ph<T>(rev_of<T, LT>(rb == 0 ? 0 : L - rb, A.rev));
             const V* na = rows + (size_t)fa * LP;
             const V* nb = rows + (size_t)fb * LP;
-            const V a_nm = na[pma], a_nc = na[pca], b_nm = nb[pmb], b_nc = nb[pcb];
+            V a_nm = na[pma], a_nc = na[pca], b_nm = nb[pmb], b_nc = nb[pcb];
             V a_sm = K::make((T)0, (T)0), a_sc = a_sm, b_sm = a_sm, b_sc = a_sm;
             if (!equator) {
                 const V* sa = na + (size_t)nf * LP;
@@ -681,6 +720,18 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
                 a_sc = sa[pca];
                 b_sm = sb[pmb];
                 b_sc = sb[pcb];
+            }
+            if constexpr (LT == -2) {   // Z_k = c_k conj(r_k)
+                const V ca = A.chirp[ra], da = A.chirp[ra == 0 ? 0 : L - ra];
+                const V cb = A.chirp[rb], db = A.chirp[rb == 0 ? 0 : L - rb];
+                a_nm = K::mul(ca, K::conj(a_nm));
+                a_nc = K::mul(da, K::conj(a_nc));
+                a_sm = K::mul(ca, K::conj(a_sm));
+                a_sc = K::mul(da, K::conj(a_sc));
+                b_nm = K::mul(cb, K::conj(b_nm));
+                b_nc = K::mul(db, K::conj(b_nc));
+                b_sm = K::mul(cb, K::conj(b_sm));
+                b_sc = K::mul(db, K::conj(b_sc));
             }
             const V wta = A.twpost[ra], wtb = A.twpost[rb];
             const T sca = ma == 0 ? sc0 : sc1;
@@ -800,7 +851,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
     using V = typename Vec2<T>::type;
     using K = C2<T>;
     const int L = LT > 0 ? LT : A.L;
-    const int LP = A.LP;
+    const int LP = LT == -2 ? row_pitch<T>(A.shape.L) : A.LP;
     V* rows = reinterpret_cast<V*>(fft_smem_raw);
     V* tws = rows + (size_t)2 * A.G * LP;
     const int f0 = fg * A.G;
@@ -834,6 +885,11 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
     // a reduced-grid row of half-length L carries the wavenumbers up to
     // min(N, L - 1) (Y_m = 0 above)
     const int kmax = A.rowoff ? min(A.N, L - 1) : A.N;
+    if constexpr (LT == -2) {   // zero padding of the convolution
+        for (int r = 0; r < nrows; ++r)
+            for (int n = L + tid; n < A.shape.L; n += NT)
+                rows[(size_t)r * LP + ph<T>(n)] = K::make((T)0, (T)0);
+    }
     const int nin = (kmax + 1) * nf;
     for (Walk2 w(tid, nf); w.major * nf + w.minor < nin; w.next()) {
         const int m = w.major, fl = w.minor;
@@ -865,6 +921,9 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
         const V wq = K::conj(tq);
         const V wc = pair ? K::conj(tc) : wq;
         const V zero = K::make((T)0, (T)0);
+        // Bluestein rows: times the chirp
+        const V hq_c = LT == -2 ? A.chirp[q] : zero, hc_c = LT == -2 && pair ? A.chirp[qc] : zero;
+        auto chirped = [&](V z, V c) -> V { return LT == -2 ? K::mul(z, c) : z; };
         for (int fl = 0; fl < nf; ++fl) {
             V* zn = rows + (size_t)fl * LP;
             V* zs = rows + (size_t)(nf + fl) * LP;
@@ -888,11 +947,11 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
             V ynq = K::scale(K::add(Sq, Aq), fq), ysq = K::scale(K::sub(Sq, Aq), fq);
             if (q == 0) ynq.y = ysq.y = (T)0;
             const V ync = K::scale(K::add(Sc, Ac), fc), ysc = K::scale(K::sub(Sc, Ac), fc);
-            zn[pq] = pack(ynq, ync, wq);
-            if (!equator) zs[pq] = pack(ysq, ysc, wq);
+            zn[pq] = chirped(pack(ynq, ync, wq), hq_c);
+            if (!equator) zs[pq] = chirped(pack(ysq, ysc, wq), hq_c);
             if (pair) {
-                zn[pc] = pack(ync, ynq, wc);
-                if (!equator) zs[pc] = pack(ysc, ysq, wc);
+                zn[pc] = chirped(pack(ync, ynq, wc), hc_c);
+                if (!equator) zs[pc] = chirped(pack(ysc, ysq, wc), hc_c);
             }
         }
     };
@@ -909,8 +968,12 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
         const bool pair = q != 0 && q != qc;
         const V zero = K::make((T)0, (T)0);
         const T fq = q == 0 ? (T)1 : mf1;
-        const V al = K::make(fq * ((T)1 + tq.y), -fq * tq.x);    // f (1 - i W^q)
-        const V be = K::make(mf1 * ((T)1 - tc.y), mf1 * tc.x);   // f (1 + i W^{L-q})
+        V al = K::make(fq * ((T)1 + tq.y), -fq * tq.x);    // f (1 - i W^q)
+        V be = K::make(mf1 * ((T)1 - tc.y), mf1 * tc.x);   // f (1 + i W^{L-q})
+        if constexpr (LT == -2) {   // times the chirp
+            al = K::mul(al, A.chirp[q]);
+            if (pair) be = K::mul(be, A.chirp[qc]);
+        }
         if (q > kmax) {
             for (int fl = 0; fl < nf; ++fl) {
                 V* zn = rows + (size_t)fl * LP;
@@ -1053,9 +1116,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
         return;
     }
     if constexpr (LT == -2) {
-        V* b1 = tws + A.shape.L;
-        V* b2 = b1 + row_pitch<T>(A.shape.L);
-        bluestein_rows<T>(rows, nrows, LP, L, A.shape, tws, A.chirp, A.dft, A.rev, b1, b2);
+        bluestein_rows<T>(rows, nrows, LP, A.shape, tws, A.dft);
     } else {
         run_passes<T, LT>(rows, nrows, LP, A.shape, tws);
     }
@@ -1097,7 +1158,9 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
             }
         } else {
             for (int k = tid; k < L; k += NT) {
-                const V v = z[ph<T>(rev_of<T, LT>(k, A.rev))];
+                V v = z[ph<T>(rev_of<T, LT>(k, A.rev))];
+                // Bluestein rows: DFT(conj Z)_k = c_k conj(r_k)
+                if constexpr (LT == -2) v = K::mul(A.chirp[k], K::conj(v));
                 put(xv, x2, k, K::make(v.x * rs, -v.y * rs));
             }
         }

@@ -92,7 +92,8 @@ struct RShape {
     int bluestein = 0;    // 1: L has a prime factor above 5; its DFT is a
                           // chirp-z convolution of length L2 = sh.L >= 2L - 1
     long long chirp_off = 0;   // Bluestein: e^{-pi i n^2 / L}, n < L (entries)
-    long long dft_off = 0;     // Bluestein: DFT of the conjugate chirp / L2 (L2 entries)
+    long long dft_off = 0;     // Bluestein: DFT of the conjugate chirp / L2 (L2 entries,
+                               // in the order the kernel reads them)
     long long shift_off = -1;  // e^{-pi i m / I_j}, m < L (entries), or -1: none
 };
 
@@ -126,10 +127,9 @@ struct RaggedGrid {
     int* d_jh = nullptr;             // latitude-pair lists of all launches
 };
 
-// Shared memory of the Bluestein FFT kernels: the padded rows of G fields
-// (pitch of half-length Lmax), the per-pass twiddles of length L2, the
-// column maxima and two padded scratch rows of length L2.
-size_t bluestein_smem_bytes(int Lmax, int L2, int G, bool fp64);
+// Shared memory of the Bluestein FFT kernels for G fields: padded rows of
+// length L2, the per-pass twiddles and the column maxima.
+size_t bluestein_smem_bytes(int L2, int G, bool fp64);
 
 // Half-lengths with compile-time FFT kernels (the standard grids).
 inline bool fft_has_fixed_kernel(int L) {
@@ -291,7 +291,8 @@ __host__ __device__ constexpr FftShape fft_factor(int L, bool fp64) {
 // The plan-time choice: the above for FP64 and where the compile-time kernel
 // of the length will run, else passes of the register DFT sizes that the
 // kernels with run-time shapes hold (2 .. 32).
-FftShape fft_shape(int L, bool fp64, bool compile_time);
+// time: the estimate the choice was made by (0 where there was none).
+FftShape fft_shape(int L, bool fp64, bool compile_time, float* time = nullptr);
 
 __host__ __device__ constexpr bool fft_factorable(int L) {
     return L == 1 || fft_factor(L, true).npass > 0;

@@ -93,11 +93,23 @@ void ragged_free(RaggedGrid* rg) {
 
 namespace {
 
-// The smallest length >= n whose FFT factors into radices 2, 3, 4, 5 and 8
-// (the run-time kernels' radices): the Bluestein convolution length.
-int small_radix_ceil(int n) {
-    for (int m = std::max(n, 1);; ++m)
-        if (fft_factorable(m)) return m;
+// The convolution length of a Bluestein row: 2-3-5-smooth and at least n; FP64
+// the smallest, FP32 the one of the least estimated FFT time up to a quarter
+// above (the smallest may need one more pass, or odd radices).
+int bluestein_length(int n, bool fp64) {
+    int best = 0;
+    float tbest = 0.f;
+    for (int m = std::max(n, 1); best == 0 || m <= n + n / 4; ++m) {
+        if (!fft_factorable(m)) continue;
+        float t = 0.f;
+        fft_shape(m, fp64, false, &t);
+        if (best == 0 || t < tbest) {
+            best = m;
+            tbest = t;
+        }
+        if (fp64) break;
+    }
+    return best;
 }
 
 // How a latitude pair's rows are transformed.
@@ -144,7 +156,7 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
             r.L = L;
             if (route == kRouteBluestein) {
                 r.bluestein = 1;
-                r.sh = fft_shape(small_radix_ceil(2 * L - 1), fp64, false);
+                r.sh = fft_shape(bluestein_length(2 * L - 1, fp64), fp64, false);
                 r.chirp_off = chirp_total;
                 r.dft_off = dft_total;
                 chirp_total += L;
@@ -174,7 +186,8 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
     rg->nshapes = (int)shapes.size();
     rg->h_shapes = shapes;
     // launch lists: latitude pairs of each compile-time length, then the
-    // generic ones, then the Bluestein ones
+    // generic ones, then the Bluestein ones, the longest rows (nearest the
+    // Equator) first so that the last CTAs are short
     std::vector<int> jh_all;
     for (int k = 0; k < rg->nshapes; ++k) {
         if (route_of[k] != kRouteClass) continue;
@@ -185,21 +198,20 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
         rg->classes.push_back(c);
     }
     rg->generic_off = (int)jh_all.size();
-    for (int jh = 0; jh < p->Jh; ++jh)
+    for (int jh = p->Jh - 1; jh >= 0; --jh)
         if (route_of[shape_of[jh]] == kRouteGeneric) jh_all.push_back(jh);
     rg->generic_count = (int)jh_all.size() - rg->generic_off;
     rg->blue_off = (int)jh_all.size();
-    for (int jh = 0; jh < p->Jh; ++jh)
+    for (int jh = p->Jh - 1; jh >= 0; --jh)
         if (route_of[shape_of[jh]] == kRouteBluestein) jh_all.push_back(jh);
     rg->blue_count = (int)jh_all.size() - rg->blue_off;
     if (rg->blue_count > 0) {
-        // fields per CTA of the Bluestein launch: as many as fit (rows at
-        // the pitch of the plan's own half-length, which the kernels use)
-        const int Lrow = std::max(Lmax, p->fft.L);
-        int G = std::min(1, p->F);
-        while (G > 1 && bluestein_smem_bytes(Lrow, L2max, G, fp64) > 227 * 1024) --G;
+        // fields per CTA of the Bluestein launch: a power of two that leaves
+        // room for two CTAs per SM, or one field
+        int G = 16;
+        while (G > 1 && (G > p->F || bluestein_smem_bytes(L2max, G, fp64) > 112 * 1024)) G /= 2;
         rg->blue_G = G;
-        rg->blue_smem = bluestein_smem_bytes(Lrow, L2max, G, fp64);
+        rg->blue_smem = bluestein_smem_bytes(L2max, G, fp64);
         if (rg->blue_smem > 227 * 1024) {
             delete rg;
             set_error("rows of %d longitudes are too long for the Bluestein FFT", 2 * Lmax);

@@ -302,9 +302,13 @@ __global__ void cos_table_kernel(double* out, int n) {
 // wrapped around L2 (b_j = conj c_j for 0 <= j < L, b_{L2-j} = conj c_j for
 // 0 < j < L, zero between): D_k = (1/L2) (1 + 2 sum_{0<j<L} conj(c_j)
 // cos(2 pi j k / L2)), a direct FP64 sum with j k reduced mod L2 exactly.
+// Stored as the FFT kernel's last pass (radix R, span 1) reads it:
+// frequency k sits at the digit-reversed position b R + t, its D at
+// t (L2 / R) + b.
 template <typename V>
 __global__ void bluestein_dft_kernel(V* out, const double2* c, const double* costab, int L,
-                                     int L2) {
+                                     FftShape sh) {
+    const int L2 = sh.L;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= L2) return;
     double re = 1.0, im = 0.0;
@@ -319,7 +323,13 @@ __global__ void bluestein_dft_kernel(V* out, const double2* c, const double* cos
     V v;
     v.x = re / (double)L2;
     v.y = im / (double)L2;
-    out[k] = v;
+    int pos = 0, kk = k;
+    for (int q = 0; q < sh.npass; ++q) {
+        pos += (kk % sh.radix[q]) * sh.span[q];
+        kk /= sh.radix[q];
+    }
+    const int R = sh.radix[sh.npass - 1];
+    out[(pos % R) * (L2 / R) + pos / R] = v;
 }
 
 template <typename V>
@@ -356,11 +366,11 @@ cudaError_t build_bluestein_tables(int L, const FftShape& sh2, bool fp64, void* 
     if (fp64) {
         twiddle_kernel<double2><<<bL, threads, 0, s>>>((double2*)twpost, L, 2 * L);
         chirp_kernel<double2><<<bL, threads, 0, s>>>((double2*)chirp, c64, L);
-        bluestein_dft_kernel<double2><<<bL2, threads, 0, s>>>((double2*)dft, c64, costab, L, L2);
+        bluestein_dft_kernel<double2><<<bL2, threads, 0, s>>>((double2*)dft, c64, costab, L, sh2);
     } else {
         twiddle_kernel<float2><<<bL, threads, 0, s>>>((float2*)twpost, L, 2 * L);
         chirp_kernel<float2><<<bL, threads, 0, s>>>((float2*)chirp, c64, L);
-        bluestein_dft_kernel<float2><<<bL2, threads, 0, s>>>((float2*)dft, c64, costab, L, L2);
+        bluestein_dft_kernel<float2><<<bL2, threads, 0, s>>>((float2*)dft, c64, costab, L, sh2);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
