@@ -113,9 +113,9 @@ template <typename T> struct C2 {
     static __device__ __forceinline__ V mul_pi(V a) { return make(-a.y, a.x); }
 };
 
-// W_N^e = exp(-2 pi i e/N) for the composite register DFT sizes, written
-// once per device by fft_constants_init.
-constexpr int kComposite[] = {6, 9, 10, 12, 15, 16, 20, 24, 25, 30, 32, 40};
+// W_N^e = exp(-2 pi i e/N) for the composite register DFT sizes whose factors
+// are not coprime, written once per device by fft_constants_init.
+constexpr int kComposite[] = {9, 16, 25, 32};
 constexpr int tw_offset(int n) {
     int off = 0;
     for (int c : kComposite) {
@@ -264,18 +264,52 @@ struct DftComposite {
     }
 };
 
-template <typename T> struct Dft<T, 6> : DftComposite<T, 2, 3> {};
+// The same for coprime A and B by the Good-Thomas index maps: with
+// n = B n1 + A n2 (mod N), W_N^{n k} = W_A^{n1 k} W_B^{n2 k}, so
+//   X[k] = sum_n2 W_B^{n2 (k mod B)} sum_n1 W_A^{n1 (k mod A)} x[n]
+// needs no twiddles (a size 40 saves 28 complex products of 4 instructions
+// and their rounding); the maps only name registers.
+template <typename T, int A, int B>
+struct DftCoprime {
+    using V = typename Vec2<T>::type;
+    static constexpr int N = A * B;
+    static __device__ __forceinline__ constexpr int pos(int k) {
+        return (B * (k % A) + A * Dft<T, B>::pos(k % B)) % N;
+    }
+    static __device__ __forceinline__ void run(V* x) {
+#pragma unroll
+        for (int n2 = 0; n2 < B; ++n2) {
+            V t[A];
+#pragma unroll
+            for (int n1 = 0; n1 < A; ++n1) t[n1] = x[(B * n1 + A * n2) % N];
+            Dft<T, A>::run(t);
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) x[(B * k1 + A * n2) % N] = t[k1];
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            V t[B];
+#pragma unroll
+            for (int n2 = 0; n2 < B; ++n2) t[n2] = x[(B * k1 + A * n2) % N];
+            Dft<T, B>::run(t);
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) x[(B * k1 + A * k2) % N] = t[k2];
+        }
+    }
+};
+
+template <typename T> struct Dft<T, 6> : DftCoprime<T, 2, 3> {};
 template <typename T> struct Dft<T, 9> : DftComposite<T, 3, 3> {};
-template <typename T> struct Dft<T, 10> : DftComposite<T, 2, 5> {};
-template <typename T> struct Dft<T, 12> : DftComposite<T, 4, 3> {};
-template <typename T> struct Dft<T, 15> : DftComposite<T, 3, 5> {};
+template <typename T> struct Dft<T, 10> : DftCoprime<T, 2, 5> {};
+template <typename T> struct Dft<T, 12> : DftCoprime<T, 4, 3> {};
+template <typename T> struct Dft<T, 15> : DftCoprime<T, 3, 5> {};
 template <typename T> struct Dft<T, 16> : DftComposite<T, 4, 4> {};
-template <typename T> struct Dft<T, 20> : DftComposite<T, 4, 5> {};
-template <typename T> struct Dft<T, 24> : DftComposite<T, 8, 3> {};
+template <typename T> struct Dft<T, 20> : DftCoprime<T, 4, 5> {};
+template <typename T> struct Dft<T, 24> : DftCoprime<T, 8, 3> {};
 template <typename T> struct Dft<T, 25> : DftComposite<T, 5, 5> {};
-template <typename T> struct Dft<T, 30> : DftComposite<T, 5, 6> {};
+template <typename T> struct Dft<T, 30> : DftCoprime<T, 5, 6> {};
 template <typename T> struct Dft<T, 32> : DftComposite<T, 8, 4> {};
-template <typename T> struct Dft<T, 40> : DftComposite<T, 8, 5> {};
+template <typename T> struct Dft<T, 40> : DftCoprime<T, 8, 5> {};
 
 // f(integral_constant<int, r>) for a radix known at run time: every register
 // DFT size for FP32, the basic ones for FP64 (Bluestein rows).
