@@ -39,8 +39,8 @@
 // chosen at plan creation (fft_shape), the forward's first pass reading the
 // grid rows and the inverse's last pass writing them.  Passes of radices 8,
 // 4, 2, 3, 5 through shared memory took 1.2 to 1.8 times as long (forward /
-// inverse us for 64 fields: Tc479, L = 960 = 30 x 32, 369 / 444 -> 289 / 290;
-// T191, L = 384 92 / 97 -> 58 / 53; T119, L = 240 51 / 46 -> 30 / 29).
+// inverse us for 64 fields: T399, L = 800, 281 / 329 -> 207 / 207; T179, L = 360,
+// 81 / 82 -> 53 / 50; T119, L = 240, 51 / 46 -> 30 / 29).
 // Grouped launches branch per CTA to the body of their plan's length, and a
 // reduced grid launches the compile-time kernel once per row length it
 // contains, over a list of latitude pairs.

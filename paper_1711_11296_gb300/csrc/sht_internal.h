@@ -133,8 +133,8 @@ size_t bluestein_smem_bytes(int L2, int G, bool fp64);
 
 // Half-lengths with compile-time FFT kernels (the standard grids).
 inline bool fft_has_fixed_kernel(int L) {
-    return L == 64 || L == 128 || L == 256 || L == 320 || L == 512 || L == 640 || L == 1024 ||
-           L == 1280;
+    return L == 64 || L == 128 || L == 256 || L == 320 || L == 384 || L == 480 || L == 512 ||
+           L == 640 || L == 768 || L == 960 || L == 1024 || L == 1280;
 }
 
 // Shared memory per field of the FP64 FFT kernels beside the rows.
@@ -248,10 +248,10 @@ void ragged_free(RaggedGrid* rg);
 int inverse_scaled(sht_plan_s* p, const void* spec, const InvScale& sc, void* grid,
                    cudaStream_t s);
 
-// Register DFT sizes of the two-pass FP32 FFT (L = Q x 32).
+// Register DFT sizes Q of the two-pass FP32 FFT (L = Q x 32).
 __host__ __device__ constexpr bool fft_big_radix(int q) {
     return q == 2 || q == 4 || q == 8 || q == 10 || q == 16 || q == 20 || q == 32 ||
-           q == 40;
+           q == 40 || q == 12 || q == 15 || q == 24 || q == 30;
 }
 
 // Mixed-radix factorisation of the half-length FFT, shared by the plans,
