@@ -388,7 +388,7 @@ __device__ __forceinline__ void bfly_fixed(typename Vec2<T>::type* z, int base,
 // In-place mixed-radix DIF FFT over `nrows` padded rows (pitch LP), passes
 // p0 .. p1 - 1 of a shape known at run time.
 template <typename T>
-__device__ __noinline__ void passes_runtime(typename Vec2<T>::type* rows, int nrows, int LP,
+__device__ __forceinline__ void passes_runtime(typename Vec2<T>::type* rows, int nrows, int LP,
                                                const FftShape& sh, int p0, int p1,
                                                const typename Vec2<T>::type* twp) {
     for (int p = p0; p < p1; ++p) {

@@ -1,11 +1,12 @@
 // Grouped execution of several plans: one launch per kernel stage covers
 // every plan of the group (uneven truncations, ensemble members, levels),
-// so a whole batch costs four launches per transform pair and can be
-// captured in one CUDA graph.  The per-plan kernel bodies are the ones the
-// single-plan entry points use; the group kernels only map their block
-// index to (plan, tile) through per-plan argument blocks.  Legendre tiles
-// of all plans are sorted by their K-loop length, longest first, so the
-// uneven per-m row counts balance over the SMs.
+// so a whole batch costs a few launches per transform pair and can be
+// captured in one CUDA graph.  (FP64 contractions are launched per plan.)
+// The per-plan kernel bodies are the ones the single-plan entry points use;
+// the group kernels only map their block index to (plan, tile) through
+// per-plan argument blocks.  Legendre tiles of all plans are sorted by their
+// K-loop length, longest first, so the uneven per-m row counts balance over
+// the SMs.
 #include <algorithm>
 #include <mutex>
 #include <new>
@@ -16,11 +17,6 @@
 
 namespace sht {
 
-void build_legendre_tiles(int N, int Jh, int C, std::vector<int4>& fwd,
-                          std::vector<int4>& inv);
-cudaError_t launch_legendre_fp64_group(sht_plan_s* const* plans, int n, bool inverse,
-                                       const void* const* in, void* const* out,
-                                       const int4* tiles, int ntiles, cudaStream_t s);
 void split_group_tiles(sht_plan_s* const* plans, int n, bool inverse, std::vector<int4>& out);
 cudaError_t launch_split_group(sht_plan_s* const* plans, int n, bool inverse,
                                const void* const* in, void* const* out, const int4* tiles,
@@ -61,28 +57,19 @@ int fail(cudaError_t e, const char* what) {
     return SHT_ERR_CUDA;
 }
 
-// FP64 tiles of all plans; tile.y = parity + 2 * plan.  Forward tiles run
-// over the plan's Jh nodes, inverse tiles over the parity's row count.
-void fp64_group_tiles(sht_plan_s* const* plans, int n, bool inverse, std::vector<int4>& out) {
-    std::vector<std::pair<int, int4>> all;
+// FP64 contractions of all plans, a launch each: a plan with tensor-core tables
+// fills the GPU by itself, and the others are a few microseconds.
+cudaError_t launch_legendre_fp64_group(sht_plan_s* const* plans, int n, bool inverse,
+                                       const void* const* in, void* const* out,
+                                       cudaStream_t s) {
     for (int q = 0; q < n; ++q) {
-        const sht_plan_s* p = plans[q];
-        std::vector<int4> tf, ti;
-        build_legendre_tiles(p->N, p->Jh, 2 * p->F, tf, ti);
-        for (int4 t : inverse ? ti : tf) {
-            const int d = p->N - t.x - t.y;
-            const int R = d >= 0 ? d / 2 + 1 : 0;
-            const int cost = inverse ? R : p->Jh;
-            t.y += 2 * q;
-            all.push_back({cost, t});
-        }
+        const double* a = static_cast<const double*>(in[q]);
+        double* b = static_cast<double*>(out[q]);
+        const cudaError_t e = inverse ? launch_legendre_inv_fp64(plans[q], a, b, s)
+                                      : launch_legendre_fwd_fp64(plans[q], a, b, s);
+        if (e) return e;
     }
-    std::stable_sort(all.begin(), all.end(),
-                     [](const std::pair<int, int4>& a, const std::pair<int, int4>& b) {
-                         return a.first > b.first;
-                     });
-    out.clear();
-    for (auto& e : all) out.push_back(e.second);
+    return cudaSuccess;
 }
 
 struct DeviceGuard {
@@ -141,10 +128,7 @@ extern "C" int sht_group_create(const sht_plan_t* plans, int nplans, sht_group_t
     g->tile_width = split_tile_width(plans[0]);
     for (int q = 0; q < nplans; ++q) g->plans[q] = plans[q];
     std::vector<int4> tf, ti;
-    if (g->prec == SHT_FP64) {
-        fp64_group_tiles(g->plans, nplans, false, tf);
-        fp64_group_tiles(g->plans, nplans, true, ti);
-    } else {
+    if (g->prec != SHT_FP64) {
         split_group_tiles(g->plans, nplans, false, tf);
         split_group_tiles(g->plans, nplans, true, ti);
     }
@@ -242,8 +226,7 @@ extern "C" int sht_group_forward(sht_group_t g, const void* const* grids, void* 
     {
         ProfScope ps(g->plans[0], kStageLegFwd, s);
         if (g->prec == SHT_FP64)
-            e = launch_legendre_fp64_group(g->plans, g->n, false, works, specs,
-                                           g->d_tiles_fwd, g->ntiles_fwd, s);
+            e = launch_legendre_fp64_group(g->plans, g->n, false, works, specs, s);
         else
             e = launch_split_group(g->plans, g->n, false, works, specs, g->d_tiles_fwd,
                                    g->ntiles_fwd, s);
@@ -264,8 +247,7 @@ extern "C" int sht_group_inverse(sht_group_t g, const void* const* specs, void* 
     {
         ProfScope ps(g->plans[0], kStageLegInv, s);
         if (g->prec == SHT_FP64)
-            e = launch_legendre_fp64_group(g->plans, g->n, true, specs, works, g->d_tiles_inv,
-                                           g->ntiles_inv, s);
+            e = launch_legendre_fp64_group(g->plans, g->n, true, specs, works, s);
         else
             e = launch_split_group(g->plans, g->n, true, specs, works, g->d_tiles_inv,
                                    g->ntiles_inv, s);

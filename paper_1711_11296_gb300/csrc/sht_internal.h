@@ -323,9 +323,11 @@ cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,
 cudaError_t launch_legendre_inv_fp64(const sht_plan_s* p, const double* spec,
                                      double* work, cudaStream_t s);
 
+// Whether a plan's FP64 contractions are small enough for a thread per output.
+bool legendre_small(const sht_plan_s* p);
 // FP64 contractions on the tensor cores (sht_slice64.cu): plan tables (none
-// where the FP64 pipe is faster) and the launches launch_legendre_*_fp64
-// hand over to when the plan has them.
+// for small ones) and the launches launch_legendre_*_fp64 hand over to when
+// the plan has them.
 cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s);
 void slice64_destroy(sht_plan_s* p);
 cudaError_t launch_legendre_slice64(const sht_plan_s* p, bool inverse, const double* in,

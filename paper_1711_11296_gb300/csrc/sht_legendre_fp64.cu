@@ -11,10 +11,12 @@
 // the symmetric (q = 0) and antisymmetric (q = 1) halves that the inverse
 // FFT unfolds into both hemispheres.
 //
-// One CTA computes a 32 x 64 output tile with 256 threads (4 x 2 outputs
-// each) over K chunks of 16 staged in shared memory.  The tile list
-// {m, q, row0, col0} is built once per plan.  On GB300 the FP64 pipe, not
-// memory, bounds this kernel.
+// These kernels run on the FP64 pipe: small transforms (legendre_small) with a
+// thread per output, and those whose plan has no tensor-core tables
+// (sht_slice64.cu) in tiles: a CTA computes a 32 x 64 output tile with 256
+// threads (4 x 2 outputs each) over K chunks of 16 staged in shared memory,
+// from a tile list {m, q, row0, col0} built once per plan.  The FP64 pipe,
+// not memory, bounds both.
 #include "sht_internal.h"
 
 namespace sht {
@@ -154,70 +156,59 @@ __global__ void __launch_bounds__(NT) legendre_inv_fp64_kernel(
     legendre_inv_body(pnm, ldp, spec, work, tiles[blockIdx.x], N, Jh, C, jmin);
 }
 
-// Grouped launches: tile.y = parity + 2 * (plan index in the group).
-struct LegGroup {
-    int n;
-    const double* pnm[kMaxGroup];
-    const double* in[kMaxGroup];
-    double* out[kMaxGroup];
-    int ldp[kMaxGroup], N[kMaxGroup], Jh[kMaxGroup], C[kMaxGroup];
-    const int* jmin[kMaxGroup];
-};
-
-__global__ void __launch_bounds__(NT) legendre_fwd_fp64_group_kernel(
-    const __grid_constant__ LegGroup G, const int4* __restrict__ tiles) {
-    const int4 t = tiles[blockIdx.x];
-    const int p = t.y >> 1;
-    legendre_fwd_body(G.pnm[p], G.ldp[p], G.in[p], G.out[p], t, G.N[p], G.Jh[p], G.C[p],
-                      G.jmin[p]);
+// Small transforms (legendre_small): a thread per output, the same sums in the
+// same order.  A tile's CTA computes 2048 products per K step whatever
+// columns and rows there are (T31 x 1: 2 columns, at most 16 rows), and the
+// slices take two launches and whole 16-column MMAs; here a K step is one
+// product per output, bound by the FP64 pipe and, below it, by latency.
+__global__ void __launch_bounds__(128) legendre_small_fp64_kernel(
+    const double* __restrict__ pnm, int ldp, const double* __restrict__ in,
+    double* __restrict__ out, int N, int Jh, int C, const int* __restrict__ jmin, int inverse) {
+    const int m = blockIdx.x >> 1, q = blockIdx.x & 1;
+    const int R = parity_rows(N, m, q);
+    const size_t row0 = dcoef_offset(N, m) + q;
+    const int o = blockIdx.y * 128 + threadIdx.x;
+    const int row = o / C, c = o - row * C;
+    if (row >= (inverse ? Jh : R)) return;
+    const double* P = pnm + row0 * ldp;
+    const size_t wrow = (size_t)(2 * m + q) * Jh;
+    double acc = 0.0;
+    if (!inverse) {
+        const double* B = in + wrow * C + c;
+        const double* A = P + 2 * (size_t)row * ldp;
+#pragma unroll 8
+        for (int k = jmin ? (jmin[2 * m + q] / BK) * BK : 0; k < Jh; ++k)
+            acc = fma(__ldg(A + k), __ldg(B + (size_t)k * C), acc);
+        out[(row0 + 2 * (size_t)row) * C + c] = acc;
+    } else {
+        const double* B = in + row0 * C + c;
+        const int kend = (jmin && row / BM * BM + BM <= jmin[2 * m + q]) ? 0 : R;
+#pragma unroll 8
+        for (int k = 0; k < kend; ++k)
+            acc = fma(__ldg(P + 2 * (size_t)k * ldp + row), __ldg(B + 2 * (size_t)k * C), acc);
+        out[(wrow + row) * C + c] = acc;
+    }
 }
 
-__global__ void __launch_bounds__(NT) legendre_inv_fp64_group_kernel(
-    const __grid_constant__ LegGroup G, const int4* __restrict__ tiles) {
-    const int4 t = tiles[blockIdx.x];
-    const int p = t.y >> 1;
-    legendre_inv_body(G.pnm[p], G.ldp[p], G.in[p], G.out[p], t, G.N[p], G.Jh[p], G.C[p],
-                      G.jmin[p]);
+cudaError_t launch_small(const sht_plan_s* p, bool inverse, const double* in, double* out,
+                         cudaStream_t s) {
+    const int C = 2 * p->F, rows = inverse ? p->Jh : p->N / 2 + 1;
+    const dim3 grid(2 * (p->N + 1), (rows * C + 127) / 128);
+    legendre_small_fp64_kernel<<<grid, 128, 0, s>>>(p->d_pnm, p->ldp, in, out, p->N, p->Jh, C,
+                                                    p->d_jmin, inverse ? 1 : 0);
+    note_launch();
+    return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_legendre_fp64_group(sht_plan_s* const* plans, int n, bool inverse,
-                                       const void* const* in, void* const* out,
-                                       const int4* tiles, int ntiles, cudaStream_t s) {
-    // a plan with tensor-core tables fills the GPU by itself: per-plan launches
-    bool sliced = false;
-    for (int q = 0; q < n; ++q) sliced = sliced || plans[q]->slice;
-    if (sliced) {
-        for (int q = 0; q < n; ++q) {
-            const cudaError_t e =
-                inverse ? launch_legendre_inv_fp64(plans[q], static_cast<const double*>(in[q]),
-                                                   static_cast<double*>(out[q]), s)
-                        : launch_legendre_fwd_fp64(plans[q], static_cast<const double*>(in[q]),
-                                                   static_cast<double*>(out[q]), s);
-            if (e) return e;
-        }
-        return cudaSuccess;
-    }
-    LegGroup G;
-    G.n = n;
-    for (int q = 0; q < n; ++q) {
-        G.pnm[q] = plans[q]->d_pnm;
-        G.ldp[q] = plans[q]->ldp;
-        G.N[q] = plans[q]->N;
-        G.Jh[q] = plans[q]->Jh;
-        G.C[q] = 2 * plans[q]->F;
-        G.in[q] = static_cast<const double*>(in[q]);
-        G.out[q] = static_cast<double*>(out[q]);
-        G.jmin[q] = plans[q]->d_jmin;
-    }
-    if (ntiles == 0) return cudaSuccess;
-    if (inverse)
-        legendre_inv_fp64_group_kernel<<<ntiles, NT, 0, s>>>(G, tiles);
-    else
-        legendre_fwd_fp64_group_kernel<<<ntiles, NT, 0, s>>>(G, tiles);
-    note_launch();
-    return cudaGetLastError();
+// us of the forward + inverse contraction, slices -> a thread per output: T31 x
+// 10 44 -> 22, T63 x 20 51 -> 39, T95 x 16 74 -> 72, T127 x 4 63 -> 57, T159 x 4
+// 103 -> 93; beyond 3e7 flops T63 x 64 62 -> 78, T200 x 4 128 -> 145, except for
+// one field, whose 2 columns fill an eighth of an MMA: T319 x 1 290 -> 179,
+// T639 x 1 1311 -> 1133.  (The tiles: T31 x 1 45, here 18.)
+bool legendre_small(const sht_plan_s* p) {
+    return p->F == 1 || 4.0 * (double)p->ncoef * p->Jh * p->F <= 3e7;
 }
 
 // Tile lists (host): forward tiles cover the parity rows of each (m, q);
@@ -242,6 +233,7 @@ void build_legendre_tiles(int N, int Jh, int C, std::vector<int4>& fwd,
 cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,
                                      double* spec, cudaStream_t s) {
     if (p->slice) return launch_legendre_slice64(p, false, work, spec, s);
+    if (legendre_small(p)) return launch_small(p, false, work, spec, s);
     if (p->ntiles_fwd == 0) return cudaSuccess;
     legendre_fwd_fp64_kernel<<<p->ntiles_fwd, NT, 0, s>>>(
         p->d_pnm, p->ldp, work, spec, p->d_tiles_fwd, p->N, p->Jh, 2 * p->F, p->d_jmin);
@@ -252,6 +244,7 @@ cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,
 cudaError_t launch_legendre_inv_fp64(const sht_plan_s* p, const double* spec,
                                      double* work, cudaStream_t s) {
     if (p->slice) return launch_legendre_slice64(p, true, spec, work, s);
+    if (legendre_small(p)) return launch_small(p, true, spec, work, s);
     if (p->ntiles_inv == 0) return cudaSuccess;
     legendre_inv_fp64_kernel<<<p->ntiles_inv, NT, 0, s>>>(
         p->d_pnm, p->ldp, spec, work, p->d_tiles_inv, p->N, p->Jh, 2 * p->F, p->d_jmin);

@@ -693,19 +693,11 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
 
 }  // namespace
 
-// The tensor cores are the faster way from about 4e5 flops per transform
-// (us of the forward + inverse stages, FP64 pipe -> slices: T31 x 1 45 -> 34,
-// one launch more; T31 x 16 46 -> 43; T63 x 1 95 -> 34; T127 x 1 406 -> 58;
-// T639 x 256 238400 -> 13200).  Below, a transform is one small wave either
-// way and the single launch is kept.
-static bool slice64_wanted(const sht_plan_s* p) {
-    return 4.0 * (double)p->ncoef * p->Jh * p->F > 4e5 && p->Jh <= 4096;
-}
-
-// The slice tables of an FP64 plan; without the memory for them the plan
-// stays on the FP64 pipe.
+// The slice tables of an FP64 plan (none for small transforms, see
+// legendre_small); without the memory for them the plan stays on the FP64
+// pipe.
 cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
-    if (!slice64_wanted(p)) return cudaSuccess;
+    if (legendre_small(p) || p->Jh > 4096) return cudaSuccess;
     Slice64* sl = new (std::nothrow) Slice64();
     if (!sl) return cudaSuccess;
     p->slice = sl;
