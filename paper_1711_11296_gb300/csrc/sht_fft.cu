@@ -10,14 +10,15 @@ namespace {
 
 template <int LT>
 cudaError_t fwd_launch(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
-                       cudaStream_t s) {
-    if (!strided) return fft_launch(fft_forward_kernel<float, LT, false>, A, grid, smem, s);
+                       cudaStream_t s, bool beside) {
+    if (!strided) return fft_launch(fft_forward_kernel<float, LT, false>, A, grid, smem, s, beside);
     return fft_launch(fft_forward_kernel<float, LT, true>, A, grid, smem, s);
 }
 
 template <int LT>
-cudaError_t inv_launch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s) {
-    return fft_launch(fft_inverse_kernel<float, LT>, A, grid, smem, s);
+cudaError_t inv_launch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
+                       bool beside) {
+    return fft_launch(fft_inverse_kernel<float, LT>, A, grid, smem, s, beside);
 }
 
 // Dispatch on the half-length: the rows of cubic grids (I = 4 (N + 1)) at the
@@ -43,15 +44,16 @@ cudaError_t inv_launch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStre
     }
 
 cudaError_t fwd_dispatch(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
-                         cudaStream_t s) {
-#define SHT_FWD(LV) fwd_launch<LV>(A, strided, grid, smem, s)
-    SHT_FFT_DISPATCH(A.L, SHT_FWD, fft_any_forward(A, strided, grid, smem, s))
+                         cudaStream_t s, bool beside = false) {
+#define SHT_FWD(LV) fwd_launch<LV>(A, strided, grid, smem, s, beside)
+    SHT_FFT_DISPATCH(A.L, SHT_FWD, fft_any_forward(A, strided, grid, smem, s, beside))
 #undef SHT_FWD
 }
 
-cudaError_t inv_dispatch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s) {
-#define SHT_INV(LV) inv_launch<LV>(A, grid, smem, s)
-    SHT_FFT_DISPATCH(A.L, SHT_INV, fft_any_inverse(A, grid, smem, s))
+cudaError_t inv_dispatch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
+                         bool beside = false) {
+#define SHT_INV(LV) inv_launch<LV>(A, grid, smem, s, beside)
+    SHT_FFT_DISPATCH(A.L, SHT_INV, fft_any_inverse(A, grid, smem, s, beside))
 #undef SHT_INV
 }
 
@@ -146,24 +148,27 @@ void set_class(Args& A, const RaggedGrid* rg, const RShape& r, int off, size_t v
 }
 
 template <typename T>
-cudaError_t fwd_ragged_class(const FwdArgs<T>& A, dim3 g, size_t smem, cudaStream_t s) {
+cudaError_t fwd_ragged_class(const FwdArgs<T>& A, dim3 g, size_t smem, cudaStream_t s,
+                             bool beside) {
     if constexpr (sizeof(T) == 8)
-        return fx_forward(A, false, g, smem, s);
+        return fx_forward(A, false, g, smem, s, beside);
     else
-        return fwd_dispatch(A, false, g, smem, s);
+        return fwd_dispatch(A, false, g, smem, s, beside);
 }
 
 template <typename T>
-cudaError_t inv_ragged_class(const InvArgs<T>& A, dim3 g, size_t smem, cudaStream_t s) {
+cudaError_t inv_ragged_class(const InvArgs<T>& A, dim3 g, size_t smem, cudaStream_t s,
+                             bool beside) {
     if constexpr (sizeof(T) == 8)
-        return fx_inverse(A, g, smem, s);
+        return fx_inverse(A, g, smem, s, beside);
     else
-        return inv_dispatch(A, g, smem, s);
+        return inv_dispatch(A, g, smem, s, beside);
 }
 
 // Reduced grid: one launch of the compile-time kernel per length class that
 // has one, then one launch of the generic kernel (a shape per CTA) over the
-// remaining latitude pairs.
+// remaining latitude pairs, then one over the Bluestein rows, side by side
+// (a class may be one latitude pair: 8 CTAs of 8 us at octahedral T319 x 64).
 template <typename T>
 cudaError_t fwd_ragged_impl(const sht_plan_s* p, const void* grid, const FwdScale& sc,
                             void* work, cudaStream_t s) {
@@ -182,11 +187,13 @@ cudaError_t fwd_ragged_impl(const sht_plan_s* p, const void* grid, const FwdScal
         if (e) return e;
     }
     const unsigned nfg = (p->F + p->G - 1) / p->G;
+    bool beside = false;   // the launches after the first run beside it
     for (const auto& c : rg->classes) {
         FwdArgs<T> A = base;
         set_class(A, rg, rg->h_shapes[c.shape], c.off, vb);
         const cudaError_t e = fwd_ragged_class<T>(A, dim3(nfg, c.count),
-                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s);
+                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s, beside);
+        beside = true;
         if (e) return e;
     }
     RaggedFwd<T> R;
@@ -205,16 +212,17 @@ cudaError_t fwd_ragged_impl(const sht_plan_s* p, const void* grid, const FwdScal
         R.a.jh_list = rg->d_jh + rg->generic_off;
         const dim3 g(nfg, rg->generic_count);
         if constexpr (sizeof(T) == 8)
-            e = fx_forward_ragged(R, g, p->fft_smem, s);
+            e = fx_forward_ragged(R, g, p->fft_smem, s, beside);
         else
-            e = fft_any_forward_ragged(R, g, p->fft_smem, s);
+            e = fft_any_forward_ragged(R, g, p->fft_smem, s, beside);
         if (e) return e;
+        beside = true;
     }
     if (rg->blue_count > 0) {
         R.a.jh_list = rg->d_jh + rg->blue_off;
         R.a.G = rg->blue_G;
         const unsigned nfb = (p->F + rg->blue_G - 1) / rg->blue_G;
-        e = fft_bluestein_forward(R, dim3(nfb, rg->blue_count), rg->blue_smem, s);
+        e = fft_bluestein_forward(R, dim3(nfb, rg->blue_count), rg->blue_smem, s, beside);
         if (e) return e;
     }
     return cudaSuccess;
@@ -230,11 +238,13 @@ cudaError_t inv_ragged_impl(const sht_plan_s* p, const void* work, const InvScal
     base.rowoff = rg->d_rowoff;
     base.fstride = rg->npts;
     const unsigned nfg = (p->F + p->G - 1) / p->G;
+    bool beside = false;   // the launches after the first run beside it
     for (const auto& c : rg->classes) {
         InvArgs<T> A = base;
         set_class(A, rg, rg->h_shapes[c.shape], c.off, vb);
         const cudaError_t e = inv_ragged_class<T>(A, dim3(nfg, c.count),
-                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s);
+                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s, beside);
+        beside = true;
         if (e) return e;
     }
     RaggedInv<T> R;
@@ -253,16 +263,17 @@ cudaError_t inv_ragged_impl(const sht_plan_s* p, const void* work, const InvScal
         R.a.jh_list = rg->d_jh + rg->generic_off;
         const dim3 g(nfg, rg->generic_count);
         if constexpr (sizeof(T) == 8)
-            e = fx_inverse_ragged(R, g, p->fft_smem, s);
+            e = fx_inverse_ragged(R, g, p->fft_smem, s, beside);
         else
-            e = fft_any_inverse_ragged(R, g, p->fft_smem, s);
+            e = fft_any_inverse_ragged(R, g, p->fft_smem, s, beside);
         if (e) return e;
+        beside = true;
     }
     if (rg->blue_count > 0) {
         R.a.jh_list = rg->d_jh + rg->blue_off;
         R.a.G = rg->blue_G;
         const unsigned nfb = (p->F + rg->blue_G - 1) / rg->blue_G;
-        e = fft_bluestein_inverse(R, dim3(nfb, rg->blue_count), rg->blue_smem, s);
+        e = fft_bluestein_inverse(R, dim3(nfb, rg->blue_count), rg->blue_smem, s, beside);
         if (e) return e;
     }
     return cudaSuccess;

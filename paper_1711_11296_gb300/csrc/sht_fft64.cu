@@ -627,29 +627,37 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
 template <int LT, bool STRIDED>
 __global__ void __launch_bounds__(NT, 4)
     fx_forward_kernel(const __grid_constant__ FwdArgs<double> A) {
+    begin_beside();
     fwd_body<LT, STRIDED>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
+    end_beside();
 }
 
 template <int LT>
 __global__ void __launch_bounds__(NT, 4)
     fx_inverse_kernel(const __grid_constant__ InvArgs<double> A) {
+    begin_beside();
     inv_body<LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
+    end_beside();
 }
 
 __global__ void __launch_bounds__(NT, 4)
     fx_forward_ragged_kernel(const __grid_constant__ RaggedFwd<double> R) {
+    begin_beside();
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<double> A = R.a;
     apply_shape(A, R, jh);
     fwd_body<-1, false>(A, blockIdx.x, jh);
+    end_beside();
 }
 
 __global__ void __launch_bounds__(NT, 4)
     fx_inverse_ragged_kernel(const __grid_constant__ RaggedInv<double> R) {
+    begin_beside();
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<double> A = R.a;
     apply_shape(A, R, jh);
     inv_body<-1>(A, blockIdx.x, jh);
+    end_beside();
 }
 
 #define SHT_FX_BODY(L, CALL)               \
@@ -719,54 +727,41 @@ cudaError_t launch_fixed_twiddles(void* table, int n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-namespace {
-
-template <class K, class A>
-cudaError_t launch(K kernel, const A& args, dim3 grid, size_t smem, cudaStream_t s) {
-    cudaError_t e = ensure_smem((const void*)kernel, smem);
-    if (e) return e;
-    kernel<<<grid, NT, smem, s>>>(args);
-    note_launch();
-    return cudaGetLastError();
-}
-
-}  // namespace
-
 cudaError_t fx_forward(const FwdArgs<double>& A, bool strided, dim3 grid, size_t smem,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool beside) {
     cudaError_t e;
 #define SHT_CALL(LV)                                                             \
-    e = strided ? launch(fx_forward_kernel<LV, true>, A, grid, smem, s)          \
-                : launch(fx_forward_kernel<LV, false>, A, grid, smem, s)
+    e = strided ? fft_launch(fx_forward_kernel<LV, true>, A, grid, smem, s, beside)          \
+                : fft_launch(fx_forward_kernel<LV, false>, A, grid, smem, s, beside)
     SHT_FX_BODY(A.L, SHT_CALL)
 #undef SHT_CALL
     return e;
 }
 
-cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s) {
+cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s, bool beside) {
     if (A.mfactor1 != 1.0 && A.mfactor1 != 0.5) return cudaErrorInvalidValue;
     cudaError_t e;
-#define SHT_CALL(LV) e = launch(fx_inverse_kernel<LV>, A, grid, smem, s)
+#define SHT_CALL(LV) e = fft_launch(fx_inverse_kernel<LV>, A, grid, smem, s, beside)
     SHT_FX_BODY(A.L, SHT_CALL)
 #undef SHT_CALL
     return e;
 }
 
-cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s) {
-    return launch(fx_forward_ragged_kernel, R, grid, smem, s);
+cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s, bool beside) {
+    return fft_launch(fx_forward_ragged_kernel, R, grid, smem, s, beside);
 }
 
-cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s) {
+cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s, bool beside) {
     if (R.a.mfactor1 != 1.0 && R.a.mfactor1 != 0.5) return cudaErrorInvalidValue;
-    return launch(fx_inverse_ragged_kernel, R, grid, smem, s);
+    return fft_launch(fx_inverse_ragged_kernel, R, grid, smem, s, beside);
 }
 
 cudaError_t fx_forward_group(const FwdGroup<double>& G, int ctas, size_t smem, cudaStream_t s) {
-    return launch(fx_forward_group_kernel, G, dim3(ctas), smem, s);
+    return fft_launch(fx_forward_group_kernel, G, dim3(ctas), smem, s);
 }
 
 cudaError_t fx_inverse_group(const InvGroup<double>& G, int ctas, size_t smem, cudaStream_t s) {
-    return launch(fx_inverse_group_kernel, G, dim3(ctas), smem, s);
+    return fft_launch(fx_inverse_group_kernel, G, dim3(ctas), smem, s);
 }
 
 }  // namespace sht

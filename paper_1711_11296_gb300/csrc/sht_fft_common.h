@@ -126,6 +126,40 @@ __device__ __forceinline__ int row_pitch(int n) {
     return n + (n >> PadShift<T>::value) + 1;
 }
 
+// The launches of one reduced-grid FFT (a class per row length, the run-time
+// shapes, Bluestein rows) work on different rows and may run side by side:
+// each but the first is launched as a programmatic dependent of the one
+// before, which lets it start once that one's CTAs have. Every kernel waits
+// for its predecessor only before it ends, so that what follows the last of
+// them in the stream follows all of them.
+__device__ __forceinline__ void begin_beside() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void end_beside() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// One FFT launch; beside: as a programmatic dependent (above).
+template <class... Params, class Args>
+cudaError_t fft_launch(void (*kernel)(Params...), const Args& args, dim3 grid, size_t smem,
+                       cudaStream_t s, bool beside = false) {
+    cudaError_t e = ensure_smem((const void*)kernel, smem);
+    if (e) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kFftThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = beside ? 1 : 0;
+    e = cudaLaunchKernelEx(&cfg, kernel, args);
+    note_launch();
+    return e ? e : cudaGetLastError();
+}
+
 // Iterates idx = tid, tid + kFftThreads, ... as (major, minor) = (idx / d, idx % d)
 // without dividing inside the loop.
 struct Walk2 {
@@ -207,21 +241,29 @@ __device__ __forceinline__ void apply_shape(Args& A, const R& Rg, int jh) {
 // their constant twiddles to the current device.
 cudaError_t fft_any_init();
 cudaError_t fft_any_forward(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
-                            cudaStream_t s);
-cudaError_t fft_any_inverse(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s);
+                            cudaStream_t s,
+    bool beside = false);
+cudaError_t fft_any_inverse(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_any_forward_ragged(const RaggedFwd<float>& R, dim3 grid, size_t smem,
-                                   cudaStream_t s);
+                                   cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_any_inverse_ragged(const RaggedInv<float>& R, dim3 grid, size_t smem,
-                                   cudaStream_t s);
+                                   cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_bluestein_init();
 cudaError_t fft_bluestein_forward(const RaggedFwd<float>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s);
+                                  cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_bluestein_forward(const RaggedFwd<double>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s);
+                                  cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_bluestein_inverse(const RaggedInv<float>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s);
+                                  cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_bluestein_inverse(const RaggedInv<double>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s);
+                                  cudaStream_t s,
+    bool beside = false);
 cudaError_t fft_group_init();
 cudaError_t fft_group_forward(const FwdGroup<float>& G, int ctas, size_t smem, cudaStream_t s);
 cudaError_t fft_group_inverse(const InvGroup<float>& G, int ctas, size_t smem, cudaStream_t s);
@@ -229,10 +271,14 @@ cudaError_t fft_group_inverse(const InvGroup<float>& G, int ctas, size_t smem, c
 // Fixed-point FFT launches of the FP64 path (sht_fft64.cu); the arguments'
 // twiddle tables are the fixed-point ones (launch_fixed_twiddles).
 cudaError_t fx_forward(const FwdArgs<double>& A, bool strided, dim3 grid, size_t smem,
-                       cudaStream_t s);
-cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s);
-cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s);
-cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s);
+                       cudaStream_t s,
+    bool beside = false);
+cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s,
+    bool beside = false);
+cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s,
+    bool beside = false);
+cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s,
+    bool beside = false);
 cudaError_t fx_forward_group(const FwdGroup<double>& G, int ctas, size_t smem, cudaStream_t s);
 cudaError_t fx_inverse_group(const InvGroup<double>& G, int ctas, size_t smem, cudaStream_t s);
 

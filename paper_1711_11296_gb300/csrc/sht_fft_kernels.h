@@ -877,7 +877,9 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
 template <typename T, int LT, bool STRIDED>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_forward_kernel(const __grid_constant__ FwdArgs<T> A) {
+    begin_beside();
     fwd_body<T, LT, STRIDED>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
+    end_beside();
 }
 
 template <typename T, int LT>
@@ -1204,7 +1206,9 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
 template <typename T, int LT>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_inverse_kernel(const __grid_constant__ InvArgs<T> A) {
+    begin_beside();
     inv_body<T, LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
+    end_beside();
 }
 
 template <typename T>
@@ -1255,38 +1259,46 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_forward_ragged_kernel(const __grid_constant__ RaggedFwd<T> R) {
+    begin_beside();
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<T> A = R.a;
     apply_shape(A, R, jh);
     fwd_body<T, -1, false>(A, blockIdx.x, jh);
+    end_beside();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_inverse_ragged_kernel(const __grid_constant__ RaggedInv<T> R) {
+    begin_beside();
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<T> A = R.a;
     apply_shape(A, R, jh);
     inv_body<T, -1>(A, blockIdx.x, jh);
+    end_beside();
 }
 
 // Rows whose half-length has a prime factor above 5: Bluestein's method.
 template <typename T>
 __global__ void __launch_bounds__(NT, 2)
     fft_forward_bluestein_kernel(const __grid_constant__ RaggedFwd<T> R) {
+    begin_beside();
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<T> A = R.a;
     apply_shape(A, R, jh);
     fwd_body<T, -2, false>(A, blockIdx.x, jh);
+    end_beside();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(NT, 2)
     fft_inverse_bluestein_kernel(const __grid_constant__ RaggedInv<T> R) {
+    begin_beside();
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<T> A = R.a;
     apply_shape(A, R, jh);
     inv_body<T, -2>(A, blockIdx.x, jh);
+    end_beside();
 }
 
 // c_twf of this translation unit on the current device.
@@ -1300,15 +1312,6 @@ cudaError_t upload_twiddles() {
             hf[tw_offset(n) + k] = make_float2((float)c, (float)sn);
         }
     return cudaMemcpyToSymbol(c_twf, hf, sizeof(hf));
-}
-
-template <class K, class A>
-cudaError_t fft_launch(K kernel, const A& args, dim3 grid, size_t smem, cudaStream_t s) {
-    const cudaError_t e = ensure_smem((const void*)kernel, smem);
-    if (e) return e;
-    kernel<<<grid, NT, smem, s>>>(args);
-    note_launch();
-    return cudaGetLastError();
 }
 
 }  // namespace

@@ -79,3 +79,29 @@ def _big_prime(n):
         while n % q == 0:
             n //= q
     return n > 1
+
+
+def test_reduced_grid_captured_in_a_graph(sht):
+    # the side-by-side launches of a reduced grid's FFTs (classes, run-time
+    # shapes, Bluestein rows) keep their order when captured and replayed
+    F = 3
+    pts = [2 * L for L in (15, 31, 64, 64, 90, 96, 101, 128, 128, 128, 133, 256, 256, 320)]
+    pts = pts + pts[-2::-1]
+    p = sht.Plan(N, J, max(pts), F, "bf16x3", grid="reduced", lat_points=pts)
+    a = torch.from_numpy(W.random_spectrum(N, F, "flat", seed=2800).astype(np.complex64)).cuda()
+    grid, spec = p.empty_grid(), p.empty_spec()
+    p.inverse(a, out=grid)
+    p.forward(grid, out=spec)
+    ref_grid, ref_spec = grid.clone(), spec.clone()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.inverse(a, out=grid)
+        p.forward(grid, out=spec)
+    for _ in range(20):
+        grid.zero_()
+        spec.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(grid, ref_grid) and torch.equal(spec, ref_spec)
+    p.status()
