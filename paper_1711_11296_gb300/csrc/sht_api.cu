@@ -214,7 +214,7 @@ extern "C" int sht_plan_create_grid(int N, int J, int I, int nfields, int precis
     p->fft = shape;
     const bool fp64 = precision == SHT_FP64;
     const size_t vbytes = fp64 ? sizeof(double2) : sizeof(float2);
-    p->G = fft_default_fields(I, p->Jh, nfields, fp64);
+    p->G = fft_default_fields(I, p->Jh, nfields, fp64, fft_plan_ctas(fp64));
     p->fft_threads = 256;
     p->fft_smem = fft_smem_bytes(I, p->G, fp64);
     if (p->G == 0) {

@@ -279,6 +279,19 @@ cudaError_t inv_ragged_impl(const sht_plan_s* p, const void* work, const InvScal
     return cudaSuccess;
 }
 
+// Fields per CTA of plan q in a grouped launch: its own tuning, else the default
+// for the latitudes of all plans together, with half the CTAs (the plans'
+// uneven rows fill the gaps: T7 .. T63 x 7 17.2 us with the 124 CTAs of whole
+// field groups, 21.0 with 496).
+int group_fields(sht_plan_s* const* plans, int n, int q) {
+    const sht_plan_s* p = plans[q];
+    if (p->tuned) return p->G;
+    int pairs = 0;
+    for (int i = 0; i < n; ++i) pairs += plans[i]->Jh;
+    const bool fp64 = p->prec == SHT_FP64;
+    return fft_default_fields(p->I, pairs, p->F, fp64, fft_plan_ctas(fp64) / 2);
+}
+
 template <typename T>
 cudaError_t fwd_group_impl(sht_plan_s* const* plans, int n, const void* const* grids,
                            cudaStream_t s) {
@@ -300,9 +313,10 @@ cudaError_t fwd_group_impl(sht_plan_s* const* plans, int n, const void* const* g
                 cudaMemsetAsync(p->d_colmax, 0, 2 * (size_t)p->F * sizeof(unsigned), s);
             if (e) return e;
         }
-        G.nfg[q] = (p->F + p->G - 1) / p->G;
+        const int g = G.a[q].G = group_fields(plans, n, q);
+        G.nfg[q] = (p->F + g - 1) / g;
         G.cta_start[q + 1] = G.cta_start[q] + G.nfg[q] * p->Jh;
-        if (p->fft_smem > smem) smem = p->fft_smem;
+        smem = std::max(smem, fft_smem_bytes(p->I, g, sizeof(T) == 8));
     }
     if constexpr (sizeof(T) == 8)
         return fx_forward_group(G, G.cta_start[n], smem, s);
@@ -321,9 +335,10 @@ cudaError_t inv_group_impl(sht_plan_s* const* plans, int n, void* const* grids,
         const sht_plan_s* p = plans[q];
         const InvScale sc{nullptr, 1.0};
         G.a[q] = make_inv_args<T>(p, p->d_work, sc, grids[q]);
-        G.nfg[q] = (p->F + p->G - 1) / p->G;
+        const int g = G.a[q].G = group_fields(plans, n, q);
+        G.nfg[q] = (p->F + g - 1) / g;
         G.cta_start[q + 1] = G.cta_start[q] + G.nfg[q] * p->Jh;
-        if (p->fft_smem > smem) smem = p->fft_smem;
+        smem = std::max(smem, fft_smem_bytes(p->I, g, sizeof(T) == 8));
     }
     if constexpr (sizeof(T) == 8)
         return fx_inverse_group(G, G.cta_start[n], smem, s);
@@ -448,9 +463,8 @@ size_t fft_smem_bytes(int I, int G, bool fp64) {
 // fields 369 / 449).  Small grids (T31 x 32 bf16x3): 16 fields, 66 CTAs
 // 10.0 / 11.4, 4 fields, 264 CTAs 8.4 / 8.0; FP64 T63 x 16: 8 fields, 130
 // CTAs 18.0 / 22.4, 2 fields, 520 CTAs 15.1 / 14.2.
-int fft_default_fields(int I, int Jh, int F, bool fp64) {
+int fft_default_fields(int I, int Jh, int F, bool fp64, int ctas) {
     const size_t budget = (fp64 ? 55 : 112) * 1024;
-    const long ctas = fp64 ? 512 : 256;
     int g = 16;
     while (g > 1 && (g > F || fft_smem_bytes(I, g, fp64) > budget ||
                      (long)Jh * ((F + g - 1) / g) < ctas))

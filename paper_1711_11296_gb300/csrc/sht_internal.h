@@ -165,6 +165,7 @@ struct sht_plan_s {
     int ldp;         // leading dimension of the P~ table (>= Jh)
     int grid;        // latitude grid: SHT_GRID_CC (Sec. 3) or SHT_GRID_FEJER1 (Sec. 3.3)
     int G;           // fields per FFT CTA
+    bool tuned;      // G was set (sht_plan_set_tuning, sht_plan_autotune)
     int fft_threads;
     size_t fft_smem;
     sht::FftShape fft;
@@ -314,8 +315,11 @@ cudaError_t launch_fft_forward_group(sht_plan_s* const* plans, int n,
 cudaError_t launch_fft_inverse_group(sht_plan_s* const* plans, int n,
                                      void* const* grids, cudaStream_t s);
 size_t fft_smem_bytes(int I, int G, bool fp64);
-// Fields per FFT CTA of a plan before any tuning (0: the rows do not fit).
-int fft_default_fields(int I, int Jh, int F, bool fp64);
+// Fields per FFT CTA before any tuning, for a launch over Jh latitude pairs
+// that should have at least so many CTAs (0: the rows do not fit).
+int fft_default_fields(int I, int Jh, int F, bool fp64, int ctas);
+// CTAs that a plan's own FFT launch should have.
+inline int fft_plan_ctas(bool fp64) { return fp64 ? 512 : 256; }
 
 // FP64 Legendre launches
 cudaError_t launch_legendre_fwd_fp64(const sht_plan_s* p, const double* work,

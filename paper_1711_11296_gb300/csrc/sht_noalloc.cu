@@ -174,7 +174,7 @@ extern "C" int sht_forward_noalloc(int N, int J, int I, int nfields,
     t.ncoef = (size_t)(N + 1) * (N + 2) / 2;
     t.ldp = (t.Jh + 7) / 8 * 8;
     t.fft = shape;
-    t.G = fft_default_fields(I, t.Jh, nfields, true);
+    t.G = fft_default_fields(I, t.Jh, nfields, true, fft_plan_ctas(true));
     t.fft_threads = 256;
     t.fft_smem = fft_smem_bytes(I, t.G, true);
     if (t.G == 0) {

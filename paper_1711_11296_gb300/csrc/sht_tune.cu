@@ -52,6 +52,7 @@ int apply_fields_per_cta(sht_plan_s* p, int G) {
         return SHT_ERR_ARG;
     }
     p->G = G;
+    p->tuned = true;
     p->fft_smem = smem;
     return SHT_OK;
 }
