@@ -10,15 +10,15 @@ namespace {
 
 template <int LT>
 cudaError_t fwd_launch(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
-                       cudaStream_t s, bool beside) {
-    if (!strided) return fft_launch(fft_forward_kernel<float, LT, false>, A, grid, smem, s, beside);
-    return fft_launch(fft_forward_kernel<float, LT, true>, A, grid, smem, s);
+                       cudaStream_t s, Follow follow) {
+    if (!strided) return fft_launch(fft_forward_kernel<float, LT, false>, A, grid, smem, s, follow);
+    return fft_launch(fft_forward_kernel<float, LT, true>, A, grid, smem, s, follow);
 }
 
 template <int LT>
 cudaError_t inv_launch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
-                       bool beside) {
-    return fft_launch(fft_inverse_kernel<float, LT>, A, grid, smem, s, beside);
+                       Follow follow) {
+    return fft_launch(fft_inverse_kernel<float, LT>, A, grid, smem, s, follow);
 }
 
 // Dispatch on the half-length: the rows of cubic grids (I = 4 (N + 1)) at the
@@ -44,16 +44,16 @@ cudaError_t inv_launch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStre
     }
 
 cudaError_t fwd_dispatch(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
-                         cudaStream_t s, bool beside = false) {
-#define SHT_FWD(LV) fwd_launch<LV>(A, strided, grid, smem, s, beside)
-    SHT_FFT_DISPATCH(A.L, SHT_FWD, fft_any_forward(A, strided, grid, smem, s, beside))
+                         cudaStream_t s, Follow follow) {
+#define SHT_FWD(LV) fwd_launch<LV>(A, strided, grid, smem, s, follow)
+    SHT_FFT_DISPATCH(A.L, SHT_FWD, fft_any_forward(A, strided, grid, smem, s, follow))
 #undef SHT_FWD
 }
 
 cudaError_t inv_dispatch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
-                         bool beside = false) {
-#define SHT_INV(LV) inv_launch<LV>(A, grid, smem, s, beside)
-    SHT_FFT_DISPATCH(A.L, SHT_INV, fft_any_inverse(A, grid, smem, s, beside))
+                         Follow follow) {
+#define SHT_INV(LV) inv_launch<LV>(A, grid, smem, s, follow)
+    SHT_FFT_DISPATCH(A.L, SHT_INV, fft_any_inverse(A, grid, smem, s, follow))
 #undef SHT_INV
 }
 
@@ -92,9 +92,9 @@ cudaError_t fwd_impl(const sht_plan_s* p, const void* grid, const RowSource& src
     const dim3 g((p->F + p->G - 1) / p->G, p->Jh);
     const bool strided = src.elem_stride != 1;
     if constexpr (sizeof(T) == 8)
-        return fx_forward(A, strided, g, p->fft_smem, s);
+        return fx_forward(A, strided, g, p->fft_smem, s, kWait);
     else
-        return fwd_dispatch(A, strided, g, p->fft_smem, s);
+        return fwd_dispatch(A, strided, g, p->fft_smem, s, A.colmax ? kPlain : kWait);
 }
 
 template <typename T>
@@ -128,9 +128,9 @@ cudaError_t inv_impl(const sht_plan_s* p, const void* work, const InvScale& sc,
     const InvArgs<T> A = make_inv_args<T>(p, work, sc, grid);
     const dim3 g((p->F + p->G - 1) / p->G, p->Jh);
     if constexpr (sizeof(T) == 8)
-        return fx_inverse(A, g, p->fft_smem, s);
+        return fx_inverse(A, g, p->fft_smem, s, kWait);
     else
-        return inv_dispatch(A, g, p->fft_smem, s);
+        return inv_dispatch(A, g, p->fft_smem, s, kWait);
 }
 
 // Arguments of one length class of a reduced grid: that shape's tables and
@@ -149,20 +149,20 @@ void set_class(Args& A, const RaggedGrid* rg, const RShape& r, int off, size_t v
 
 template <typename T>
 cudaError_t fwd_ragged_class(const FwdArgs<T>& A, dim3 g, size_t smem, cudaStream_t s,
-                             bool beside) {
+                             Follow follow) {
     if constexpr (sizeof(T) == 8)
-        return fx_forward(A, false, g, smem, s, beside);
+        return fx_forward(A, false, g, smem, s, follow);
     else
-        return fwd_dispatch(A, false, g, smem, s, beside);
+        return fwd_dispatch(A, false, g, smem, s, follow);
 }
 
 template <typename T>
 cudaError_t inv_ragged_class(const InvArgs<T>& A, dim3 g, size_t smem, cudaStream_t s,
-                             bool beside) {
+                             Follow follow) {
     if constexpr (sizeof(T) == 8)
-        return fx_inverse(A, g, smem, s, beside);
+        return fx_inverse(A, g, smem, s, follow);
     else
-        return inv_dispatch(A, g, smem, s, beside);
+        return inv_dispatch(A, g, smem, s, follow);
 }
 
 // Reduced grid: one launch of the compile-time kernel per length class that
@@ -187,13 +187,13 @@ cudaError_t fwd_ragged_impl(const sht_plan_s* p, const void* grid, const FwdScal
         if (e) return e;
     }
     const unsigned nfg = (p->F + p->G - 1) / p->G;
-    bool beside = false;   // the launches after the first run beside it
+    Follow follow = kPlain;   // the launches after the first run beside it
     for (const auto& c : rg->classes) {
         FwdArgs<T> A = base;
         set_class(A, rg, rg->h_shapes[c.shape], c.off, vb);
         const cudaError_t e = fwd_ragged_class<T>(A, dim3(nfg, c.count),
-                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s, beside);
-        beside = true;
+                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s, follow);
+        follow = kBeside;
         if (e) return e;
     }
     RaggedFwd<T> R;
@@ -212,17 +212,17 @@ cudaError_t fwd_ragged_impl(const sht_plan_s* p, const void* grid, const FwdScal
         R.a.jh_list = rg->d_jh + rg->generic_off;
         const dim3 g(nfg, rg->generic_count);
         if constexpr (sizeof(T) == 8)
-            e = fx_forward_ragged(R, g, p->fft_smem, s, beside);
+            e = fx_forward_ragged(R, g, p->fft_smem, s, follow);
         else
-            e = fft_any_forward_ragged(R, g, p->fft_smem, s, beside);
+            e = fft_any_forward_ragged(R, g, p->fft_smem, s, follow);
         if (e) return e;
-        beside = true;
+        follow = kBeside;
     }
     if (rg->blue_count > 0) {
         R.a.jh_list = rg->d_jh + rg->blue_off;
         R.a.G = rg->blue_G;
         const unsigned nfb = (p->F + rg->blue_G - 1) / rg->blue_G;
-        e = fft_bluestein_forward(R, dim3(nfb, rg->blue_count), rg->blue_smem, s, beside);
+        e = fft_bluestein_forward(R, dim3(nfb, rg->blue_count), rg->blue_smem, s, follow);
         if (e) return e;
     }
     return cudaSuccess;
@@ -238,13 +238,13 @@ cudaError_t inv_ragged_impl(const sht_plan_s* p, const void* work, const InvScal
     base.rowoff = rg->d_rowoff;
     base.fstride = rg->npts;
     const unsigned nfg = (p->F + p->G - 1) / p->G;
-    bool beside = false;   // the launches after the first run beside it
+    Follow follow = kPlain;   // the launches after the first run beside it
     for (const auto& c : rg->classes) {
         InvArgs<T> A = base;
         set_class(A, rg, rg->h_shapes[c.shape], c.off, vb);
         const cudaError_t e = inv_ragged_class<T>(A, dim3(nfg, c.count),
-                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s, beside);
-        beside = true;
+                                                  fft_smem_bytes(2 * A.L, p->G, vb == 16), s, follow);
+        follow = kBeside;
         if (e) return e;
     }
     RaggedInv<T> R;
@@ -263,17 +263,17 @@ cudaError_t inv_ragged_impl(const sht_plan_s* p, const void* work, const InvScal
         R.a.jh_list = rg->d_jh + rg->generic_off;
         const dim3 g(nfg, rg->generic_count);
         if constexpr (sizeof(T) == 8)
-            e = fx_inverse_ragged(R, g, p->fft_smem, s, beside);
+            e = fx_inverse_ragged(R, g, p->fft_smem, s, follow);
         else
-            e = fft_any_inverse_ragged(R, g, p->fft_smem, s, beside);
+            e = fft_any_inverse_ragged(R, g, p->fft_smem, s, follow);
         if (e) return e;
-        beside = true;
+        follow = kBeside;
     }
     if (rg->blue_count > 0) {
         R.a.jh_list = rg->d_jh + rg->blue_off;
         R.a.G = rg->blue_G;
         const unsigned nfb = (p->F + rg->blue_G - 1) / rg->blue_G;
-        e = fft_bluestein_inverse(R, dim3(nfb, rg->blue_count), rg->blue_smem, s, beside);
+        e = fft_bluestein_inverse(R, dim3(nfb, rg->blue_count), rg->blue_smem, s, follow);
         if (e) return e;
     }
     return cudaSuccess;
@@ -319,9 +319,9 @@ cudaError_t fwd_group_impl(sht_plan_s* const* plans, int n, const void* const* g
         smem = std::max(smem, fft_smem_bytes(p->I, g, sizeof(T) == 8));
     }
     if constexpr (sizeof(T) == 8)
-        return fx_forward_group(G, G.cta_start[n], smem, s);
+        return fx_forward_group(G, G.cta_start[n], smem, s, kWait);
     else
-        return fft_group_forward(G, G.cta_start[n], smem, s);
+        return fft_group_forward(G, G.cta_start[n], smem, s, plans[0]->d_colmax ? kPlain : kWait);
 }
 
 template <typename T>
@@ -341,9 +341,9 @@ cudaError_t inv_group_impl(sht_plan_s* const* plans, int n, void* const* grids,
         smem = std::max(smem, fft_smem_bytes(p->I, g, sizeof(T) == 8));
     }
     if constexpr (sizeof(T) == 8)
-        return fx_inverse_group(G, G.cta_start[n], smem, s);
+        return fx_inverse_group(G, G.cta_start[n], smem, s, kWait);
     else
-        return fft_group_inverse(G, G.cta_start[n], smem, s);
+        return fft_group_inverse(G, G.cta_start[n], smem, s, kWait);
 }
 
 }  // namespace

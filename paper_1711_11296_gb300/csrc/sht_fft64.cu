@@ -627,37 +627,37 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
 template <int LT, bool STRIDED>
 __global__ void __launch_bounds__(NT, 4)
     fx_forward_kernel(const __grid_constant__ FwdArgs<double> A) {
-    begin_beside();
+    begin_fft(A.follow);
     fwd_body<LT, STRIDED>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
-    end_beside();
+    end_fft();
 }
 
 template <int LT>
 __global__ void __launch_bounds__(NT, 4)
     fx_inverse_kernel(const __grid_constant__ InvArgs<double> A) {
-    begin_beside();
+    begin_fft(A.follow);
     inv_body<LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
-    end_beside();
+    end_fft();
 }
 
 __global__ void __launch_bounds__(NT, 4)
     fx_forward_ragged_kernel(const __grid_constant__ RaggedFwd<double> R) {
-    begin_beside();
+    begin_fft(R.follow);
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<double> A = R.a;
     apply_shape(A, R, jh);
     fwd_body<-1, false>(A, blockIdx.x, jh);
-    end_beside();
+    end_fft();
 }
 
 __global__ void __launch_bounds__(NT, 4)
     fx_inverse_ragged_kernel(const __grid_constant__ RaggedInv<double> R) {
-    begin_beside();
+    begin_fft(R.follow);
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<double> A = R.a;
     apply_shape(A, R, jh);
     inv_body<-1>(A, blockIdx.x, jh);
-    end_beside();
+    end_fft();
 }
 
 #define SHT_FX_BODY(L, CALL)               \
@@ -676,6 +676,7 @@ __global__ void __launch_bounds__(NT, 4)
 // the plan's half-length picks its compile-time body (one branch per CTA)
 __global__ void __launch_bounds__(NT, 4)
     fx_forward_group_kernel(const __grid_constant__ FwdGroup<double> G) {
+    begin_fft(G.follow);
     const int b = blockIdx.x;
     int p = 0;
     while (p + 1 < G.n && b >= G.cta_start[p + 1]) ++p;
@@ -689,6 +690,7 @@ __global__ void __launch_bounds__(NT, 4)
 
 __global__ void __launch_bounds__(NT, 4)
     fx_inverse_group_kernel(const __grid_constant__ InvGroup<double> G) {
+    begin_fft(G.follow);
     const int b = blockIdx.x;
     int p = 0;
     while (p + 1 < G.n && b >= G.cta_start[p + 1]) ++p;
@@ -728,40 +730,42 @@ cudaError_t launch_fixed_twiddles(void* table, int n, cudaStream_t s) {
 }
 
 cudaError_t fx_forward(const FwdArgs<double>& A, bool strided, dim3 grid, size_t smem,
-                       cudaStream_t s, bool beside) {
+                       cudaStream_t s, Follow follow) {
     cudaError_t e;
 #define SHT_CALL(LV)                                                             \
-    e = strided ? fft_launch(fx_forward_kernel<LV, true>, A, grid, smem, s, beside)          \
-                : fft_launch(fx_forward_kernel<LV, false>, A, grid, smem, s, beside)
+    e = strided ? fft_launch(fx_forward_kernel<LV, true>, A, grid, smem, s, follow)          \
+                : fft_launch(fx_forward_kernel<LV, false>, A, grid, smem, s, follow)
     SHT_FX_BODY(A.L, SHT_CALL)
 #undef SHT_CALL
     return e;
 }
 
-cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s, bool beside) {
+cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s, Follow follow) {
     if (A.mfactor1 != 1.0 && A.mfactor1 != 0.5) return cudaErrorInvalidValue;
     cudaError_t e;
-#define SHT_CALL(LV) e = fft_launch(fx_inverse_kernel<LV>, A, grid, smem, s, beside)
+#define SHT_CALL(LV) e = fft_launch(fx_inverse_kernel<LV>, A, grid, smem, s, follow)
     SHT_FX_BODY(A.L, SHT_CALL)
 #undef SHT_CALL
     return e;
 }
 
-cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s, bool beside) {
-    return fft_launch(fx_forward_ragged_kernel, R, grid, smem, s, beside);
+cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s, Follow follow) {
+    return fft_launch(fx_forward_ragged_kernel, R, grid, smem, s, follow);
 }
 
-cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s, bool beside) {
+cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s, Follow follow) {
     if (R.a.mfactor1 != 1.0 && R.a.mfactor1 != 0.5) return cudaErrorInvalidValue;
-    return fft_launch(fx_inverse_ragged_kernel, R, grid, smem, s, beside);
+    return fft_launch(fx_inverse_ragged_kernel, R, grid, smem, s, follow);
 }
 
-cudaError_t fx_forward_group(const FwdGroup<double>& G, int ctas, size_t smem, cudaStream_t s) {
-    return fft_launch(fx_forward_group_kernel, G, dim3(ctas), smem, s);
+cudaError_t fx_forward_group(const FwdGroup<double>& G, int ctas, size_t smem, cudaStream_t s,
+                             Follow follow) {
+    return fft_launch(fx_forward_group_kernel, G, dim3(ctas), smem, s, follow);
 }
 
-cudaError_t fx_inverse_group(const InvGroup<double>& G, int ctas, size_t smem, cudaStream_t s) {
-    return fft_launch(fx_inverse_group_kernel, G, dim3(ctas), smem, s);
+cudaError_t fx_inverse_group(const InvGroup<double>& G, int ctas, size_t smem, cudaStream_t s,
+                             Follow follow) {
+    return fft_launch(fx_inverse_group_kernel, G, dim3(ctas), smem, s, follow);
 }
 
 }  // namespace sht

@@ -7,23 +7,23 @@ namespace sht {
 cudaError_t fft_bluestein_init() { return upload_twiddles(); }
 
 cudaError_t fft_bluestein_forward(const RaggedFwd<float>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s, bool beside) {
-    return fft_launch(fft_forward_bluestein_kernel<float>, R, grid, smem, s, beside);
+                                  cudaStream_t s, Follow follow) {
+    return fft_launch(fft_forward_bluestein_kernel<float>, R, grid, smem, s, follow);
 }
 
 cudaError_t fft_bluestein_forward(const RaggedFwd<double>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s, bool beside) {
-    return fft_launch(fft_forward_bluestein_kernel<double>, R, grid, smem, s, beside);
+                                  cudaStream_t s, Follow follow) {
+    return fft_launch(fft_forward_bluestein_kernel<double>, R, grid, smem, s, follow);
 }
 
 cudaError_t fft_bluestein_inverse(const RaggedInv<float>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s, bool beside) {
-    return fft_launch(fft_inverse_bluestein_kernel<float>, R, grid, smem, s, beside);
+                                  cudaStream_t s, Follow follow) {
+    return fft_launch(fft_inverse_bluestein_kernel<float>, R, grid, smem, s, follow);
 }
 
 cudaError_t fft_bluestein_inverse(const RaggedInv<double>& R, dim3 grid, size_t smem,
-                                  cudaStream_t s, bool beside) {
-    return fft_launch(fft_inverse_bluestein_kernel<double>, R, grid, smem, s, beside);
+                                  cudaStream_t s, Follow follow) {
+    return fft_launch(fft_inverse_bluestein_kernel<double>, R, grid, smem, s, follow);
 }
 
 }  // namespace sht

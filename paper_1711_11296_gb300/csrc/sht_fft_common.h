@@ -68,6 +68,7 @@ struct FwdArgs {
     const V* chirp;            // Bluestein rows: e^{-i pi n^2 / L}
     const V* dft;              // Bluestein rows: DFT of the conjugate chirp / L2
     int F, J, Jh, L, LP, N, G;
+    int follow;                // see Follow
     FftShape shape;
 };
 
@@ -93,6 +94,7 @@ struct InvArgs {
     const V* chirp;            // Bluestein rows: e^{-i pi n^2 / L}
     const V* dft;              // Bluestein rows: DFT of the conjugate chirp / L2
     int F, J, Jh, I, L, LP, N, G;
+    int follow;                // see Follow
     FftShape shape;
 };
 
@@ -126,38 +128,39 @@ __device__ __forceinline__ int row_pitch(int n) {
     return n + (n >> PadShift<T>::value) + 1;
 }
 
+// How an FFT launch follows the kernel before it in the stream.
 // The launches of one reduced-grid FFT (a class per row length, the run-time
-// shapes, Bluestein rows) work on different rows and may run side by side:
-// each but the first is launched as a programmatic dependent of the one
-// before, which lets it start once that one's CTAs have. Every kernel waits
-// for its predecessor only before it ends, so that what follows the last of
-// them in the stream follows all of them.
-__device__ __forceinline__ void begin_beside() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// shapes, Bluestein rows) work on different rows and may run side by side: the
+// first is launched plainly, each other one as a programmatic dependent of the
+// one before that waits for it only before it ends (kBeside), so that what
+// follows the last of them in the stream follows all of them.
+enum Follow {
+    kPlain = 0,    // after that kernel has ended
+    kWait = 1,     // a dependent launch that waits at its start
+    kBeside = 2,   // a dependent launch that waits at its end
+};
+__device__ __forceinline__ void begin_fft(int follow) {
+    grid_trigger();
+    if (follow == kWait) grid_wait();
 }
-__device__ __forceinline__ void end_beside() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// (unconditional: it returns at once unless the launch is kBeside, and behind a
+// branch the FP64 forward came out 4 to 7 % slower)
+__device__ __forceinline__ void end_fft() { grid_wait(); }
 
-// One FFT launch; beside: as a programmatic dependent (above).
+template <typename T> inline void set_follow(FwdArgs<T>& a, int f) { a.follow = f; }
+template <typename T> inline void set_follow(InvArgs<T>& a, int f) { a.follow = f; }
+template <class G> inline void set_follow(G& g, int f) { g.follow = f; }
+
+// One FFT launch; kWait is taken where it pays (short_launch).
 template <class... Params, class Args>
 cudaError_t fft_launch(void (*kernel)(Params...), const Args& args, dim3 grid, size_t smem,
-                       cudaStream_t s, bool beside = false) {
-    cudaError_t e = ensure_smem((const void*)kernel, smem);
+                       cudaStream_t s, Follow follow) {
+    const cudaError_t e = ensure_smem((const void*)kernel, smem);
     if (e) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kFftThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = beside ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kernel, args);
-    note_launch();
-    return e ? e : cudaGetLastError();
+    if (follow == kWait && !short_launch((long long)grid.x * grid.y)) follow = kPlain;
+    Args a = args;
+    set_follow(a, follow);
+    return launch_kernel(kernel, grid, dim3(kFftThreads), smem, s, follow != kPlain, a);
 }
 
 // Iterates idx = tid, tid + kFftThreads, ... as (major, minor) = (idx / d, idx % d)
@@ -182,14 +185,14 @@ struct Walk2 {
 
 // ---- grouped launches: several plans' rows in one grid ----------------
 template <typename T> struct FwdGroup {
-    int n;
+    int n, follow;
     int cta_start[kMaxGroup + 1];   // first CTA of each plan
     int nfg[kMaxGroup];             // field groups per latitude of each plan
     FwdArgs<T> a[kMaxGroup];
 };
 
 template <typename T> struct InvGroup {
-    int n;
+    int n, follow;
     int cta_start[kMaxGroup + 1];
     int nfg[kMaxGroup];
     InvArgs<T> a[kMaxGroup];
@@ -201,6 +204,7 @@ template <typename T> struct InvGroup {
 // longest row of the grid.
 template <typename T> struct RaggedFwd {
     FwdArgs<T> a;
+    int follow;
     const RShape* shapes;
     const int* shape_of;
     const int* shift_of;                       // per latitude pair (null: none shifted)
@@ -211,6 +215,7 @@ template <typename T> struct RaggedFwd {
 
 template <typename T> struct RaggedInv {
     InvArgs<T> a;
+    int follow;
     const RShape* shapes;
     const int* shape_of;
     const int* shift_of;
@@ -242,44 +247,48 @@ __device__ __forceinline__ void apply_shape(Args& A, const R& Rg, int jh) {
 cudaError_t fft_any_init();
 cudaError_t fft_any_forward(const FwdArgs<float>& A, bool strided, dim3 grid, size_t smem,
                             cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_any_inverse(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_any_forward_ragged(const RaggedFwd<float>& R, dim3 grid, size_t smem,
                                    cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_any_inverse_ragged(const RaggedInv<float>& R, dim3 grid, size_t smem,
                                    cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_bluestein_init();
 cudaError_t fft_bluestein_forward(const RaggedFwd<float>& R, dim3 grid, size_t smem,
                                   cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_bluestein_forward(const RaggedFwd<double>& R, dim3 grid, size_t smem,
                                   cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_bluestein_inverse(const RaggedInv<float>& R, dim3 grid, size_t smem,
                                   cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_bluestein_inverse(const RaggedInv<double>& R, dim3 grid, size_t smem,
                                   cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fft_group_init();
-cudaError_t fft_group_forward(const FwdGroup<float>& G, int ctas, size_t smem, cudaStream_t s);
-cudaError_t fft_group_inverse(const InvGroup<float>& G, int ctas, size_t smem, cudaStream_t s);
+cudaError_t fft_group_forward(const FwdGroup<float>& G, int ctas, size_t smem, cudaStream_t s,
+    Follow follow);
+cudaError_t fft_group_inverse(const InvGroup<float>& G, int ctas, size_t smem, cudaStream_t s,
+    Follow follow);
 
 // Fixed-point FFT launches of the FP64 path (sht_fft64.cu); the arguments'
 // twiddle tables are the fixed-point ones (launch_fixed_twiddles).
 cudaError_t fx_forward(const FwdArgs<double>& A, bool strided, dim3 grid, size_t smem,
                        cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fx_inverse(const InvArgs<double>& A, dim3 grid, size_t smem, cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fx_forward_ragged(const RaggedFwd<double>& R, dim3 grid, size_t smem, cudaStream_t s,
-    bool beside = false);
+    Follow follow);
 cudaError_t fx_inverse_ragged(const RaggedInv<double>& R, dim3 grid, size_t smem, cudaStream_t s,
-    bool beside = false);
-cudaError_t fx_forward_group(const FwdGroup<double>& G, int ctas, size_t smem, cudaStream_t s);
-cudaError_t fx_inverse_group(const InvGroup<double>& G, int ctas, size_t smem, cudaStream_t s);
+    Follow follow);
+cudaError_t fx_forward_group(const FwdGroup<double>& G, int ctas, size_t smem, cudaStream_t s,
+    Follow follow);
+cudaError_t fx_inverse_group(const InvGroup<double>& G, int ctas, size_t smem, cudaStream_t s,
+    Follow follow);
 
 }  // namespace sht

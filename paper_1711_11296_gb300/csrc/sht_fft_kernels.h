@@ -877,9 +877,9 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
 template <typename T, int LT, bool STRIDED>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_forward_kernel(const __grid_constant__ FwdArgs<T> A) {
-    begin_beside();
+    begin_fft(A.follow);
     fwd_body<T, LT, STRIDED>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
-    end_beside();
+    end_fft();
 }
 
 template <typename T, int LT>
@@ -1206,14 +1206,15 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
 template <typename T, int LT>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_inverse_kernel(const __grid_constant__ InvArgs<T> A) {
-    begin_beside();
+    begin_fft(A.follow);
     inv_body<T, LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
-    end_beside();
+    end_fft();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_forward_group_kernel(const __grid_constant__ FwdGroup<T> G) {
+    begin_fft(G.follow);
     const int b = blockIdx.x;
     int p = 0;
     while (p + 1 < G.n && b >= G.cta_start[p + 1]) ++p;
@@ -1237,6 +1238,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_inverse_group_kernel(const __grid_constant__ InvGroup<T> G) {
+    begin_fft(G.follow);
     const int b = blockIdx.x;
     int p = 0;
     while (p + 1 < G.n && b >= G.cta_start[p + 1]) ++p;
@@ -1259,46 +1261,46 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_forward_ragged_kernel(const __grid_constant__ RaggedFwd<T> R) {
-    begin_beside();
+    begin_fft(R.follow);
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<T> A = R.a;
     apply_shape(A, R, jh);
     fwd_body<T, -1, false>(A, blockIdx.x, jh);
-    end_beside();
+    end_fft();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_inverse_ragged_kernel(const __grid_constant__ RaggedInv<T> R) {
-    begin_beside();
+    begin_fft(R.follow);
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<T> A = R.a;
     apply_shape(A, R, jh);
     inv_body<T, -1>(A, blockIdx.x, jh);
-    end_beside();
+    end_fft();
 }
 
 // Rows whose half-length has a prime factor above 5: Bluestein's method.
 template <typename T>
 __global__ void __launch_bounds__(NT, 2)
     fft_forward_bluestein_kernel(const __grid_constant__ RaggedFwd<T> R) {
-    begin_beside();
+    begin_fft(R.follow);
     const int jh = R.a.jh_list[blockIdx.y];
     FwdArgs<T> A = R.a;
     apply_shape(A, R, jh);
     fwd_body<T, -2, false>(A, blockIdx.x, jh);
-    end_beside();
+    end_fft();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(NT, 2)
     fft_inverse_bluestein_kernel(const __grid_constant__ RaggedInv<T> R) {
-    begin_beside();
+    begin_fft(R.follow);
     const int jh = R.a.jh_list[blockIdx.y];
     InvArgs<T> A = R.a;
     apply_shape(A, R, jh);
     inv_body<T, -2>(A, blockIdx.x, jh);
-    end_beside();
+    end_fft();
 }
 
 // c_twf of this translation unit on the current device.

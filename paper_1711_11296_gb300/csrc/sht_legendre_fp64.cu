@@ -163,7 +163,10 @@ __global__ void __launch_bounds__(NT) legendre_inv_fp64_kernel(
 // product per output, bound by the FP64 pipe and, below it, by latency.
 __global__ void __launch_bounds__(128) legendre_small_fp64_kernel(
     const double* __restrict__ pnm, int ldp, const double* __restrict__ in,
-    double* __restrict__ out, int N, int Jh, int C, const int* __restrict__ jmin, int inverse) {
+    double* __restrict__ out, int N, int Jh, int C, const int* __restrict__ jmin, int inverse,
+    int wait) {
+    grid_trigger();
+    if (wait) grid_wait();
     const int m = blockIdx.x >> 1, q = blockIdx.x & 1;
     const int R = parity_rows(N, m, q);
     const size_t row0 = dcoef_offset(N, m) + q;
@@ -194,10 +197,9 @@ cudaError_t launch_small(const sht_plan_s* p, bool inverse, const double* in, do
                          cudaStream_t s) {
     const int C = 2 * p->F, rows = inverse ? p->Jh : p->N / 2 + 1;
     const dim3 grid(2 * (p->N + 1), (rows * C + 127) / 128);
-    legendre_small_fp64_kernel<<<grid, 128, 0, s>>>(p->d_pnm, p->ldp, in, out, p->N, p->Jh, C,
-                                                    p->d_jmin, inverse ? 1 : 0);
-    note_launch();
-    return cudaGetLastError();
+    const bool wait = short_launch((long long)grid.x * grid.y);
+    return launch_kernel(legendre_small_fp64_kernel, grid, dim3(128), 0, s, wait, p->d_pnm, p->ldp,
+                         in, out, p->N, p->Jh, C, p->d_jmin, inverse ? 1 : 0, wait ? 1 : 0);
 }
 
 }  // namespace

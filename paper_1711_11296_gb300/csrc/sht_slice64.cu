@@ -152,9 +152,11 @@ __global__ void __launch_bounds__(512)
     slice_b_kernel(const double* __restrict__ B, const S64Prob* __restrict__ probs, int p0, int C,
                    int C16, unsigned char* __restrict__ out, int* __restrict__ eb,
                    const double* __restrict__ pnm, int ldp, int N, int Jh,
-                   double* __restrict__ O) {
+                   double* __restrict__ O, int wait) {
     __shared__ int red[16][32];
     __shared__ double redq[16][32];
+    grid_trigger();
+    if (wait) grid_wait();
     const int p = p0 + blockIdx.x;
     const S64Prob pr = probs[p];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -315,6 +317,7 @@ struct S64Args {
     const int* jmin;   // reduced transform (Sec. 4.1): first significant node per problem
     int inverse;
     int C, C16;
+    int wait;          // a dependent launch: wait for the kernel before
     int* status;
 };
 
@@ -345,6 +348,7 @@ __device__ __forceinline__ double scale2(double d, int k) {
 // main loop.
 template <bool MCOLS>
 __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant__ S64Args g) {
+    grid_trigger();
     extern __shared__ __align__(1024) unsigned char s64_smem[];
     unsigned char* smem = s64_smem;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NSTAGE * STAGE);
@@ -381,6 +385,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    if (g.wait) grid_wait();
 
     // first K slab and number of slabs of a tile (the reduced transform skips
     // forward slabs, and inverse tiles whose outputs are then zero, of nodes
@@ -633,17 +638,19 @@ void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
 }
 
 template <bool INV>
-void launch_slice_b(int maxK, dim3 grid, cudaStream_t s, const double* B, const S64Prob* probs,
+cudaError_t launch_slice_b(int maxK, dim3 grid, cudaStream_t s, const double* B, const S64Prob* probs,
                     int p0, int C, int C16, unsigned char* out, int* eb, const double* pnm,
                     int ldp, int N, int Jh, double* O) {
     using Fn = void (*)(const double*, const S64Prob*, int, int, int, unsigned char*, int*,
-                        const double*, int, int, int, double*);
+                        const double*, int, int, int, double*, int);
     static const Fn tab[7] = {slice_b_kernel<0, INV>, slice_b_kernel<1, INV>,
                               slice_b_kernel<2, INV>, slice_b_kernel<3, INV>,
                               slice_b_kernel<4, INV>, slice_b_kernel<5, INV>,
                               slice_b_kernel<6, INV>};
     const int ng = (maxK + 127) / 128;
-    tab[ng <= 6 ? ng : 0]<<<grid, 512, 0, s>>>(B, probs, p0, C, C16, out, eb, pnm, ldp, N, Jh, O);
+    const bool wait = short_launch((long long)grid.x * grid.y);
+    return launch_kernel(tab[ng <= 6 ? ng : 0], grid, dim3(512), 0, s, wait, B, probs, p0, C, C16,
+                         out, eb, pnm, ldp, N, Jh, O, wait ? 1 : 0);
 }
 
 cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, double* O,
@@ -658,13 +665,12 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
     for (const S64Chunk& c : d.chunks) {
         const dim3 grid(c.p1 - c.p0, (sl->C16 + 31) / 32);
         if (inverse)
-            launch_slice_b<true>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
+            e = launch_slice_b<true>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
                                  sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
         else
-            launch_slice_b<false>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
+            e = launch_slice_b<false>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
                                   sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
-        note_launch();
-        if ((e = cudaGetLastError())) return e;
+        if (e) return e;
         S64Args g;
         g.table = d.table;
         g.bbuf = sl->bbuf;
@@ -679,14 +685,12 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
         g.C = C;
         g.C16 = sl->C16;
         g.status = p->d_status;
+        g.wait = short_launch(g.ntiles) ? 1 : 0;
         if (g.ntiles == 0) continue;
         const int ctas = std::min(g.ntiles, p->num_sms);
-        if (d.mcols)
-            slice_gemm_kernel<true><<<ctas, NT, SMEM, s>>>(g);
-        else
-            slice_gemm_kernel<false><<<ctas, NT, SMEM, s>>>(g);
-        note_launch();
-        if ((e = cudaGetLastError())) return e;
+        e = launch_kernel(d.mcols ? slice_gemm_kernel<true> : slice_gemm_kernel<false>, dim3(ctas),
+                          dim3(NT), SMEM, s, g.wait != 0, g);
+        if (e) return e;
     }
     return cudaSuccess;
 }

@@ -163,6 +163,7 @@ struct GemmArgs {
     long long bplane_bytes;
     int nct;                        // column tiles (pre-split B tile index = it * nct + ct)
     int stall;                      // fault injection for tests: CTA 0 never arms stage 0
+    int wait;                       // a dependent launch: wait for the kernel before
     // raw_bulk: B as a row-major matrix [rows][C] of floats (problem
     // rows at b_off / b_stride), box TN columns x TK rows; out-of-range
     // columns and rows read as zero
@@ -273,6 +274,7 @@ extern __shared__ __align__(1024) unsigned char split_smem[];
 struct OnePlanArgs {
     const GemmArgs& g;
     __device__ __forceinline__ const GemmArgs& operator()(const int4&) const { return g; }
+    __device__ __forceinline__ bool wait() const { return g.wait != 0; }
     __device__ __forceinline__ void mark_timeout() const {
         if (g.status) atomicOr(g.status, 1);
     }
@@ -281,6 +283,7 @@ struct GroupPlanArgs {
     const GemmArgs* a;
     int n;
     __device__ __forceinline__ const GemmArgs& operator()(const int4& t) const { return a[t.w]; }
+    __device__ __forceinline__ bool wait() const { return a[0].wait != 0; }
     __device__ __forceinline__ void mark_timeout() const {
         for (int q = 0; q < n; ++q)
             if (a[q].status) atomicOr(a[q].status, 1);
@@ -322,6 +325,7 @@ __device__ __forceinline__ void split_gemm_body(const Args& args, const int4* __
     volatile int* abort_flag =
         reinterpret_cast<volatile int*>(smem + CF::BAR_OFF + 8 * NB + 8);
 
+    grid_trigger();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t bar0 = smem_u32(bars);
     auto full_a = [&](int s) { return bar0 + 8u * s; };
@@ -364,6 +368,7 @@ __device__ __forceinline__ void split_gemm_body(const Args& args, const int4* __
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    if (args.wait()) grid_wait();
 
     // stages it = kb .. kb + nst - 1 of a tile (the reduced transform skips
     // the K tiles of negligible P~ in the forward direction and whole row
@@ -834,10 +839,11 @@ __global__ void __launch_bounds__(256)
     split_b_kernel(const float* __restrict__ B, const SplitProb* __restrict__ probs, int C,
                    int nct, const unsigned* __restrict__ colmax, unsigned char* planes,
                    long long plane_bytes, const double* __restrict__ pnm, int ldp, int N,
-                   int Jh, float* __restrict__ O) {
+                   int Jh, float* __restrict__ O, int wait) {
     constexpr int B_TILE_BYTES = Wid<TN>::B_TILE_BYTES;
     extern __shared__ float2 peq[];   // [K] P~(0) of the problem's rows, (hi, lo)
     __shared__ float2 red[8][32];
+    grid_trigger();
     const int p = blockIdx.x;
     const SplitProb pr = probs[p];
     const bool even = (p & 1) == 0;
@@ -850,6 +856,7 @@ __global__ void __launch_bounds__(256)
         }
     }
     __syncthreads();
+    if (wait) grid_wait();   // (the table of P~(0) above is the plan's own)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int c = blockIdx.y * 128 + (w & 3) * 32 + lane;
     const bool cin = c < C;
@@ -996,6 +1003,7 @@ __global__ void __launch_bounds__(256) colmax_kernel(const float* __restrict__ B
                                                      long long nrows, int C, int skip_odd,
                                                      unsigned* colmax) {
     __shared__ float red[8][32];
+    grid_trigger();
     const int c = blockIdx.x * 32 + threadIdx.x;
     const long long per = (nrows + gridDim.y - 1) / gridDim.y;
     const long long r0 = (long long)blockIdx.y * per;
@@ -1156,6 +1164,7 @@ GemmArgs make_gemm_args(const sht_plan_s* p, bool inverse, const void* B, void* 
     g.O = static_cast<float*>(O);
     g.C = 2 * p->F;
     g.raw_bulk = 0;
+    g.wait = 0;
     g.status = p->d_status;
     g.rs_inv = inverse ? st->rs_inv : st->rs_fwd;
     g.colmax = p->d_colmax ? p->d_colmax + (inverse ? g.C : 0) : nullptr;
@@ -1199,7 +1208,9 @@ int persistent_ctas(int per_sm, int ntiles) {
 }
 
 template <int T, bool F16, bool BPRE, int TN>
-cudaError_t gemm_launch(const GemmArgs& g, int ntiles, cudaStream_t s) {
+cudaError_t gemm_launch(const GemmArgs& args, int ntiles, cudaStream_t s) {
+    GemmArgs g = args;
+    g.wait = short_launch(ntiles) ? 1 : 0;
     constexpr int smem = Cfg<T, BPRE, TN>::SMEM;
     const void* fn = (const void*)split_gemm_kernel<T, F16, BPRE, TN>;
     cudaError_t e = ensure_smem(fn, smem);
@@ -1210,9 +1221,8 @@ cudaError_t gemm_launch(const GemmArgs& g, int ntiles, cudaStream_t s) {
     // schedules in list order, so that the column tiles sharing a P~ tile
     // run together and that tile comes from L2 after its first read
     const int nctas = BPRE ? persistent_ctas(Wid<TN>::CTAS_PER_SM, ntiles) : ntiles;
-    split_gemm_kernel<T, F16, BPRE, TN><<<nctas, NTHREADS, smem, s>>>(g);
-    note_launch();
-    return cudaGetLastError();
+    return launch_kernel(split_gemm_kernel<T, F16, BPRE, TN>, dim3(nctas), dim3(NTHREADS), smem, s,
+                         g.wait != 0, g);
 }
 
 // Variant index: bit 0 three terms, bit 1 FP16, bit 2 pre-split B, bit 3 TN = 64.
@@ -1248,16 +1258,15 @@ cudaError_t launch_split_b_inverse(const sht_plan_s* p, const void* spec, void* 
     const unsigned* cm = p->d_colmax ? p->d_colmax + C : nullptr;
     const long long pb = (long long)st->inv_bplane_bytes;
     using Fn = void (*)(const float*, const SplitProb*, int, int, const unsigned*,
-                        unsigned char*, long long, const double*, int, int, int, float*);
+                        unsigned char*, long long, const double*, int, int, int, float*, int);
     static const Fn tab[8] = {split_b_kernel<2, false, 128>, split_b_kernel<3, false, 128>,
                               split_b_kernel<2, true, 128>,  split_b_kernel<3, true, 128>,
                               split_b_kernel<2, false, 64>,  split_b_kernel<3, false, 64>,
                               split_b_kernel<2, true, 64>,   split_b_kernel<3, true, 64>};
     const Fn k = tab[(variant(st->terms, st->fp16, false, st->tn) & 3) | (st->tn == 64 ? 4 : 0)];
-    k<<<grid, 256, smem, s>>>(B, st->d_probs_inv, C, nct, cm, st->inv_bplanes, pb, p->d_pnm,
-                              p->ldp, p->N, p->Jh, O);
-    note_launch();
-    return cudaGetLastError();
+    const bool wait = short_launch((long long)grid.x * grid.y);
+    return launch_kernel(k, grid, dim3(256), smem, s, wait, B, st->d_probs_inv, C, nct, cm,
+                         st->inv_bplanes, pb, p->d_pnm, p->ldp, p->N, p->Jh, O, wait ? 1 : 0);
 }
 
 cudaError_t launch_gemm(const sht_plan_s* p, bool inverse, const void* B, void* O,
@@ -1520,9 +1529,8 @@ cudaError_t group_launch(const GemmGroup& G, int ntiles, cudaStream_t s) {
     // schedules in list order, so that the column tiles sharing a P~ tile
     // run together and that tile comes from L2 after its first read
     const int nctas = BPRE ? persistent_ctas(Wid<TN>::CTAS_PER_SM, ntiles) : ntiles;
-    split_gemm_group_kernel<T, F16, BPRE, TN><<<nctas, NTHREADS, smem, s>>>(G);
-    note_launch();
-    return cudaGetLastError();
+    return launch_kernel(split_gemm_group_kernel<T, F16, BPRE, TN>, dim3(nctas), dim3(NTHREADS),
+                         smem, s, G.a[0].wait != 0, G);
 }
 
 cudaError_t launch_split_group(sht_plan_s* const* plans, int n, bool inverse,
@@ -1532,7 +1540,10 @@ cudaError_t launch_split_group(sht_plan_s* const* plans, int n, bool inverse,
     G.n = n;
     G.ntiles = ntiles;
     G.tiles = tiles;
-    for (int q = 0; q < n; ++q) G.a[q] = make_gemm_args(plans[q], inverse, in[q], out[q]);
+    for (int q = 0; q < n; ++q) {
+        G.a[q] = make_gemm_args(plans[q], inverse, in[q], out[q]);
+        G.a[q].wait = short_launch(ntiles) ? 1 : 0;
+    }
     const SplitTables* st = plans[0]->split;
     if (inverse)
         for (int q = 0; q < n; ++q) {
