@@ -84,7 +84,9 @@ FwdArgs<T> make_fwd_args(const sht_plan_s* p, const void* grid, const RowSource&
 template <typename T>
 cudaError_t fwd_impl(const sht_plan_s* p, const void* grid, const RowSource& src,
                      const FwdScale& sc, void* work, cudaStream_t s) {
-    const FwdArgs<T> A = make_fwd_args<T>(p, grid, src, sc, work);
+    FwdArgs<T> A = make_fwd_args<T>(p, grid, src, sc, work);
+    A.src.quads = sizeof(T) == 4 && src.elem_stride == 2 && ((uintptr_t)grid & 15) == 0 &&
+                  src.field_stride % 4 == 0 && src.row_stride % 4 == 0 && src.row_offset % 4 == 0;
     if (A.colmax) {
         const cudaError_t e = cudaMemsetAsync(A.colmax, 0, 2 * (size_t)p->F * sizeof(unsigned), s);
         if (e) return e;

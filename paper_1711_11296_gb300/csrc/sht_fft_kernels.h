@@ -565,50 +565,66 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
                (long long)j * A.src.row_stride;
     };
 
-    if constexpr (!STRIDED && first_pass_from_global<T, LT>()) {
-        // The first pass (radix Q, span 32) reads its inputs straight from
-        // the grid rows into registers: butterfly n1 of a row takes
-        // z[n1 + 32 t], t < Q, so for each t the lanes of a warp load 256
-        // contiguous bytes.  Only the twiddle table is copied
-        // asynchronously; the first butterfly's loads are in flight while
-        // the CTA waits for it.
-        constexpr FftShape FS = FacOf<LT, false>::v;
-        constexpr int Q = FS.radix[0];
-        constexpr int M = FS.span[0];                                  // 32
-        constexpr int STEP = M + (M >> PadShift<T>::value);            // padded
-        load_twiddles_async(tws, A.twp, FS.twtotal);
-        const int total = nrows * M;
-        V a[Q];
-        auto load = [&](int idx) {
-            const int r = idx / M, n1 = idx - r * M;
-            const V* x = reinterpret_cast<const V*>(row_ptr(r)) + n1;
-#pragma unroll
-            for (int t = 0; t < Q; ++t) a[t] = x[t * M];
-        };
-        auto finish = [&](int idx) {
-            const int r = idx / M, n1 = idx - r * M;
-            Dft<T, Q>::run(a);
-            if (n1 != 0) {
-#pragma unroll
-                for (int k1 = 1; k1 < Q; ++k1)
-                    a[Dft<T, Q>::pos(k1)] =
-                        K::mul(a[Dft<T, Q>::pos(k1)], tws[(k1 - 1) * M + n1]);
-            }
-            V* zb = rows + (size_t)r * LP + n1;
-#pragma unroll
-            for (int k1 = 0; k1 < Q; ++k1) zb[k1 * STEP] = a[Dft<T, Q>::pos(k1)];
-        };
-        if (tid < total) load(tid);
-        cp_async_wait_all();
-        __syncthreads();
-        if (tid < total) finish(tid);
-        for (int idx = tid + NT; idx < total; idx += NT) {
-            load(idx);
-            finish(idx);
+    // Complex element k of a row straight from the grid.  In a nested fine grid
+    // of twice the longitudes one 16-byte load holds the two samples wanted and
+    // the two between (T511 -> T255 x 64: 88 -> 76 us); larger strides are copied
+    // to shared memory first (as two loads into registers T1279 -> T319 x 64 took
+    // 199 us against 185).
+    auto load_z = [&](const V* x, int k) -> V {
+        if constexpr (!STRIDED) {
+            return x[k];
+        } else {
+            const float4 v = reinterpret_cast<const float4*>(x)[k];
+            return K::make((T)v.x, (T)v.z);
         }
-        __syncthreads();
-        passes_fixed<T, LT, 1>(rows, nrows, LP, tws);
-    } else if (LT == -1 && !STRIDED && sizeof(T) == 4 && A.shape.npass > 0) {
+    };
+    const bool direct = !STRIDED || A.src.quads;
+    if (first_pass_from_global<T, LT>() && direct) {
+        if constexpr (first_pass_from_global<T, LT>()) {
+            // The first pass (radix Q, span 32) reads its inputs straight from
+            // the grid rows into registers: butterfly n1 of a row takes
+            // z[n1 + 32 t], t < Q, so for each t the lanes of a warp load 256
+            // contiguous bytes.  Only the twiddle table is copied
+            // asynchronously; the first butterfly's loads are in flight while
+            // the CTA waits for it.
+            constexpr FftShape FS = FacOf<LT, false>::v;
+            constexpr int Q = FS.radix[0];
+            constexpr int M = FS.span[0];                                  // 32
+            constexpr int STEP = M + (M >> PadShift<T>::value);            // padded
+            load_twiddles_async(tws, A.twp, FS.twtotal);
+            const int total = nrows * M;
+            V a[Q];
+            auto load = [&](int idx) {
+                const int r = idx / M, n1 = idx - r * M;
+                const V* x = reinterpret_cast<const V*>(row_ptr(r));
+#pragma unroll
+                for (int t = 0; t < Q; ++t) a[t] = load_z(x, n1 + t * M);
+            };
+            auto finish = [&](int idx) {
+                const int r = idx / M, n1 = idx - r * M;
+                Dft<T, Q>::run(a);
+                if (n1 != 0) {
+#pragma unroll
+                    for (int k1 = 1; k1 < Q; ++k1)
+                        a[Dft<T, Q>::pos(k1)] =
+                            K::mul(a[Dft<T, Q>::pos(k1)], tws[(k1 - 1) * M + n1]);
+                }
+                V* zb = rows + (size_t)r * LP + n1;
+#pragma unroll
+                for (int k1 = 0; k1 < Q; ++k1) zb[k1 * STEP] = a[Dft<T, Q>::pos(k1)];
+            };
+            if (tid < total) load(tid);
+            cp_async_wait_all();
+            __syncthreads();
+            if (tid < total) finish(tid);
+            for (int idx = tid + NT; idx < total; idx += NT) {
+                load(idx);
+                finish(idx);
+            }
+            __syncthreads();
+            passes_fixed<T, LT, 1>(rows, nrows, LP, tws);
+        }
+    } else if (LT == -1 && sizeof(T) == 4 && A.shape.npass > 0 && direct) {
         // the same with the shape known at run time
         const int M = A.shape.span[0];
         load_twiddles_async(tws, A.twp, A.shape.twtotal);
@@ -621,9 +637,9 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
                 const int r = work ? idx / M : 0, n1 = idx - r * M;
                 V a[R];
                 if (work) {
-                    const V* x = reinterpret_cast<const V*>(row_ptr(r)) + n1;
+                    const V* x = reinterpret_cast<const V*>(row_ptr(r));
 #pragma unroll
-                    for (int t = 0; t < R; ++t) a[t] = x[t * M];
+                    for (int t = 0; t < R; ++t) a[t] = load_z(x, n1 + t * M);
                 }
                 if (!waited) {
                     cp_async_wait_all();

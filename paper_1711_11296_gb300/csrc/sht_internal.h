@@ -58,6 +58,7 @@ struct RowSource {
     long long row_stride = 0;     // elements between consecutive (coarse) rows
     long long row_offset = 0;     // element offset of row 0
     int elem_stride = 1;          // elements between consecutive longitudes
+    int quads = 0;                // FP32, elem_stride 2, every row 16-byte aligned
 };
 
 // Scaling applied by the forward (analysis-type) FFT kernel.

@@ -105,3 +105,18 @@ def test_reduced_grid_captured_in_a_graph(sht):
         torch.cuda.synchronize()
         assert torch.equal(grid, ref_grid) and torch.equal(spec, ref_spec)
     p.status()
+
+
+@pytest.mark.parametrize("I", [40, 128, 1280])
+@pytest.mark.parametrize("k,offset", [(1, 0), (1, 2), (1, 4), (2, 0)])
+def test_restriction_reads_any_alignment(sht, I, k, offset):
+    # the nested rows' 16-byte loads (k = 1, aligned) and the copies of other
+    # strides and alignments give the transform of the injected grid
+    F, Nc, Jc = 3, 7, 15
+    p = sht.Plan(Nc, Jc, I, F, "bf16x3")
+    shape = (F, 2 ** k * (Jc + 1) - 1, 2 ** k * I)
+    n = int(np.prod(shape))
+    buf = torch.randn(n + offset, device="cuda", generator=torch.Generator("cuda").manual_seed(I))
+    fine = buf[offset:].view(shape)
+    ref = p.forward(p.inject_nested(fine, k))
+    assert torch.equal(p.restrict_nested(fine, k), ref)
