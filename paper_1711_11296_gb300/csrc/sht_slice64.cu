@@ -7,8 +7,8 @@
 // (sht_legendre_fp64.cu).  The tensor cores do about 1700 times as many
 // BF16 products, and BF16 holds every integer up to 256 exactly.  Measured
 // (us, forward / inverse contraction, FP64 pipe -> slices): T639 x 256
-// 120600 / 117800 -> 6650 / 6570; T319 x 100 8530 / 8090 -> 673 / 952;
-// T159 x 256 2721 / 2411 -> 310 / 327.
+// 120600 / 117800 -> 6660 / 7500; T319 x 100 8530 / 8090 -> 685 / 845;
+// T159 x 256 2721 / 2411 -> 316 / 362.
 //
 // Every row r of A (the P~ table) and every column c of B (the Fourier data
 // or the spectrum) is scaled by a power of two to an integer of at most
@@ -63,6 +63,7 @@ struct S64Chunk { int p0, p1, t0, t1; };
 
 struct S64Dir {
     bool mcols = true;              // the MMA's 128-wide M side holds columns (else rows)
+    int tn = 80;                    // N width of the tiles
     unsigned char* table = nullptr; // A slices: per problem [K slab][slice][R16][16]
     int* ea = nullptr;              // exponent of every row of A
     S64Prob* d_probs = nullptr;
@@ -80,15 +81,22 @@ struct Slice64 {
 
 namespace {
 
-constexpr int TM = 128, TN = 64, TK = 16;   // MMA tile: M x N, K slab
-constexpr int NSTAGE = 5;
-constexpr int M_SLICE = TM * TK * 2, N_SLICE = TN * TK * 2;   // bytes
-constexpr int STAGE = kSlices * (M_SLICE + N_SLICE);          // 43 KB
+constexpr int TM = 128, TK = 16;            // MMA tile: M, K slab
 constexpr int NACC = 6;                     // accumulators of TN TMEM columns
 constexpr int TMEM_COLS = 512;
-constexpr int NBAR = 2 * NSTAGE + 3;
-constexpr int SMEM = NSTAGE * STAGE + 256;
-static_assert(SMEM <= 227 * 1024 && 8 * NBAR + 16 <= 256, "one CTA's shared memory");
+constexpr int M_SLICE = TM * TK * 2;        // bytes
+
+// By the tile's N width: a stage holds the 14 slices of a K slab; as many
+// stages as fit.
+template <int TN> struct Cfg {
+    static constexpr int N_SLICE = TN * TK * 2;
+    static constexpr int STAGE = kSlices * (M_SLICE + N_SLICE);
+    static constexpr int NSTAGE = (227 * 1024 - 256) / STAGE;
+    static constexpr int NBAR = 2 * NSTAGE + 3;
+    static constexpr int SMEM = NSTAGE * STAGE + 256;
+    static_assert(8 * NBAR + 16 <= 256 && NACC * TN <= TMEM_COLS, "barriers and accumulators fit");
+};
+
 constexpr int NEPI = 256;                   // epilogue threads (8 warps)
 constexpr int NT = NEPI + 64;               // + copy warp + MMA warp
 constexpr int kNonFinite = INT_MAX;         // column exponent of Inf / NaN columns
@@ -337,17 +345,22 @@ __device__ __forceinline__ double scale2(double d, int k) {
     return scalbn(d, k);
 }
 
-// Persistent CTAs, one per SM: 128 x 64 tiles (M x N) with six FP32
-// accumulators (384 of the 512 TMEM columns), K slabs of 16 through a ring
-// of 5 stages of 43 KB (14 slices).  Warps 0-7 the epilogue, warp 8 the bulk
-// copies (a lane per slice), one thread of warp 9 the 34 MMAs of a stage.
-// The ring runs on across tiles, so the next tile's operands load during
-// the epilogue.
-// Per stage the MMAs read 34 x 6 KB of shared memory (48 cycles each at 128
-// bytes per clock, against 32 at the tensor rate): that port bounds the
-// main loop.
-template <bool MCOLS>
+// Persistent CTAs, one per SM: 128 x TN tiles (M x N) with six FP32
+// accumulators (480 of the 512 TMEM columns at TN = 80), K slabs of 16
+// through a ring of 4 (TN = 80) to 6 (32) stages of 14 slices, 35 to 46 KB.
+// Warps 0-7 the epilogue, warp 8 the bulk copies (a lane per slice), one
+// thread of warp 9 the 34 MMAs of a stage.  The ring runs on across tiles, so
+// the next tile's operands load during the epilogue.  An MMA reads 4 KB of M
+// and TN 32 bytes of N from shared memory, 128 bytes per clock: 52 cycles at
+// TN = 80 against 40 at the tensor rate, which bounds the main loop; the wider
+// tile shares the M side among more columns (TN = 64 -> 80, us forward /
+// inverse: T639 x 256 7114 / 8087 -> 6660 / 7522, T319 x 100 727 / 983 -> 687 / 845, T159 x 256
+// 346 / 425 -> 316 / 362).  Where N never exceeds 64 or 32 the narrower
+// configuration's deeper ring is faster (T200 x 20: TN = 80 100 / 119, 64 94 / 110).
+template <bool MCOLS, int TN>
 __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant__ S64Args g) {
+    using CF = Cfg<TN>;
+    constexpr int NSTAGE = CF::NSTAGE, STAGE = CF::STAGE, NBAR = CF::NBAR, N_SLICE = CF::N_SLICE;
     grid_trigger();
     extern __shared__ __align__(1024) unsigned char s64_smem[];
     unsigned char* smem = s64_smem;
@@ -493,7 +506,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
         }
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (the M
-        // side), N columns 32 (w / 4) .. +31 ----
+        // side), half w / 4 of the N columns ----
         uint32_t nacc = 0;
         bool ok = true;
         const int lq = warp & 3, half = warp >> 2;
@@ -516,7 +529,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             double* om = g.O + pr.o_off + (MCOLS ? (long long)im : (long long)im * pr.o_stride);
             const long long on = MCOLS ? pr.o_stride : 1;
             const int k0 = 56 - 2 * pr.sh;
-            for (int i0 = half * 32; i0 < half * 32 + 32; i0 += 8) {
+            for (int i0 = half * (TN / 2); i0 < (half + 1) * (TN / 2); i0 += 8) {
                 const int n0 = t.z + i0;
                 if (n0 >= nv || !ok) break;   // uniform over the warp
                 uint32_t r[NACC][8];
@@ -613,6 +626,12 @@ void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
         mac_rows += (long long)s.nkt * ((s.R16 + TM - 1) / TM * TM) * C16;
     }
     d.mcols = mac_cols <= mac_rows;
+    int nmax = C16;
+    if (d.mcols) {
+        nmax = 0;
+        for (const S64Prob& s : h.probs) nmax = std::max(nmax, s.R16);
+    }
+    d.tn = nmax <= 32 ? 32 : nmax <= 64 ? 64 : 80;
     S64Chunk ch{0, 0, 0, 0};
     size_t used = 0;
     for (int p = 0; p < nprob; ++p) {
@@ -630,7 +649,7 @@ void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
         h.bbytes = std::max(h.bbytes, used);
         const int mr = d.mcols ? C16 : s.R16, nr = d.mcols ? s.R16 : C16;
         for (int m0 = 0; m0 < mr; m0 += TM)
-            for (int n0 = 0; n0 < nr; n0 += TN) h.tiles.push_back(make_int4(p, m0, n0, 0));
+            for (int n0 = 0; n0 < nr; n0 += d.tn) h.tiles.push_back(make_int4(p, m0, n0, 0));
     }
     ch.p1 = nprob;
     ch.t1 = (int)h.tiles.size();
@@ -658,9 +677,20 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
     const Slice64* sl = p->slice;
     const S64Dir& d = sl->dir[inverse ? 1 : 0];
     const int C = 2 * p->F;
-    const void* fn = d.mcols ? (const void*)slice_gemm_kernel<true>
-                             : (const void*)slice_gemm_kernel<false>;
-    cudaError_t e = ensure_smem(fn, SMEM);
+    using Gemm = void (*)(const S64Args);
+    Gemm fn;
+    int smem;
+    if (d.tn == 32) {
+        fn = d.mcols ? slice_gemm_kernel<true, 32> : slice_gemm_kernel<false, 32>;
+        smem = Cfg<32>::SMEM;
+    } else if (d.tn == 64) {
+        fn = d.mcols ? slice_gemm_kernel<true, 64> : slice_gemm_kernel<false, 64>;
+        smem = Cfg<64>::SMEM;
+    } else {
+        fn = d.mcols ? slice_gemm_kernel<true, 80> : slice_gemm_kernel<false, 80>;
+        smem = Cfg<80>::SMEM;
+    }
+    cudaError_t e = ensure_smem((const void*)fn, smem);
     if (e) return e;
     for (const S64Chunk& c : d.chunks) {
         const dim3 grid(c.p1 - c.p0, (sl->C16 + 31) / 32);
@@ -688,8 +718,7 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
         g.wait = short_launch(g.ntiles) ? 1 : 0;
         if (g.ntiles == 0) continue;
         const int ctas = std::min(g.ntiles, p->num_sms);
-        e = launch_kernel(d.mcols ? slice_gemm_kernel<true> : slice_gemm_kernel<false>, dim3(ctas),
-                          dim3(NT), SMEM, s, g.wait != 0, g);
+        e = launch_kernel(fn, dim3(ctas), dim3(NT), smem, s, g.wait != 0, g);
         if (e) return e;
     }
     return cudaSuccess;

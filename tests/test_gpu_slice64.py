@@ -33,6 +33,11 @@ CASES = [
     (40, 71, 96, 321),      # inexact grid (J < 2 N + 1)
 ]
 
+# Either side of the tile widths 32, 64 and 80: by columns, then by rows.
+WIDTHS = [(159, 321, 640, 16), (159, 321, 640, 17), (159, 321, 640, 32), (159, 321, 640, 33),
+          (159, 321, 640, 40), (159, 321, 640, 41),
+          (95, 193, 192, 64), (127, 257, 288, 64), (159, 321, 640, 64), (161, 325, 648, 64)]
+
 # Transforms with a thread per output, on either side of its row chunks.
 SMALL = [(31, 65, 128, 1), (42, 87, 180, 4), (63, 129, 256, 5), (159, 321, 640, 1),
          (12, 27, 30, 300), (0, 1, 2, 3)]
@@ -45,7 +50,7 @@ def sht():
     return S
 
 
-@pytest.mark.parametrize("N,J,I,F", CASES + SMALL)
+@pytest.mark.parametrize("N,J,I,F", CASES + WIDTHS + SMALL)
 def test_matches_oracle(sht, N, J, I, F):
     p = sht.Plan(N, J, I, F, "fp64")
     x = W.random_grid(F, J, I, seed=2100 + N)
