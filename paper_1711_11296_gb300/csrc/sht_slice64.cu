@@ -7,8 +7,8 @@
 // (sht_legendre_fp64.cu).  The tensor cores do about 1700 times as many
 // BF16 products, and BF16 holds every integer up to 256 exactly.  Measured
 // (us, forward / inverse contraction, FP64 pipe -> slices): T639 x 256
-// 120600 / 117800 -> 6660 / 7500; T319 x 100 8530 / 8090 -> 685 / 845;
-// T159 x 256 2721 / 2411 -> 316 / 362.
+// 120600 / 117800 -> 5780 / 5140; T319 x 100 8530 / 8090 -> 554 / 587;
+// T159 x 256 2721 / 2411 -> 247 / 311.
 //
 // Every row r of A (the P~ table) and every column c of B (the Fourier data
 // or the spectrum) is scaled by a power of two to an integer of at most
@@ -97,7 +97,7 @@ template <int TN> struct Cfg {
     static_assert(8 * NBAR + 16 <= 256 && NACC * TN <= TMEM_COLS, "barriers and accumulators fit");
 };
 
-constexpr int NEPI = 256;                   // epilogue threads (8 warps)
+constexpr int NEPI = 512;                   // epilogue threads (16 warps)
 constexpr int NT = NEPI + 64;               // + copy warp + MMA warp
 constexpr int kNonFinite = INT_MAX;         // column exponent of Inf / NaN columns
 
@@ -325,18 +325,17 @@ struct S64Args {
     const int* jmin;   // reduced transform (Sec. 4.1): first significant node per problem
     int inverse;
     int C, C16;
+    int pairs;         // O is 16-byte aligned
     int wait;          // a dependent launch: wait for the kernel before
     int* status;
 };
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                   "=r"(r[6]), "=r"(r[7])
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr));
 }
 
-// d 2^k for an integer-valued d (0 or 2^0 <= |d| < 2^63).
 __device__ __forceinline__ double scale2(double d, int k) {
     const long long bits = __double_as_longlong(d);
     const int e = (int)((bits >> 52) & 0x7ff) + k;
@@ -348,15 +347,23 @@ __device__ __forceinline__ double scale2(double d, int k) {
 // Persistent CTAs, one per SM: 128 x TN tiles (M x N) with six FP32
 // accumulators (480 of the 512 TMEM columns at TN = 80), K slabs of 16
 // through a ring of 4 (TN = 80) to 6 (32) stages of 14 slices, 35 to 46 KB.
-// Warps 0-7 the epilogue, warp 8 the bulk copies (a lane per slice), one
-// thread of warp 9 the 34 MMAs of a stage.  The ring runs on across tiles, so
+// Warps 0-15 the epilogue, warp 16 the bulk copies (a lane per slice), one
+// thread of warp 17 the 34 MMAs of a stage.  The ring runs on across tiles, so
 // the next tile's operands load during the epilogue.  An MMA reads 4 KB of M
 // and TN 32 bytes of N from shared memory, 128 bytes per clock: 52 cycles at
 // TN = 80 against 40 at the tensor rate, which bounds the main loop; the wider
 // tile shares the M side among more columns (TN = 64 -> 80, us forward /
-// inverse: T639 x 256 7114 / 8087 -> 6660 / 7522, T319 x 100 727 / 983 -> 687 / 845, T159 x 256
-// 346 / 425 -> 316 / 362).  Where N never exceeds 64 or 32 the narrower
-// configuration's deeper ring is faster (T200 x 20: TN = 80 100 / 119, 64 94 / 110).
+// inverse: T639 x 256 7114 / 8087 -> 6660 / 7522, T319 x 100 727 / 983 ->
+// 687 / 845, T159 x 256 346 / 425 -> 316 / 362).  Where N never exceeds 64 or
+// 32 the narrower configuration's deeper ring is faster (T200 x 20: TN = 80
+// 100 / 119, 64 94 / 110).
+// Six accumulators leave no room for a second set, so the MMAs wait while the
+// epilogue reads them: it only forms the 64-bit sums in registers (60 a
+// thread) before it hands them back, and converts, scales and stores beside
+// the next tile's products.  With 16 warps against 8, and the sums by 32-bit
+// multiply-adds: T639 x 256 6660 / 7500 -> 5780 / 5140, T319 x 100 685 / 845
+// -> 554 / 587, T159 x 256 316 / 362 -> 247 / 311 (8 warps alone 5820 / 5550,
+// 562 / 676, 259 / 338).
 template <bool MCOLS, int TN>
 __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant__ S64Args g) {
     using CF = Cfg<TN>;
@@ -506,10 +513,10 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
         }
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (the M
-        // side), half w / 4 of the N columns ----
+        // side), quarter w / 4 of the N columns ----
         uint32_t nacc = 0;
         bool ok = true;
-        const int lq = warp & 3, half = warp >> 2;
+        const int lq = warp & 3, quarter = warp >> 2;
         for (int tt = blockIdx.x; tt < g.ntiles && ok && !aborted(); tt += gridDim.x) {
             const int4 t = g.tiles[tt];
             const S64Prob pr = g.probs[t.x];
@@ -527,46 +534,76 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             auto row_exp = [&](int r) { return max(__ldg(eap + r), 1) - 1022; };
             const int em = mok ? (MCOLS ? __ldg(ebp + im) : row_exp(im)) : 0;
             double* om = g.O + pr.o_off + (MCOLS ? (long long)im : (long long)im * pr.o_stride);
-            const long long on = MCOLS ? pr.o_stride : 1;
             const int k0 = 56 - 2 * pr.sh;
-            for (int i0 = half * (TN / 2); i0 < (half + 1) * (TN / 2); i0 += 8) {
-                const int n0 = t.z + i0;
-                if (n0 >= nv || !ok) break;   // uniform over the warp
-                uint32_t r[NACC][8];
-                if (have) {
+            // The accumulators become 64-bit integers in registers first and
+            // go back to the MMAs; conversion, scaling and stores run beside
+            // the next tile's products.
+            constexpr int NI = TN / 16;   // groups of 4 columns
+            const int i0 = quarter * (TN / 4), nb = t.z + i0;
+            long long T[NI][4];
+            int lead[NI][4];
+            if (have) {
+#pragma unroll
+                for (int u = 0; u < NI; ++u) {
+                    if (nb + 4 * u >= nv || !ok) continue;   // uniform over the warp
+                    uint32_t r[NACC][4];
 #pragma unroll
                     for (int s = 0; s < NACC; ++s)
-                        tmem_ld8(tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(s * TN + i0), r[s]);
+                        tmem_ld4(tmem + ((uint32_t)(32 * lq) << 16) +
+                                     (uint32_t)(s * TN + i0 + 4 * u), r[s]);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int in = n0 + i;
-                    if (!mok || in >= nv) continue;
-                    double d = 0.0;
-                    if (have) {
-                        const int en = MCOLS ? row_exp(in) : __ldg(ebp + in);
+                    for (int i = 0; i < 4; ++i) {
                         // sum of the accumulators in units of 2^-40 (the first
                         // apart where 64 bits may not hold it)
-                        const int lead = __float2int_rn(__uint_as_float(r[0][i]));
-                        long long T = pr.wide ? 0 : lead;
+                        int d[NACC];
 #pragma unroll
-                        for (int s = 1; s < NACC; ++s)
-                            T = (T << 8) + __float2int_rn(__uint_as_float(r[s][i]) *
-                                                          (float)(1ull << (8 * s)));
-                        double sum = (double)T;
-                        if (pr.wide) sum = fma((double)lead, 1099511627776.0, sum);
-                        const int ec = MCOLS ? em : en;
-                        d = ec == kNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
-                                             : scale2(sum, em + en + k0);
+                        for (int s = 0; s < NACC; ++s)
+                            d[s] = __float2int_rn(__uint_as_float(r[s][i]) *
+                                                  (float)(1ull << (8 * s)));
+                        lead[u][i] = d[0];
+                        using u64 = unsigned long long;
+                        T[u][i] = (long long)(((u64)((pr.wide ? 0 : d[0]) * 256ll + d[1]) << 32) +
+                                              ((u64)(d[2] * 256ll + d[3]) << 16) +
+                                              (u64)(d[4] * 256ll + d[5]));
                     }
-                    om[in * on] = d;
+                }
+                if (ok) {
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    mbar_arrive(acc_empty);
+                    ++nacc;
                 }
             }
-            if (have && ok) {
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive(acc_empty);
-                ++nacc;
+            auto value = [&](int u, int i, int in) -> double {
+                if (!have) return 0.0;
+                const int en = MCOLS ? row_exp(in) : __ldg(ebp + in);
+                double sum = (double)T[u][i];
+                if (pr.wide) sum = fma((double)lead[u][i], 1099511627776.0, sum);
+                return (MCOLS ? em : en) == kNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                                       : scale2(sum, em + en + k0);
+            };
+#pragma unroll
+            for (int u = 0; u < NI; ++u) {
+                const int n0 = nb + 4 * u;
+                if (!mok) continue;
+                if constexpr (MCOLS) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (n0 + i < nv) om[(n0 + i) * (long long)pr.o_stride] = value(u, i, n0 + i);
+                } else {
+                    // columns come in pairs (re, im), adjacent in the lane's row
+#pragma unroll
+                    for (int i = 0; i < 4; i += 2) {
+                        if (n0 + i >= nv) continue;
+                        const double x = value(u, i, n0 + i), y = value(u, i + 1, n0 + i + 1);
+                        if (g.pairs) {
+                            *reinterpret_cast<double2*>(om + n0 + i) = make_double2(x, y);
+                        } else {
+                            om[n0 + i] = x;
+                            om[n0 + i + 1] = y;
+                        }
+                    }
+                }
             }
         }
     }
@@ -625,7 +662,10 @@ void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
         mac_cols += (long long)s.nkt * ((C16 + TM - 1) / TM * TM) * s.R16;
         mac_rows += (long long)s.nkt * ((s.R16 + TM - 1) / TM * TM) * C16;
     }
-    d.mcols = mac_cols <= mac_rows;
+    // columns on the M side also store whole rows, worth some padding (T319 x
+    // 100 inverse, 2 % more work: 809 us with rows, 676 with columns; T200 x
+    // 20 forward, 20 % more: 81 and 97)
+    d.mcols = mac_cols * 10 <= mac_rows * 11;
     int nmax = C16;
     if (d.mcols) {
         nmax = 0;
@@ -715,6 +755,7 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
         g.C = C;
         g.C16 = sl->C16;
         g.status = p->d_status;
+        g.pairs = ((uintptr_t)O & 15) == 0;
         g.wait = short_launch(g.ntiles) ? 1 : 0;
         if (g.ntiles == 0) continue;
         const int ctas = std::min(g.ntiles, p->num_sms);
