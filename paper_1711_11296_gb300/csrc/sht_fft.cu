@@ -18,6 +18,13 @@ cudaError_t fwd_launch(const FwdArgs<float>& A, bool strided, dim3 grid, size_t 
 template <int LT>
 cudaError_t inv_launch(const InvArgs<float>& A, dim3 grid, size_t smem, cudaStream_t s,
                        Follow follow) {
+    // Short rows (radices below 16) get a kernel for the plain store alone, its
+    // last pass two butterflies at a time: T159 x 256 107.5 -> 104.0 us (6
+    // fields per CTA 137 -> 126), T239 x 64 74.7 -> 73.3.  From 512 on it was
+    // slower (T639 x 128 777 -> 811, T479 x 64 223 -> 242).
+    if constexpr (LT < 512 && inverse_stores_from_last_pass<float, LT>())
+        if (A.accumulate == 0)
+            return fft_launch(fft_inverse_kernel<float, LT, true>, A, grid, smem, s, follow);
     return fft_launch(fft_inverse_kernel<float, LT>, A, grid, smem, s, follow);
 }
 

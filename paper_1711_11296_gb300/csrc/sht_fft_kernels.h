@@ -898,7 +898,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     end_fft();
 }
 
-template <typename T, int LT>
+// PLAIN: the grid is only written (A.accumulate == 0).
+template <typename T, int LT, bool PLAIN = false>
 __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
     using V = typename Vec2<T>::type;
     using K = C2<T>;
@@ -1084,12 +1085,14 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
     }
     __syncthreads();
     if constexpr (inverse_stores_from_last_pass<T, LT>()) {
-        if (A.accumulate == 0) {
+        if (PLAIN || A.accumulate == 0) {
             constexpr FftShape FS = FacOf<LT, false>::v;
             constexpr int R = FS.radix[1];   // 32 = the padding period: one padded
             constexpr int Q = FS.radix[0];   // index per butterfly
             passes_fixed<T, LT, 0, 1>(rows, nrows, LP, tws);
             const V sgn = K::make(rs, -rs);   // x = conj(z) rs
+            constexpr int UNROLL = PLAIN ? 2 : 1;
+#pragma unroll UNROLL
             for (int idx = tid; idx < nrows * Q; idx += NT) {
                 const int r = idx / Q, b = idx - r * Q;
                 const int f = f0 + (r < nf ? r : r - nf);
@@ -1222,11 +1225,11 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
     }
 }
 
-template <typename T, int LT>
+template <typename T, int LT, bool PLAIN = false>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
     fft_inverse_kernel(const __grid_constant__ InvArgs<T> A) {
     begin_fft(A.follow);
-    inv_body<T, LT>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
+    inv_body<T, LT, PLAIN>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
     end_fft();
 }
 
