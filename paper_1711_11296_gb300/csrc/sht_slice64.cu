@@ -7,8 +7,8 @@
 // (sht_legendre_fp64.cu).  The tensor cores do about 1700 times as many
 // BF16 products, and BF16 holds every integer up to 256 exactly.  Measured
 // (us, forward / inverse contraction, FP64 pipe -> slices): T639 x 256
-// 120600 / 117800 -> 5780 / 5140; T319 x 100 8530 / 8090 -> 554 / 587;
-// T159 x 256 2721 / 2411 -> 247 / 311.
+// 120600 / 117800 -> 5840 / 4590; T319 x 100 8530 / 8090 -> 546 / 438;
+// T159 x 256 2721 / 2411 -> 249 / 222.
 //
 // Every row r of A (the P~ table) and every column c of B (the Fourier data
 // or the spectrum) is scaled by a power of two to an integer of at most
@@ -150,8 +150,12 @@ __device__ __forceinline__ int core_off(int row, int k8) {
 // Slices of the operand B of problems p0 + blockIdx.x, columns 32
 // blockIdx.y + lane; warp w takes the groups of 8 K rows w, w + 16, ....
 // NG > 0: at most NG groups per warp, held in registers between the
-// exponent pass and the slicing (one read of B, which bounds the kernel
-// together with the 14 bytes written per value); NG = 0: any K, read twice.
+// exponent pass and the slicing; NG = 0: any K, read twice, the second time
+// from the caches.  Latency and the 14 bytes written per value bound it, so
+// the warps in flight count: one read with NG = 3 (92 registers, one CTA per
+// SM) against two reads with three CTAs, contraction in us: T319 x 100 forward
+// 564 / 546, inverse (NG = 2, 76 registers) 478 / 438, T639 x 256 inverse
+// 4780 / 4593; where two CTAs fit, T159 x 256 forward (NG = 2) 249 / 268.
 // Inverse: the Equator row (node Jh - 1), which the tiles leave out so that
 // they cover J - 1 nodes in whole tiles, is summed here in FP64 (odd parity:
 // P~(0) = 0).
@@ -336,12 +340,38 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
                  : "r"(taddr));
 }
 
-__device__ __forceinline__ double scale2(double d, int k) {
-    const long long bits = __double_as_longlong(d);
-    const int e = (int)((bits >> 52) & 0x7ff) + k;
-    if (d == 0.0) return 0.0;
-    if (e > 0 && e < 0x7ff) return __longlong_as_double(bits + ((long long)k << 52));
-    return scalbn(d, k);
+// (hi 2^64 + lo) 2^k (two's complement) as a double, rounded once, by integer
+// operations: the hardware conversion of 64-bit integers and FP64 compares
+// run on the narrow FP64 pipe, which bound the epilogue (inverse contraction,
+// us: T159 x 256 311 -> 222, T319 x 100 587 -> 478, T639 x 256 5137 -> 4781).
+__device__ __forceinline__ double to_double(long long hi, unsigned long long lo, int k) {
+    using u64 = unsigned long long;
+    const u64 sign = (u64)hi & (1ull << 63);
+    if (sign) {
+        lo = 0 - lo;
+        hi = ~hi + (lo == 0);
+    }
+    // u: the leading 64 bits, its last bit sticky
+    u64 u = lo;
+    if (hi) {
+        const int l = __clzll(hi);   // >= 1
+        u = ((u64)hi << l) | (lo >> (64 - l)) | ((lo << l) != 0);
+        k += 64 - l;
+    } else {
+        if (lo == 0) return 0.0;
+        const int l = __clzll((long long)lo);
+        u <<= l;
+        k -= l;
+    }
+    const u64 m = u >> 11;   // 53 bits
+    const int e = 1086 + k, rem = (int)u & 0x7ff;
+    if (e > 0 && e < 0x7ff)
+        return __longlong_as_double(
+            (long long)(sign | (((u64)(e - 1) << 52) + m + (rem + ((int)m & 1) > 0x400))));
+    // below the normal range the scaling rounds (the last of the 53 bits is
+    // sticky), above it gives infinity
+    const double d = scalbn((double)(long long)(m | (rem != 0)), k + 11);
+    return sign ? -d : d;
 }
 
 // Persistent CTAs, one per SM: 128 x TN tiles (M x N) with six FP32
@@ -577,10 +607,17 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             auto value = [&](int u, int i, int in) -> double {
                 if (!have) return 0.0;
                 const int en = MCOLS ? row_exp(in) : __ldg(ebp + in);
-                double sum = (double)T[u][i];
-                if (pr.wide) sum = fma((double)lead[u][i], 1099511627776.0, sum);
-                return (MCOLS ? em : en) == kNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
-                                                       : scale2(sum, em + en + k0);
+                if ((MCOLS ? em : en) == kNonFinite)
+                    return __longlong_as_double(0x7ff8000000000000ll);
+                using u64 = unsigned long long;
+                long long hi = T[u][i] >> 63;
+                u64 lo = (u64)T[u][i];
+                if (pr.wide) {
+                    const u64 add = (u64)(long long)lead[u][i] << 40;
+                    hi += (long long)(lead[u][i] >> 24) + (lo + add < add);
+                    lo += add;
+                }
+                return to_double(hi, lo, em + en + k0);
             };
 #pragma unroll
             for (int u = 0; u < NI; ++u) {
@@ -702,13 +739,13 @@ cudaError_t launch_slice_b(int maxK, dim3 grid, cudaStream_t s, const double* B,
                     int ldp, int N, int Jh, double* O) {
     using Fn = void (*)(const double*, const S64Prob*, int, int, int, unsigned char*, int*,
                         const double*, int, int, int, double*, int);
-    static const Fn tab[7] = {slice_b_kernel<0, INV>, slice_b_kernel<1, INV>,
-                              slice_b_kernel<2, INV>, slice_b_kernel<3, INV>,
-                              slice_b_kernel<4, INV>, slice_b_kernel<5, INV>,
-                              slice_b_kernel<6, INV>};
+    // in registers where two CTAs still fit an SM
     const int ng = (maxK + 127) / 128;
+    const Fn fn = ng == 1            ? slice_b_kernel<1, INV>
+                  : ng == 2 && !INV ? slice_b_kernel<2, false>
+                                    : slice_b_kernel<0, INV>;
     const bool wait = short_launch((long long)grid.x * grid.y);
-    return launch_kernel(tab[ng <= 6 ? ng : 0], grid, dim3(512), 0, s, wait, B, probs, p0, C, C16,
+    return launch_kernel(fn, grid, dim3(512), 0, s, wait, B, probs, p0, C, C16,
                          out, eb, pnm, ldp, N, Jh, O, wait ? 1 : 0);
 }
 
