@@ -405,7 +405,12 @@ def roofline_for(name, tot_ms, n, w, F, prec, pk, pk_src, npts=None, grid="cc"):
             src = "nominal GB300 FP64 1.25 TFLOP/s (no FP64 probe in this run)"
         roof = {"kernel": name + "_fp64", "bound": "alu",
                 "achieved": fl / per_launch_s / 1e12, "peak": peak,
-                "unit": "TFLOP/s", "traffic": None, "peak_source": src}
+                "unit": "TFLOP/s", "traffic": None, "peak_source": src,
+                # 34 BF16 products of 8-bit slices per FP64 product
+                "tensor_frac": 34 * fl / per_launch_s / 1e12 / pk["bf16_tflops_sustained"],
+                "note": "FP64 flops against the FP64 pipe's rate; large contractions run "
+                        "as 34 BF16 products on the tensor cores (tensor_frac), so "
+                        "fractions above 1 are expected"}
     elif name.startswith("legendre"):
         # tensor-core products per split: x_a y_b with a + b < terms, less
         # x_2 y_2 for FP16 (weight 2^-22)
@@ -433,7 +438,8 @@ def roofline_for(name, tot_ms, n, w, F, prec, pk, pk_src, npts=None, grid="cc"):
             roof = {"kernel": name + "_f64", "bound": "alu",
                     "achieved": b / per_launch_s / 1e9, "peak": None,
                     "unit": "GB/s", "traffic": None,
-                    "peak_source": "FP64 pipe bound; HBM figure for context"}
+                    "peak_source": "integer pipes (64-bit fixed point); HBM "
+                                   "figure for context"}
         else:
             roof = {"kernel": name + "_f32", "bound": "hbm",
                     "achieved": b / per_launch_s / 1e9, "peak": pk["hbm_gbs"],
@@ -712,7 +718,7 @@ def native_arm(args):
     if prec != "fp64" and args.precision == "auto" and not args.no_fp64:
         import copy
         a64 = copy.copy(args)
-        a64.steps = min(args.steps, 10)      # the FP64 path is ~50x slower
+        a64.steps = min(args.steps, 10)      # the FP64 path is ~5x slower
         r64 = run_path(a64, w, F, "fp64", device, dist, local, rank, world, False,
                        a_host=a)
         n64, (t64, c64) = max(r64["prof"].items(), key=lambda kv: kv[1][0])
