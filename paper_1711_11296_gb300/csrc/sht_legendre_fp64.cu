@@ -205,12 +205,13 @@ cudaError_t launch_small(const sht_plan_s* p, bool inverse, const double* in, do
 }  // namespace
 
 // us of the forward + inverse contraction, slices -> a thread per output: T31 x
-// 10 44 -> 22, T63 x 20 51 -> 39, T95 x 16 74 -> 72, T127 x 4 63 -> 57, T159 x 4
-// 103 -> 93; beyond 3e7 flops T63 x 64 62 -> 78, T200 x 4 128 -> 145, except for
-// one field, whose 2 columns fill an eighth of an MMA: T319 x 1 290 -> 179,
-// T639 x 1 1311 -> 1133.  (The tiles: T31 x 1 45, here 18.)
+// 10 30 -> 23, T63 x 20 40 -> 39, T95 x 8 51 -> 50, T127 x 2 55 -> 43; from
+// 1.5e7 flops on T127 x 4 56 -> 57, T95 x 16 55 -> 72, T159 x 4 96 -> 100, T63
+// x 64 47 -> 78, T200 x 4 116 -> 143, except for one field, whose 2 columns
+// fill an eighth of an MMA: T319 x 1 274 -> 178, T639 x 1 1260 -> 1137.  (The
+// tiles: T31 x 1 45, here 18.)
 bool legendre_small(const sht_plan_s* p) {
-    return p->F == 1 || 4.0 * (double)p->ncoef * p->Jh * p->F <= 3e7;
+    return p->F == 1 || 4.0 * (double)p->ncoef * p->Jh * p->F <= 1.5e7;
 }
 
 // Tile lists (host): forward tiles cover the parity rows of each (m, q);
