@@ -392,9 +392,12 @@ cudaError_t launch_fft_inverse_group(sht_plan_s* const* plans, int n,
 // (with_radix), with the least estimated time: per pass and value 14
 // instructions of shared-memory traffic, twiddles and addresses plus the
 // DFT's own, over the share of the CTA's threads that have a butterfly in
-// the rounds of its (nominal) rows.  Two or three passes of large radices
-// then replace up to five of 2 .. 8.
-FftShape fft_shape(int L, bool fp64, bool compile_time, float* time) {
+// the rounds of its rows.  Two or three passes of large radices then replace
+// up to five of 2 .. 8; with few fields (and so rows) in a CTA, small radices
+// keep its threads busy (forward / inverse us, L = 288 x 1 field: 12 24
+// 18.3 / 16.4, 3 4 4 6 14.7 / 12.3; L = 900 x 1: 30 30 29.9 / 29.1, 9 10 10
+// 25.1 / 22.2).
+FftShape fft_shape(int L, bool fp64, bool compile_time, float* time, int F) {
     if (time) *time = 0.f;
     if (fp64 || L == 1 || compile_time) return fft_factor(L, fp64);
     struct Size { int r; float work; };   // instructions of the DFT per value
@@ -402,7 +405,7 @@ FftShape fft_shape(int L, bool fp64, bool compile_time, float* time) {
                                  {9, 7.8f}, {10, 8.6f}, {12, 7.5f}, {15, 11.f}, {16, 7.3f},
                                  {20, 10.9f}, {24, 10.3f}, {25, 14.6f}, {30, 14.f}, {32, 10.1f}};
     int g = 16;
-    while (g > 1 && fft_smem_bytes(2 * L, g, false) > 112 * 1024) g /= 2;
+    while (g > 1 && (g > F || fft_smem_bytes(2 * L, g, false) > 112 * 1024)) g /= 2;
     auto cost = [&](const Size& z) {
         const int n = 2 * g * (L / z.r), rounds = (n + kFftThreads - 1) / kFftThreads;
         return (14.f + z.work) * (float)(rounds * kFftThreads) / (float)n;

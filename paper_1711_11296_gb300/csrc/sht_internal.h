@@ -334,7 +334,8 @@ __host__ __device__ constexpr FftShape fft_factor(int L, bool fp64) {
 // of the length will run, else passes of the register DFT sizes that the
 // kernels with run-time shapes hold (2 .. 32).
 // time: the estimate the choice was made by (0 where there was none).
-FftShape fft_shape(int L, bool fp64, bool compile_time, float* time = nullptr);
+// F: the plan's fields.
+FftShape fft_shape(int L, bool fp64, bool compile_time, float* time = nullptr, int F = 16);
 
 __host__ __device__ constexpr bool fft_factorable(int L) {
     return L == 1 || fft_factor(L, true).npass > 0;

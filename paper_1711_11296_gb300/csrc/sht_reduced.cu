@@ -163,7 +163,7 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
                 dft_total += r.sh.L;
                 L2max = std::max(L2max, r.sh.L);
             } else {
-                r.sh = fft_shape(L, fp64, route == kRouteClass);
+                r.sh = fft_shape(L, fp64, route == kRouteClass, nullptr, p->F);
             }
             r.tw_off = tw_total;
             r.post_off = post_total;
