@@ -253,6 +253,31 @@ __device__ __forceinline__ void grid_trigger() {
 __device__ __forceinline__ void grid_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// What another kernel writes, read after grid_wait.  A dependent launch may be
+// resident while that kernel still writes, so these operands are not read-only
+// for its whole life: __ldg, and the read-only loads that the compiler makes of
+// const __restrict__ parameters, are for the plan's own tables.  (The asm is
+// volatile, so it stays behind the wait.)
+__device__ __forceinline__ double ld_dep(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_dep(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld_dep(const int* p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned ld_dep(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 #endif
 
 struct ProfScope {

@@ -162,9 +162,8 @@ __global__ void __launch_bounds__(NT) legendre_inv_fp64_kernel(
 // slices take two launches and whole 16-column MMAs; here a K step is one
 // product per output, bound by the FP64 pipe and, below it, by latency.
 __global__ void __launch_bounds__(128) legendre_small_fp64_kernel(
-    const double* __restrict__ pnm, int ldp, const double* __restrict__ in,
-    double* __restrict__ out, int N, int Jh, int C, const int* __restrict__ jmin, int inverse,
-    int wait) {
+    const double* __restrict__ pnm, int ldp, const double* in, double* __restrict__ out, int N,
+    int Jh, int C, const int* __restrict__ jmin, int inverse, int wait) {
     grid_trigger();
     if (wait) grid_wait();
     const int m = blockIdx.x >> 1, q = blockIdx.x & 1;
@@ -181,14 +180,14 @@ __global__ void __launch_bounds__(128) legendre_small_fp64_kernel(
         const double* A = P + 2 * (size_t)row * ldp;
 #pragma unroll 8
         for (int k = jmin ? (jmin[2 * m + q] / BK) * BK : 0; k < Jh; ++k)
-            acc = fma(__ldg(A + k), __ldg(B + (size_t)k * C), acc);
+            acc = fma(__ldg(A + k), ld_dep(B + (size_t)k * C), acc);
         out[(row0 + 2 * (size_t)row) * C + c] = acc;
     } else {
         const double* B = in + row0 * C + c;
         const int kend = (jmin && row / BM * BM + BM <= jmin[2 * m + q]) ? 0 : R;
 #pragma unroll 8
         for (int k = 0; k < kend; ++k)
-            acc = fma(__ldg(P + 2 * (size_t)k * ldp + row), __ldg(B + 2 * (size_t)k * C), acc);
+            acc = fma(__ldg(P + 2 * (size_t)k * ldp + row), ld_dep(B + 2 * (size_t)k * C), acc);
         out[(wrow + row) * C + c] = acc;
     }
 }

@@ -161,7 +161,7 @@ __device__ __forceinline__ int core_off(int row, int k8) {
 // P~(0) = 0).
 template <int NG, bool INV>
 __global__ void __launch_bounds__(512)
-    slice_b_kernel(const double* __restrict__ B, const S64Prob* __restrict__ probs, int p0, int C,
+    slice_b_kernel(const double* B, const S64Prob* __restrict__ probs, int p0, int C,
                    int C16, unsigned char* __restrict__ out, int* __restrict__ eb,
                    const double* __restrict__ pnm, int ldp, int N, int Jh,
                    double* __restrict__ O, int wait) {
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(512)
     const bool cin = c < C;
     const double* col = B + pr.src_off + c;
     auto load = [&](int k) -> double {
-        return (k < pr.K && cin) ? __ldg(col + (long long)k * pr.src_stride) : 0.0;
+        return (k < pr.K && cin) ? ld_dep(col + (long long)k * pr.src_stride) : 0.0;
     };
     const int ng = 2 * pr.nkt;
     double v[NG > 0 ? 8 * NG : 8];
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             const int* ebp = g.eb + (size_t)t.x * g.C16;
             const int* eap = g.ea + pr.ea_off;
             auto row_exp = [&](int r) { return max(__ldg(eap + r), 1) - 1022; };
-            const int em = mok ? (MCOLS ? __ldg(ebp + im) : row_exp(im)) : 0;
+            const int em = mok ? (MCOLS ? ld_dep(ebp + im) : row_exp(im)) : 0;
             double* om = g.O + pr.o_off + (MCOLS ? (long long)im : (long long)im * pr.o_stride);
             const int k0 = 56 - 2 * pr.sh;
             // The accumulators become 64-bit integers in registers first and
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             }
             auto value = [&](int u, int i, int in) -> double {
                 if (!have) return 0.0;
-                const int en = MCOLS ? row_exp(in) : __ldg(ebp + in);
+                const int en = MCOLS ? row_exp(in) : ld_dep(ebp + in);
                 if ((MCOLS ? em : en) == kNonFinite)
                     return __longlong_as_double(0x7ff8000000000000ll);
                 using u64 = unsigned long long;

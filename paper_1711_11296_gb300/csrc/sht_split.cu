@@ -569,7 +569,7 @@ __device__ __forceinline__ void split_gemm_body(const Args& args, const int4* __
             float cs = 1.f;
             if (F16) {
                 const int cg = cbase + tid % TN;
-                if (cg < g.C) cs = col_scale(g.colmax[cg]);
+                if (cg < g.C) cs = col_scale(ld_dep(g.colmax + cg));
             }
             // Thread tid converts column c, K rows k8 * 8 .. + 7 of each
             // stage (threads past TN * TK / 8 only take part in the
@@ -598,7 +598,7 @@ __device__ __forceinline__ void split_gemm_body(const Args& args, const int4* __
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
                         x[e] = (cin && k + e < pr.K)
-                                   ? __ldg(g.B + pr.b_off + (long long)(k + e) * pr.b_stride + cg)
+                                   ? ld_dep(g.B + pr.b_off + (long long)(k + e) * pr.b_stride + cg)
                                    : 0.f;
                 }
                 return true;
@@ -666,7 +666,7 @@ __device__ __forceinline__ void split_gemm_body(const Args& args, const int4* __
                 // rows n.  For each row the 32 lanes store 32 adjacent columns.
                 const int c = cbase + 32 * lq + lane;
                 const bool col_ok = c < g.C && ok && !*abort_flag;
-                const float csi = (F16 && c < g.C) ? col_unscale(g.colmax[c]) : 0.f;
+                const float csi = (F16 && c < g.C) ? col_unscale(ld_dep(g.colmax + c)) : 0.f;
                 constexpr int NCH = TN / 16 / (NCONV / 128);
                 for (int cc = 0; cc < NCH; ++cc) {
                     const int ch = half * NCH + cc;
@@ -731,7 +731,7 @@ __device__ __forceinline__ void split_gemm_body(const Args& args, const int4* __
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
                                 const float csi =
-                                    c0 + i < g.C ? col_unscale(g.colmax[c0 + i]) : 0.f;
+                                    c0 + i < g.C ? col_unscale(ld_dep(g.colmax + c0 + i)) : 0.f;
                                 r[i] = __float_as_uint((__uint_as_float(r[i]) +
                                                         __uint_as_float(r2[i]) * (1.f / 2048.f)) *
                                                        rsi * csi);
@@ -836,8 +836,8 @@ __device__ __forceinline__ void two_sum_acc(float& h, float& l, float a, float a
 
 template <int T, bool F16, int TN>
 __global__ void __launch_bounds__(256)
-    split_b_kernel(const float* __restrict__ B, const SplitProb* __restrict__ probs, int C,
-                   int nct, const unsigned* __restrict__ colmax, unsigned char* planes,
+    split_b_kernel(const float* B, const SplitProb* __restrict__ probs, int C,
+                   int nct, const unsigned* colmax, unsigned char* planes,
                    long long plane_bytes, const double* __restrict__ pnm, int ldp, int N,
                    int Jh, float* __restrict__ O, int wait) {
     constexpr int B_TILE_BYTES = Wid<TN>::B_TILE_BYTES;
@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(256)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int c = blockIdx.y * 128 + (w & 3) * 32 + lane;
     const bool cin = c < C;
-    const float cs = (F16 && cin) ? col_scale(colmax[c]) : 1.f;
+    const float cs = (F16 && cin) ? col_scale(ld_dep(colmax + c)) : 1.f;
     const int ct = c / TN, cc = c % TN;
     float eh = 0.f, el = 0.f;
     for (int g = w >> 2; g < pr.nkt * (TK / 8); g += 2) {
@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = g * 8 + e;
-            x[e] = (k < pr.K && cin) ? __ldg(B + pr.b_off + (long long)k * pr.b_stride + c)
+            x[e] = (k < pr.K && cin) ? ld_dep(B + pr.b_off + (long long)k * pr.b_stride + c)
                                      : 0.f;
         }
         if (even) {
