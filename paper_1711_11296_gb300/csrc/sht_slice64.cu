@@ -7,21 +7,38 @@
 // (sht_legendre_fp64.cu).  The tensor cores do about 1700 times as many
 // BF16 products, and BF16 holds every integer up to 256 exactly.  Measured
 // (us, forward / inverse contraction, FP64 pipe -> slices): T639 x 256
-// 120600 / 117800 -> 5840 / 4590; T319 x 100 8530 / 8090 -> 546 / 438;
-// T159 x 256 2721 / 2411 -> 249 / 222.
+// 120600 / 117800 -> 6070 / 4720; T319 x 100 8530 / 8090 -> 558 / 445;
+// T159 x 256 2721 / 2411 -> 254 / 225.
 //
 // Every row r of A (the P~ table) and every column c of B (the Fourier data
-// or the spectrum) is scaled by a power of two to an integer of at most
-// 2^sh (sh = 53..55, more bits than the 53 of the input for all but the
-// entries far below their row's or column's largest), written with seven
-// digits d_0 .. d_6 in [-128, 128], value = sum_a d_a 256^(6 - a).  Digit a
-// is stored as the BF16 number d_a 2^(-8a) in slice a.  A product of two
-// slices sums integers below 2^24 in the FP32 accumulators, which is exact;
-// the products of equal a + b share an accumulator:
+// or the spectrum) is scaled by a power of two to an integer of at most 2^sh (sh =
+// 55; 54 and 53 for sums of more than 1000 and 4000 products), written with seven
+// digits d_0 .. d_6 in [-128, 128], value = sum_a d_a 256^(6 - a).  An entry 2^-k
+// of its row's or column's largest so keeps sh - k bits, an error of at most 2^-56
+// of the largest at sh = 55; those within 2^-2 of it keep all 53.  Digit a is
+// stored as the BF16 number d_a 2^(-8a) in slice a.  The products of equal a + b
+// share an FP32 accumulator:
 //   a + b = 0, 1, 2, 3, 4 | 5, 6, 7 together,
 // 34 products of the 49 (the 15 left out are below 2^-60 of row times
-// column maximum, under the rounding of the operands).  The last
-// accumulator rounds at 2^-24 of its leading term, 2^-62 of the maxima.
+// column maximum, under the rounding of the operands).
+//
+// The first five accumulators sum integers, exactly as long as these stay
+// within 2^24.  Digits of ordinary data average out far below that, but those of
+// a constant column and of the constant P~_0^0 do not (over the 776 nodes of
+// T774 they reached 1.3 2^24, and the result was rounded at 6.6e-10).  So a
+// tile's K slabs come in segments.  Accumulator a + b = s grows by at most
+//   128 sum_k (|d_0| + .. + |d_s|) <= 128 sum_k (|d_0| + .. + |d_4|)
+// of A's digits, whatever B holds, and table_segment_kernel ends a segment, when
+// the plan is made, before any row's bound would pass 2^24 less what a carry
+// leaves: after 12 slabs of 16 at the least, usually after about 25.  Between
+// two segments the epilogue's warps carry: what accumulators 1 .. 4 hold beyond
+// their own digit is added to the one before.  The first then holds the whole
+// sum to within 2^9, at most K 2^(2 sh - 96), which sh keeps below 2^24.  The
+// segments cost T639 x 256 5850 -> 6070 us forward (two a tile) and 4600 ->
+// 4720 inverse, T319 x 100 547 -> 558 and 440 -> 445, T159 x 256 250 -> 254 and
+// 222 -> 225 (one: the registers alone).
+//
+// The last accumulator rounds at 2^-24 of its leading term, 2^-62 of the maxima.
 // The epilogue adds the six sums as a 64-bit integer, converts it once and
 // scales it back, so an output carries the operands' rounding (2^-56 of the
 // row and column maxima) and one final rounding: less than the sum of K
@@ -44,6 +61,10 @@
 namespace sht {
 
 constexpr int kSlices = 7;
+constexpr int kMaxJh = 4096;        // longest K
+// segments of a problem, each of (2^24 - 2^16 - 2^7) / (5 128^2) = 203 or more K
+// rows: 12 slabs
+constexpr int kMaxSeg = kMaxJh / 16 / 12 + 1;
 
 struct S64Prob {
     long long a_off;     // byte offset of the problem's A slices in the table
@@ -54,7 +75,8 @@ struct S64Prob {
     int K, nkt;          // depth, and its K slabs of 16
     int src_stride, o_stride;
     int ea_off;          // first row in the exponent table
-    int sh;              // operands are scaled below 2^sh
+    int sh;              // operands are integers of at most 2^sh
+    int end0;            // end of the first segment (table_segment_kernel)
     int wide;            // the sum of the accumulators may need more than 63 bits
 };
 
@@ -66,6 +88,7 @@ struct S64Dir {
     int tn = 80;                    // N width of the tiles
     unsigned char* table = nullptr; // A slices: per problem [K slab][slice][R16][16]
     int* ea = nullptr;              // exponent of every row of A
+    int* seg = nullptr;             // [problem][kMaxSeg]: last K slab + 1 of its segments
     S64Prob* d_probs = nullptr;
     int4* d_tiles = nullptr;        // {problem, m0, n0, -}
     std::vector<S64Chunk> chunks;
@@ -315,6 +338,71 @@ __global__ void table_slice_kernel(const double* __restrict__ pnm, int ldp, int 
     }
 }
 
+// Ends of the K segments of every problem (see the top): the longest that keep
+// 128 sum_k (|d_0| + .. + |d_4|) within 2^24 for every row, less the 2^16 + 2^7
+// that a carry may leave in an accumulator.  One CTA per problem,
+// a warp per row (forward) or a thread per row (inverse), as in
+// table_exp_kernel.
+__global__ void table_segment_kernel(const double* __restrict__ pnm, int ldp, int N,
+                                     S64Prob* probs, int inverse, const int* __restrict__ ea,
+                                     int* __restrict__ seg) {
+    constexpr int LIM = ((1 << 24) - (1 << 16) - 128) / 128;
+    __shared__ int end;
+    const int p = blockIdx.x;
+    const S64Prob pr = probs[p];
+    const double* P = pnm + (coef_offset(N, p >> 1) + (p & 1)) * ldp;
+    auto digits = [&](int r, int k) -> int {
+        if (k >= pr.K) return 0;
+        const double v = inverse ? P[2 * (size_t)k * ldp + r] : P[2 * (size_t)r * ldp + k];
+        const long long x = bias(to_fixed(v, ea[pr.ea_off + r], pr.sh));
+        int sum = abs((int)((x >> 48) & 0x1ff) - 128);
+#pragma unroll
+        for (int a = 1; a < 5; ++a) sum += abs((int)((x >> (8 * (6 - a))) & 0xff) - 128);
+        return sum;
+    };
+    int n = 0;
+    for (int q0 = 0; q0 < pr.nkt; ++n) {
+        if (threadIdx.x == 0) end = pr.nkt;
+        __syncthreads();
+        if (!inverse) {
+            const int lane = threadIdx.x & 31;
+            for (int r = threadIdx.x >> 5; r < pr.R; r += blockDim.x >> 5) {
+                int sum = 0;
+                // two slabs at a time, eight loaded together
+                for (int q = q0; q < pr.nkt && sum <= LIM; q += 8) {
+                    int w[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) w[i] = digits(r, (q + 2 * i) * TK + lane);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const bool in = sum <= LIM;
+                        sum += __reduce_add_sync(0xffffffffu, w[i]);
+                        if (in && sum > LIM && lane == 0) atomicMin(&end, q + 2 * i);
+                    }
+                }
+            }
+        } else {
+            for (int r = threadIdx.x; r < pr.R; r += blockDim.x) {
+                int sum = 0;
+                for (int q = q0; q < pr.nkt; ++q) {
+                    for (int e = 0; e < TK; ++e) sum += digits(r, q * TK + e);
+                    if (sum > LIM) {
+                        atomicMin(&end, q);
+                        break;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        q0 = end;
+        if (threadIdx.x == 0) {
+            seg[(size_t)p * kMaxSeg + n] = q0;
+            if (n == 0) probs[p].end0 = q0;
+        }
+        __syncthreads();   // end is written again only after all have read it
+    }
+}
+
 // ---- the product ------------------------------------------------------------
 
 struct S64Args {
@@ -326,6 +414,7 @@ struct S64Args {
     double* O;
     const int* ea;
     const int* eb;
+    const int* seg;
     const int* jmin;   // reduced transform (Sec. 4.1): first significant node per problem
     int inverse;
     int C, C16;
@@ -338,6 +427,11 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr),
+                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]));
 }
 
 // (hi 2^64 + lo) 2^k (two's complement) as a double, rounded once, by integer
@@ -388,12 +482,12 @@ __device__ __forceinline__ double to_double(long long hi, unsigned long long lo,
 // 32 the narrower configuration's deeper ring is faster (T200 x 20: TN = 80
 // 100 / 119, 64 94 / 110).
 // Six accumulators leave no room for a second set, so the MMAs wait while the
-// epilogue reads them: it only forms the 64-bit sums in registers (60 a
-// thread) before it hands them back, and converts, scales and stores beside
-// the next tile's products.  With 16 warps against 8, and the sums by 32-bit
-// multiply-adds: T639 x 256 6660 / 7500 -> 5780 / 5140, T319 x 100 685 / 845
-// -> 554 / 587, T159 x 256 316 / 362 -> 247 / 311 (8 warps alone 5820 / 5550,
-// 562 / 676, 259 / 338).
+// epilogue reads them (or carries, between segments): it only forms the 64-bit
+// sums in registers (60 a thread) before it hands them back, and converts,
+// scales and stores beside the next tile's products.  With 16 warps against 8,
+// and the sums by 32-bit multiply-adds: T639 x 256 6660 / 7500 -> 5780 / 5140,
+// T319 x 100 685 / 845 -> 554 / 587, T159 x 256 316 / 362 -> 247 / 311 (8 warps
+// alone 5820 / 5550, 562 / 676, 259 / 338).
 template <bool MCOLS, int TN>
 __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant__ S64Args g) {
     using CF = Cfg<TN>;
@@ -512,9 +606,16 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
                 const int hn = min(TN, (MCOLS ? pr.R16 : g.C16) - t.z);
                 const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
                                        ((uint32_t)(hn >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-                if (nacc > 0 && !(ok = mbar_wait(acc_empty, (nacc - 1) & 1u, abort_flag))) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int li = 0; li < nst; ++li, ++q) {
+                const int* seg = g.seg + (size_t)t.x * kMaxSeg;
+                int end = pr.end0;
+                while (end <= kb) end = *++seg;   // (the last ends at nkt > kb)
+                bool first = true;                // of its segment
+                for (int kt = kb; kt < pr.nkt; ++kt, ++q) {
+                    if (first) {
+                        if (nacc > 0 && !(ok = mbar_wait(acc_empty, (nacc - 1) & 1u, abort_flag)))
+                            break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
                     const int s = q % NSTAGE;
                     if (!(ok = mbar_wait(full(s), (q / NSTAGE) & 1u, abort_flag))) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -528,16 +629,20 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
                             if (a + b > 7) continue;
                             const int acc = a + b < NACC ? a + b : NACC - 1;
                             // (0, b) opens accumulator b
-                            const uint32_t add = (li > 0 || !(a == 0 && b < NACC)) ? 1u : 0u;
+                            const uint32_t add = (kt > kb || !(a == 0 && b < NACC)) ? 1u : 0u;
                             mma_f16_rt(tmem + acc * TN, md + (uint64_t)(a * M_SLICE / 16),
                                        nd + (uint64_t)(b * N_SLICE / 16), idesc, add);
                         }
                     }
                     mma_commit(empty(s));
+                    first = kt + 1 == end;
+                    if (first) {
+                        mma_commit(done);
+                        ++nacc;
+                        if (end < pr.nkt) end = *++seg;
+                    }
                 }
                 if (!ok) break;
-                mma_commit(done);
-                ++nacc;
             }
             mma_commit(fin);
         }
@@ -553,11 +658,58 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             int kb;
             const int nst = range(pr, t, kb);
             const bool have = nst > 0;
-            if (have) ok = mbar_wait(done, nacc & 1u, abort_flag);
-            ok = __all_sync(0xffffffffu, ok) != 0;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            constexpr int NI = TN / 16;   // groups of 4 columns
+            const int i0 = quarter * (TN / 4), nb = t.z + i0;
+            const int nv = MCOLS ? pr.R : g.C;
+            const uint32_t acc = tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)i0;
+            // wait for the accumulators of a segment
+            auto take = [&]() {
+                ok = mbar_wait(done, nacc & 1u, abort_flag);
+                ok = __all_sync(0xffffffffu, ok) != 0;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            };
+            auto hand_back = [&]() {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                mbar_arrive(acc_empty);
+                ++nacc;
+            };
+            // at the end of each segment but the last, carry (see the top)
+            const int* seg = g.seg + (size_t)t.x * kMaxSeg;
+            int end = pr.end0;
+            while (have && end <= kb) end = *++seg;
+            for (; have && ok && end < pr.nkt; end = *++seg) {
+                take();
+                if (!ok) break;
+#pragma unroll
+                for (int u = 0; u < NI; ++u) {
+                    if (nb + 4 * u >= nv) continue;   // uniform over the warp
+                    uint32_t r[NACC - 1][4];
+#pragma unroll
+                    for (int s = 0; s < NACC - 1; ++s)
+                        tmem_ld4(acc + (uint32_t)(s * TN + 4 * u), r[s]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                        for (int s = 1; s < NACC - 1; ++s) {
+                            // to the nearest multiple of the unit of s - 1
+                            const float a = __uint_as_float(r[s][i]);
+                            const float big = 12582912.f / (float)(1ull << (8 * (s - 1)));
+                            const float c = (a + big) - big;
+                            r[s - 1][i] = __float_as_uint(__uint_as_float(r[s - 1][i]) + c);
+                            r[s][i] = __float_as_uint(a - c);
+                        }
+                    }
+#pragma unroll
+                    for (int s = 0; s < NACC - 1; ++s)
+                        tmem_st4(acc + (uint32_t)(s * TN + 4 * u), r[s]);
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                hand_back();
+            }
+            if (have && ok) take();
             const int im = t.y + 32 * lq + lane;           // this lane's M index
-            const int mv = MCOLS ? g.C : pr.R, nv = MCOLS ? pr.R : g.C;
+            const int mv = MCOLS ? g.C : pr.R;
             const bool mok = im < mv && ok;
             const int* ebp = g.eb + (size_t)t.x * g.C16;
             const int* eap = g.ea + pr.ea_off;
@@ -568,8 +720,6 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
             // The accumulators become 64-bit integers in registers first and
             // go back to the MMAs; conversion, scaling and stores run beside
             // the next tile's products.
-            constexpr int NI = TN / 16;   // groups of 4 columns
-            const int i0 = quarter * (TN / 4), nb = t.z + i0;
             long long T[NI][4];
             int lead[NI][4];
             if (have) {
@@ -579,8 +729,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
                     uint32_t r[NACC][4];
 #pragma unroll
                     for (int s = 0; s < NACC; ++s)
-                        tmem_ld4(tmem + ((uint32_t)(32 * lq) << 16) +
-                                     (uint32_t)(s * TN + i0 + 4 * u), r[s]);
+                        tmem_ld4(acc + (uint32_t)(s * TN + 4 * u), r[s]);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -598,11 +747,7 @@ __global__ void __launch_bounds__(NT, 1) slice_gemm_kernel(const __grid_constant
                                               (u64)(d[4] * 256ll + d[5]));
                     }
                 }
-                if (ok) {
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    mbar_arrive(acc_empty);
-                    ++nacc;
-                }
+                if (ok) hand_back();
             }
             auto value = [&](int u, int i, int in) -> double {
                 if (!have) return 0.0;
@@ -682,10 +827,11 @@ void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
         s.K = inverse ? Rn : Jh;
         s.R16 = (s.R + 15) / 16 * 16;
         s.nkt = (s.K + TK - 1) / TK;
-        // K products of the leading digits (up to 2^(sh - 48)) fit the 24
-        // bits that FP32 adds exactly; the six accumulators fit one 64-bit
+        // K products of the operands are at most K 2^(2 sh - 96) in the first
+        // accumulator's units, within the 2^24 that FP32 adds exactly (the
+        // others: table_segment_kernel); the sum of the six fits a 64-bit
         // integer (K 2^14 2^40 and the rest below 2^63) up to K = 480
-        s.sh = s.K <= 1024 ? 55 : 54;
+        s.sh = s.K <= 1000 ? 55 : s.K <= 4000 ? 54 : 53;
         s.wide = s.K > 480;
         s.src_off = inverse ? row0 * C : (long long)p * Jh * C;
         s.src_stride = inverse ? 2 * C : C;
@@ -787,6 +933,7 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
         g.O = O;
         g.ea = d.ea;
         g.eb = sl->eb;
+        g.seg = d.seg;
         g.jmin = p->d_jmin;
         g.inverse = inverse ? 1 : 0;
         g.C = C;
@@ -808,7 +955,7 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
 // legendre_small); without the memory for them the plan stays on the FP64
 // pipe.
 cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
-    if (legendre_small(p) || p->Jh > 4096) return cudaSuccess;
+    if (legendre_small(p) || p->Jh > kMaxJh) return cudaSuccess;
     Slice64* sl = new (std::nothrow) Slice64();
     if (!sl) return cudaSuccess;
     p->slice = sl;
@@ -822,6 +969,7 @@ cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
         S64Dir& d = sl->dir[i];
         e = cudaMalloc(&d.table, (size_t)h[i].table_bytes + 16);
         if (e == cudaSuccess) e = cudaMalloc(&d.ea, (size_t)(h[i].ea_rows + 1) * sizeof(int));
+        if (e == cudaSuccess) e = cudaMalloc(&d.seg, (size_t)nprob * kMaxSeg * sizeof(int));
         if (e == cudaSuccess) e = cudaMalloc(&d.d_probs, nprob * sizeof(S64Prob));
         if (e == cudaSuccess) e = cudaMalloc(&d.d_tiles, (h[i].tiles.size() + 1) * sizeof(int4));
     }
@@ -841,6 +989,8 @@ cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
         table_exp_kernel<<<nprob, 256, 0, s>>>(p->d_pnm, p->ldp, p->N, d.d_probs, i, d.ea);
         table_slice_kernel<<<dim3(nprob, 8), 256, 0, s>>>(p->d_pnm, p->ldp, p->N, d.d_probs, i,
                                                          d.ea, d.table);
+        table_segment_kernel<<<nprob, 256, 0, s>>>(p->d_pnm, p->ldp, p->N, d.d_probs, i, d.ea,
+                                                   d.seg);
         e = cudaGetLastError();
     }
     // (the host lists above must outlive the copies)
@@ -854,7 +1004,7 @@ void slice64_destroy(sht_plan_s* p) {
     if (sl->bbuf) cudaFree(sl->bbuf);
     if (sl->eb) cudaFree(sl->eb);
     for (S64Dir& d : sl->dir) {
-        void* ptrs[] = {d.table, d.ea, d.d_probs, d.d_tiles};
+        void* ptrs[] = {d.table, d.ea, d.seg, d.d_probs, d.d_tiles};
         for (void* q : ptrs)
             if (q) cudaFree(q);
     }

@@ -98,3 +98,42 @@ def test_non_finite_fields_stay_apart(sht, bad):
     keep = [f for f in range(F) if f != 2]
     np.testing.assert_array_equal(got[keep], good[keep])
     assert not np.isfinite(got[2]).any()
+
+
+# Constant fields: the column's digits are then the same at every node, as are
+# those of P~_0^0, and the products' sums do not average out (N = 774 with J =
+# 2 N + 3 is the worst of the truncations 303 .. 1023 for the cotangent of a
+# mean; J = 2301 has more than 1024 nodes).  Tolerance: an exact sum has the
+# operands' rounding, 2^-56 of the maxima for each of K <= 1151 terms of one
+# sign, and the FFT's (2e-16); 1e-13 is far above both.
+@pytest.mark.parametrize("N,J,I,F,c", [
+    (774, 1551, 1600, 2, None), (928, 1859, 1920, 2, None), (639, 1281, 1280, 2, 0.949412),
+    (639, 1281, 1280, 2, 0.98831), (100, 2301, 216, 4, None), (100, 2301, 216, 4, 0.949412),
+])
+def test_constant_fields(sht, N, J, I, F, c):
+    p = sht.Plan(N, J, I, F, "fp64")
+    c = 1.0 / (J * I) if c is None else c
+    noise = np.random.default_rng(2500 + N).standard_normal((J, I)) * (1e-6 * c)
+    x = np.stack([np.full((J, I), c), c + noise] + [np.full((J, I), -3.0 * c)] * (F - 2))
+    got = p.adjoint(1, to_cuda(x, torch.float64)).cpu().numpy()
+    p.status()
+    # X_0^0 = sum over the points x P~_0^0, in extended precision
+    ref = x.astype(np.longdouble).sum(axis=(1, 2)) * np.sqrt(np.longdouble(0.5))
+    assert np.abs(got[0] / ref.astype(np.float64) - 1.0).max() <= 1e-13
+
+
+# The segments of a long sum: fields whose digits are random, so that the whole
+# range of rows and columns is summed, against the oracle.
+@pytest.mark.parametrize("N,J,I,F", [
+    (20, 2051, 48, 40),     # 1026 nodes: three segments of a forward sum
+    (20, 8191, 48, 12),     # 4096 nodes, the most that are sliced
+    (340, 700 + 1, 720, 3), # two segments forward, one inverse
+])
+def test_long_sums(sht, N, J, I, F):
+    p = sht.Plan(N, J, I, F, "fp64")
+    x = W.random_grid(F, J, I, seed=2600 + J)
+    a = W.random_spectrum(N, F, "flat", seed=2700 + J)
+    assert_fp64_close(p.forward(to_cuda(x, torch.float64)).cpu().numpy(), O.analysis(x, N))
+    assert_fp64_close(p.inverse(to_cuda(a, torch.complex128)).cpu().numpy(),
+                      O.synthesis(a, N, J, I))
+    p.status()
