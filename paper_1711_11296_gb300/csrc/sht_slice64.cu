@@ -170,7 +170,7 @@ __device__ __forceinline__ int core_off(int row, int k8) {
     return ((row >> 3) * 2 + k8) * 128 + (row & 7) * 16;
 }
 
-// Slices of the operand B of problems p0 + blockIdx.x, columns 32
+// Slices of the operand B of problems p0 + blockIdx.x, columns c0 + 32
 // blockIdx.y + lane; warp w takes the groups of 8 K rows w, w + 16, ....
 // NG > 0: at most NG groups per warp, held in registers between the
 // exponent pass and the slicing; NG = 0: any K, read twice, the second time
@@ -184,8 +184,8 @@ __device__ __forceinline__ int core_off(int row, int k8) {
 // P~(0) = 0).
 template <int NG, bool INV>
 __global__ void __launch_bounds__(512)
-    slice_b_kernel(const double* B, const S64Prob* __restrict__ probs, int p0, int C,
-                   int C16, unsigned char* __restrict__ out, int* __restrict__ eb,
+    slice_b_kernel(const double* B, const S64Prob* __restrict__ probs, int p0, int c0,
+                   int C, int C16, unsigned char* __restrict__ out, int* __restrict__ eb,
                    const double* __restrict__ pnm, int ldp, int N, int Jh,
                    double* __restrict__ O, int wait) {
     __shared__ int red[16][32];
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(512)
     const int p = p0 + blockIdx.x;
     const S64Prob pr = probs[p];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int c = blockIdx.y * 32 + lane;
+    const int c = c0 + blockIdx.y * 32 + lane;
     const bool cin = c < C;
     const double* col = B + pr.src_off + c;
     auto load = [&](int k) -> double {
@@ -880,19 +880,26 @@ void build_dir(int N, int Jh, int C, bool inverse, S64Dir& d, HostDir& h) {
 }
 
 template <bool INV>
-cudaError_t launch_slice_b(int maxK, dim3 grid, cudaStream_t s, const double* B, const S64Prob* probs,
-                    int p0, int C, int C16, unsigned char* out, int* eb, const double* pnm,
-                    int ldp, int N, int Jh, double* O) {
-    using Fn = void (*)(const double*, const S64Prob*, int, int, int, unsigned char*, int*,
+cudaError_t launch_slice_b(int maxK, cudaStream_t s, const double* B, const S64Prob* probs, int p0,
+                           int np, int C, int C16, unsigned char* out, int* eb, const double* pnm,
+                           int ldp, int N, int Jh, double* O) {
+    using Fn = void (*)(const double*, const S64Prob*, int, int, int, int, unsigned char*, int*,
                         const double*, int, int, int, double*, int);
     // in registers where two CTAs still fit an SM
     const int ng = (maxK + 127) / 128;
     const Fn fn = ng == 1            ? slice_b_kernel<1, INV>
                   : ng == 2 && !INV ? slice_b_kernel<2, false>
                                     : slice_b_kernel<0, INV>;
-    const bool wait = short_launch((long long)grid.x * grid.y);
-    return launch_kernel(fn, grid, dim3(512), 0, s, wait, B, probs, p0, C, C16,
-                         out, eb, pnm, ldp, N, Jh, O, wait ? 1 : 0);
+    // (a grid's second dimension holds 65535 blocks, 2^20 fields)
+    for (int y0 = 0, ny = (C16 + 31) / 32; y0 < ny; y0 += 65535) {
+        const dim3 grid(np, std::min(ny - y0, 65535));
+        const bool wait = short_launch((long long)grid.x * grid.y);
+        const cudaError_t e =
+            launch_kernel(fn, grid, dim3(512), 0, s, wait, B, probs, p0, 32 * y0, C, C16, out, eb,
+                          pnm, ldp, N, Jh, O, wait ? 1 : 0);
+        if (e) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, double* O,
@@ -916,13 +923,13 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
     cudaError_t e = ensure_smem((const void*)fn, smem);
     if (e) return e;
     for (const S64Chunk& c : d.chunks) {
-        const dim3 grid(c.p1 - c.p0, (sl->C16 + 31) / 32);
+        const int np = c.p1 - c.p0;
         if (inverse)
-            e = launch_slice_b<true>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
-                                 sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
+            e = launch_slice_b<true>(d.maxK, s, B, d.d_probs, c.p0, np, C, sl->C16, sl->bbuf,
+                                     sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
         else
-            e = launch_slice_b<false>(d.maxK, grid, s, B, d.d_probs, c.p0, C, sl->C16, sl->bbuf,
-                                  sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
+            e = launch_slice_b<false>(d.maxK, s, B, d.d_probs, c.p0, np, C, sl->C16, sl->bbuf,
+                                      sl->eb, p->d_pnm, p->ldp, p->N, p->Jh, O);
         if (e) return e;
         S64Args g;
         g.table = d.table;

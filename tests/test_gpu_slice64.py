@@ -137,3 +137,17 @@ def test_long_sums(sht, N, J, I, F):
     assert_fp64_close(p.inverse(to_cuda(a, torch.complex128)).cpu().numpy(),
                       O.synthesis(a, N, J, I))
     p.status()
+
+
+def test_more_than_a_million_fields(sht):
+    # 2 F columns in blocks of 32: more blocks than a grid's second dimension holds
+    N, J, I, F = 1, 5, 8, (1 << 20) + 1
+    p = sht.Plan(N, J, I, F, "fp64")
+    x = torch.randn(F, J, I, dtype=torch.float64, device="cuda",
+                    generator=torch.Generator("cuda").manual_seed(2800))
+    got = p.forward(x)
+    pick = [0, 1, 12345, F - 2, F - 1]
+    assert_fp64_close(got[:, pick].cpu().numpy(), O.analysis(x[pick].cpu().numpy(), N))
+    back = p.inverse(got)
+    assert_fp64_close(back[pick].cpu().numpy(), O.synthesis(got[:, pick].cpu().numpy(), N, J, I))
+    p.status()
