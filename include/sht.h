@@ -112,6 +112,21 @@ int sht_plan_create_grid(int N, int J, int I, int nfields, int precision, int gr
  * as long as its memory has not been reused. */
 int sht_plan_destroy(sht_plan_t plan);
 
+/* FP64 plans contract on the tensor cores from 1.5e7 flops up (more than one
+ * field, J < 8192), which needs slices of the P~ table and a buffer: 28 bytes
+ * for every 8 of the table and up to 1 GiB or a wavenumber's share of the fields
+ * (T639 x 256: 4.6 GiB).  Plan creation takes that memory if it is at most an
+ * eighth of what the device has free; else, or if an allocation fails, the plan
+ * works without, on the FP64 pipe, about 12 times slower.
+ *
+ * sht_plan_get_tensor_tables writes whether the plan has them (*on = 1 or 0)
+ * and their bytes; either pointer may be NULL.  sht_plan_set_tensor_tables frees
+ * them (on = 0), or builds them whatever they take (on != 0; SHT_ERR_ALLOC leaves
+ * the plan without).  Synchronises the device; groups that hold the plan follow.
+ * SHT_ERR_UNSUPPORTED for split plans and for plans outside the range above. */
+int sht_plan_set_tensor_tables(sht_plan_t plan, int on);
+int sht_plan_get_tensor_tables(sht_plan_t plan, int* on, size_t* bytes);
+
 /* Plan parameters; any output pointer may be NULL.  exact = (J >= 2N+1). */
 int sht_plan_query(sht_plan_t plan, int* N, int* J, int* I, int* nfields,
                    int* precision, int* exact, size_t* ncoef);

@@ -23,6 +23,7 @@ EXPORTED = [
     "sht_plan_grid_points", "sht_profile_read_kernels", "sht_prolong_spectral_add",
     "sht_measure_fma_peak", "sht_alias_products", "sht_plan_create_reduced_shifted",
     "sht_octahedral_grid_sizes", "sht_icositetrahedral_grid_sizes",
+    "sht_plan_set_tensor_tables", "sht_plan_get_tensor_tables",
 ]
 PROFILE_STAGES = 8
 STAGE_NAMES = ["fft_forward", "legendre_forward", "legendre_inverse",
@@ -60,6 +61,8 @@ def _load():
     lib.sht_prolong_spectral_add.argtypes = [vp, vp, i, vp, vp]
     lib.sht_inject_nested.argtypes = [vp, vp, i, vp, vp]
     lib.sht_plan_destroy.argtypes = [vp]
+    lib.sht_plan_set_tensor_tables.argtypes = [vp, i]
+    lib.sht_plan_get_tensor_tables.argtypes = [vp, ip, ctypes.POINTER(ctypes.c_size_t)]
     lib.sht_plan_query.argtypes = [vp, ip, ip, ip, ip, ip, ip,
                                    ctypes.POINTER(ctypes.c_size_t)]
     lib.sht_forward.argtypes = [vp, vp, vp, vp]

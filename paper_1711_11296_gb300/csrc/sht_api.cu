@@ -229,12 +229,18 @@ extern "C" int sht_plan_create_grid(int N, int J, int I, int nfields, int precis
     // allocation of the plan's tables as if the device were out of memory
     int inject_alloc = 0, nalloc = 0;
     if (const char* v = getenv("SHT_INJECT_ALLOC_FAIL")) inject_alloc = atoi(v);
-    auto alloc = [&](void** ptr, size_t bytes, const char* what) -> bool {
-        e = (++nalloc == inject_alloc) ? cudaErrorMemoryAllocation
-                                       : cudaMalloc(ptr, bytes > 0 ? bytes : 16);
-        if (e != cudaSuccess) {
+    auto try_alloc = [&](void** ptr, size_t bytes) -> cudaError_t {
+        const cudaError_t r = (++nalloc == inject_alloc) ? cudaErrorMemoryAllocation
+                                                         : cudaMalloc(ptr, bytes > 0 ? bytes : 16);
+        if (r != cudaSuccess) {
             *ptr = nullptr;
             cudaGetLastError();
+        }
+        return r;
+    };
+    auto alloc = [&](void** ptr, size_t bytes, const char* what) -> bool {
+        e = try_alloc(ptr, bytes);
+        if (e != cudaSuccess) {
             set_error("cudaMalloc(%zu) for %s failed: %s", bytes, what,
                       cudaGetErrorString(e));
             rc = SHT_ERR_ALLOC;
@@ -275,7 +281,11 @@ extern "C" int sht_plan_create_grid(int N, int J, int I, int nfields, int precis
         if (e == cudaSuccess) e = build_pnm_table(p, s);
         if (e == cudaSuccess) e = build_twiddles(p, s);
         if (e == cudaSuccess && !fp64) e = split_tables_create(p, s);
-        if (e == cudaSuccess && fp64) e = slice64_create(p, s);
+        if (e == cudaSuccess && fp64) {
+            // (the plan works without them)
+            e = slice64_create(p, kSliceShare, try_alloc, s);
+            if (e == cudaErrorMemoryAllocation) e = cudaSuccess;
+        }
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e != cudaSuccess) {
             if (e == cudaErrorNotSupported) {
@@ -316,6 +326,38 @@ extern "C" int sht_plan_destroy(sht_plan_t plan) {
     free_plan_memory(plan);
     plan->magic = 0;
     delete plan;
+    return SHT_OK;
+}
+
+extern "C" int sht_plan_set_tensor_tables(sht_plan_t p, int on) {
+    int rc = check_plan(p);
+    if (rc) return rc;
+    if (p->prec != SHT_FP64 || !slice64_takes(p)) {
+        set_error(p->prec != SHT_FP64 ? "split plans have no FP64 slice tables"
+                                      : "this plan's contractions are not sliced");
+        return SHT_ERR_UNSUPPORTED;
+    }
+    DeviceGuard dg(p->device);
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(e, "synchronise");
+    if (!on) {
+        slice64_destroy(p);
+        return SHT_OK;
+    }
+    e = slice64_create(
+        p, 0, [](void** ptr, size_t bytes) { return cudaMalloc(ptr, bytes); }, nullptr);
+    if (e == cudaErrorMemoryAllocation) {
+        set_error("no memory for the slice tables; the contractions stay on the FP64 pipe");
+        return SHT_ERR_ALLOC;
+    }
+    return e == cudaSuccess ? SHT_OK : cuda_fail(e, "slice tables");
+}
+
+extern "C" int sht_plan_get_tensor_tables(sht_plan_t p, int* on, size_t* bytes) {
+    int rc = check_plan(p);
+    if (rc) return rc;
+    if (on) *on = p->slice ? 1 : 0;
+    if (bytes) *bytes = slice64_bytes(p);
     return SHT_OK;
 }
 

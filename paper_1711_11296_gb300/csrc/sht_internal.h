@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -399,8 +400,16 @@ bool legendre_small(const sht_plan_s* p);
 // FP64 contractions on the tensor cores (sht_slice64.cu): plan tables (none
 // for small ones) and the launches launch_legendre_*_fp64 hand over to when
 // the plan has them.
-cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s);
+using DeviceAlloc = std::function<cudaError_t(void**, size_t)>;
+bool slice64_takes(const sht_plan_s* p);      // not small, nor too long for its sums
+size_t slice64_bytes(const sht_plan_s* p);    // device memory of the tables (0: none)
+cudaError_t slice64_create(sht_plan_s* p, int share, const DeviceAlloc& alloc, cudaStream_t s);
 void slice64_destroy(sht_plan_s* p);
+// Plan creation builds the tables where they take at most this part of the
+// device's free memory: 28 bytes for every 8 of the P~ table, and up to 1 GiB of
+// slices of the data (T639 x 256 4.6 GiB, T1279 x 64 29 GiB, a ninth of an empty
+// GB300).
+constexpr int kSliceShare = 8;
 cudaError_t launch_legendre_slice64(const sht_plan_s* p, bool inverse, const double* in,
                                     double* out, cudaStream_t s);
 

@@ -50,6 +50,7 @@
 // K-major core-matrix layout; slice_gemm_kernel multiplies, both operands
 // arriving by bulk copies.  The slices of A are made once per plan.
 #include <limits.h>
+#include <stdlib.h>
 
 #include <algorithm>
 #include <new>
@@ -100,6 +101,7 @@ struct Slice64 {
     unsigned char* bbuf = nullptr;  // B slices of one chunk: [K slab][slice][C16][16]
     int* eb = nullptr;              // [problem][C16] column exponents
     int C16 = 0;
+    size_t bytes = 0;               // device memory of all of it
 };
 
 namespace {
@@ -958,32 +960,62 @@ cudaError_t launch_dir(const sht_plan_s* p, bool inverse, const double* B, doubl
 
 }  // namespace
 
-// The slice tables of an FP64 plan (none for small transforms, see
-// legendre_small); without the memory for them the plan stays on the FP64
-// pipe.
-cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
-    if (legendre_small(p) || p->Jh > kMaxJh) return cudaSuccess;
+bool slice64_takes(const sht_plan_s* p) { return !legendre_small(p) && p->Jh <= kMaxJh; }
+
+size_t slice64_bytes(const sht_plan_s* p) { return p->slice ? p->slice->bytes : 0; }
+
+// The slice tables of an FP64 plan that slice64_takes.  share > 0: only if they
+// take no more than 1 / share of the device's free memory.  Without them (also
+// when an allocation fails, cudaErrorMemoryAllocation) the plan's contractions
+// stay on the FP64 pipe.
+cudaError_t slice64_create(sht_plan_s* p, int share, const DeviceAlloc& alloc, cudaStream_t s) {
+    if (!slice64_takes(p) || p->slice) return cudaSuccess;
     Slice64* sl = new (std::nothrow) Slice64();
-    if (!sl) return cudaSuccess;
+    if (!sl) return cudaErrorMemoryAllocation;
     p->slice = sl;
     const int C = 2 * p->F, nprob = 2 * (p->N + 1);
     sl->C16 = (C + 15) / 16 * 16;
     HostDir h[2];
-    for (int i = 0; i < 2; ++i) build_dir(p->N, p->Jh, C, i == 1, sl->dir[i], h[i]);
-    cudaError_t e = cudaMalloc(&sl->bbuf, std::max(h[0].bbytes, h[1].bbytes));
-    if (e == cudaSuccess) e = cudaMalloc(&sl->eb, (size_t)nprob * sl->C16 * sizeof(int));
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-        S64Dir& d = sl->dir[i];
-        e = cudaMalloc(&d.table, (size_t)h[i].table_bytes + 16);
-        if (e == cudaSuccess) e = cudaMalloc(&d.ea, (size_t)(h[i].ea_rows + 1) * sizeof(int));
-        if (e == cudaSuccess) e = cudaMalloc(&d.seg, (size_t)nprob * kMaxSeg * sizeof(int));
-        if (e == cudaSuccess) e = cudaMalloc(&d.d_probs, nprob * sizeof(S64Prob));
-        if (e == cudaSuccess) e = cudaMalloc(&d.d_tiles, (h[i].tiles.size() + 1) * sizeof(int4));
+    struct Part { void** ptr; size_t bytes; };
+    std::vector<Part> parts;
+    try {
+        for (int i = 0; i < 2; ++i) build_dir(p->N, p->Jh, C, i == 1, sl->dir[i], h[i]);
+        parts.reserve(12);
+    } catch (const std::bad_alloc&) {
+        slice64_destroy(p);
+        return cudaErrorMemoryAllocation;
     }
+    auto part = [&](auto& ptr, size_t bytes) {
+        parts.push_back({reinterpret_cast<void**>(&ptr), bytes});
+        sl->bytes += bytes;
+    };
+    part(sl->bbuf, std::max(h[0].bbytes, h[1].bbytes));
+    part(sl->eb, (size_t)nprob * sl->C16 * sizeof(int));
+    for (int i = 0; i < 2; ++i) {
+        S64Dir& d = sl->dir[i];
+        part(d.table, (size_t)h[i].table_bytes + 16);
+        part(d.ea, (size_t)(h[i].ea_rows + 1) * sizeof(int));
+        part(d.seg, (size_t)nprob * kMaxSeg * sizeof(int));
+        part(d.d_probs, nprob * sizeof(S64Prob));
+        part(d.d_tiles, (h[i].tiles.size() + 1) * sizeof(int4));
+    }
+    cudaError_t e = cudaSuccess;
+    if (share > 0) {
+        size_t avail = 0, total = 0;
+        e = cudaMemGetInfo(&avail, &total);
+        // (tests: SHT_INJECT_FREE_BYTES stands for what is free)
+        if (const char* v = getenv("SHT_INJECT_FREE_BYTES")) avail = (size_t)strtoull(v, nullptr, 10);
+        if (e == cudaSuccess && sl->bytes > avail / share) {
+            slice64_destroy(p);
+            return cudaSuccess;
+        }
+    }
+    for (const Part& q : parts)
+        if (e == cudaSuccess) e = alloc(q.ptr, q.bytes);
     if (e != cudaSuccess) {
         slice64_destroy(p);
         cudaGetLastError();
-        return cudaSuccess;
+        return e;
     }
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         S64Dir& d = sl->dir[i];
@@ -1001,8 +1033,8 @@ cudaError_t slice64_create(sht_plan_s* p, cudaStream_t s) {
         e = cudaGetLastError();
     }
     // (the host lists above must outlive the copies)
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    return e;
+    const cudaError_t es = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? es : e;
 }
 
 void slice64_destroy(sht_plan_s* p) {

@@ -244,6 +244,21 @@ class Plan:
         with torch.cuda.device(self.device):
             check(lib.sht_plan_set_reduced(self._h, 1 if on else 0))
 
+    @property
+    def tensor_tables(self):
+        """{"on": bool, "bytes": n}: whether an FP64 plan has the tables of its
+        tensor-core contractions, and the device memory they take; see
+        ``sht_plan_set_tensor_tables``."""
+        on, n = ctypes.c_int(), ctypes.c_size_t()
+        check(lib.sht_plan_get_tensor_tables(self._h, ctypes.byref(on), ctypes.byref(n)))
+        return {"on": bool(on.value), "bytes": n.value}
+
+    def set_tensor_tables(self, on=True):
+        """Free those tables (the contractions then run on the FP64 pipe), or
+        build them whatever memory they take."""
+        with torch.cuda.device(self.device):
+            check(lib.sht_plan_set_tensor_tables(self._h, 1 if on else 0))
+
     def autotune(self, reps=3):
         """Time the candidate launch shapes on this plan and keep the fastest;
         returns the choice and the mean ms of an inverse + forward pair."""
