@@ -194,7 +194,7 @@ __device__ __forceinline__ float abs_f32(unsigned h) {
     return __int_as_float(max((int)h - (896 << 20), 0) << 3);
 }
 
-// round(v 2^shift), |result| <= 2^61.  Integer operations: as a conversion on
+// round(v 2^shift), |result| <= 2^61, shift <= 1082.  Integer operations: as a conversion on
 // the FP64 pipe the first pass of the forward took 7 % longer.
 __device__ __forceinline__ ll to_fx(double v, int shift) {
     const ll bits = __double_as_longlong(v);
@@ -212,19 +212,19 @@ __device__ __forceinline__ ll to_fx(double v, int shift) {
 // integer * 2^(e - SH + k), times f.
 template <class Bound>
 __device__ __forceinline__ void finish_field(Field& fd, float l1, Bound bound, double f) {
-    const int E = max((int)(fd.hmax >> 20), 1);   // biased exponent field
-    const int e = E - 1022;
+    const int E = (int)(fd.hmax >> 20);   // biased exponent field
+    // (subnormals: below 2^(bits of the high word - 1042))
+    const int e = E > 0 ? E - 1022 : 32 - __clz((int)fd.hmax) - 1042;
     // without a usable FP32 sum the maximum alone bounds the growth
     l1 = (E >= 940 && E <= 1140) ? l1 * 1.0001f * __int_as_float((127 - e) << 23)
                                  : __int_as_float(0x7f800000);
     int k;
     const float b = bound(l1, k);
     const int SH = min(61, (int)floorf(61.4f - log2f(b)));
-    fd.shift = SH - e;
-    const int p2 = e - SH + k;
+    fd.shift = min(SH - e, 1082);   // as far as to_fx shifts
+    const int p2 = k - fd.shift;
     const bool tiny = p2 < -900;   // 2^p2 would be subnormal
-    // (zero rows give zeros, not the last place's rounding; values that are
-    // all below 2^-1042, whose high words are 0, count as zero)
+    // (zero rows give zeros, not the last place's rounding)
     fd.sc = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
             : fd.hmax == 0u ? 0.0
                             : ldexp(f, tiny ? p2 + 200 : p2);
@@ -368,8 +368,10 @@ __device__ __forceinline__ float pass_bound(const FftShape& sh, float zmax, floa
     }
 }
 
-// Reduce a thread's share of one row into its field.
-__device__ __forceinline__ void gather_row(Field& fd, int row, unsigned hm, float l1) {
+// Reduce a thread's share of one row into its field.  low: its values' low words,
+// which tell the smallest subnormals (high word 0) from zeros.
+__device__ __forceinline__ void gather_row(Field& fd, int row, unsigned hm, int low, float l1) {
+    if (low != 0) hm = max(hm, 1u);
     hm = __reduce_max_sync(0xffffffffu, hm);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
@@ -421,14 +423,16 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<double>& A, int fg, int j
     // the largest component of each field and the L1 norm of each row
     for (int r = 0; r < nrows; ++r) {
         unsigned hm = 0u;
+        int low = 0;
         float l1 = 0.f;
         for (int k = tid; k < L; k += NT) {
             const double2 v = raw[(size_t)r * LP + ph<double>(k)];
             const unsigned hx = hi_abs(v.x), hy = hi_abs(v.y);
             hm = max(hm, max(hx, hy));
+            low |= __double2loint(v.x) | __double2loint(v.y);
             l1 += abs_f32(hx) + abs_f32(hy);
         }
-        gather_row(fd[r < nf ? r : r - nf], r < nf ? 0 : 1, hm, l1);
+        gather_row(fd[r < nf ? r : r - nf], r < nf ? 0 : 1, hm, low, l1);
     }
     __syncthreads();
     if (tid < nf) {
@@ -516,14 +520,17 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
     // at m = 0 is not an input; Re there counts twice, as Y_0 may)
     for (int r = 0; r < nrows; ++r) {
         unsigned hm = 0u;
+        int low = 0;
         float l1 = 0.f;
         for (int k = tid; k <= kmax; k += NT) {
             const double2 v = raw[(size_t)r * LP + ph<double>(k)];
-            const unsigned hx = hi_abs(v.x), hy = k == 0 ? hx : hi_abs(v.y);
+            const double y = k == 0 ? v.x : v.y;
+            const unsigned hx = hi_abs(v.x), hy = hi_abs(y);
             hm = max(hm, max(hx, hy));
+            low |= __double2loint(v.x) | __double2loint(y);
             l1 += abs_f32(hx) + abs_f32(hy);
         }
-        gather_row(fd[r < nf ? r : r - nf], r < nf ? 0 : 1, hm, l1);
+        gather_row(fd[r < nf ? r : r - nf], r < nf ? 0 : 1, hm, low, l1);
     }
     __syncthreads();
     // The factor of the m >= 1 terms (1, or 1/2 for an adjoint) goes into the
@@ -533,7 +540,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<double>& A, int fg, int j
         Field& q = fd[tid];
         // packed values: |Z_q| / 2 <= |Y_q| + |Y_{L-q}|, |Y| <= |S| + |A|; the
         // phase of a shifted row may raise a component by sqrt(2)
-        if (A.shiftph && q.hmax != 0u && q.hmax < 0x7fe00000u) q.hmax += 0x100000u;
+        if (A.shiftph && q.hmax < 0x7fe00000u) q.hmax += min(q.hmax, 0x100000u);
         finish_field(
             q, q.norm(0) + q.norm(1),
             [&](float l1, int& k) {

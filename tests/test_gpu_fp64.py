@@ -152,3 +152,19 @@ def test_errors_are_reported(sht):
     p = _plan(sht, 3, 7, 8, 1)
     with pytest.raises(ValueError):
         p.forward(torch.zeros((1, 7, 8), dtype=torch.float32, device="cuda"))
+
+
+# Values below 2^-1042 have no bits in their high words.  Tolerance: every value
+# formed on the way is rounded to a multiple of 2^-1074, the forward's sum adds J of
+# them (and the folded rows' weights are below 1).
+@pytest.mark.parametrize("N,J,I,F", [(12, 27, 48, 2), (12, 27, 54, 2), (63, 129, 256, 64)])
+@pytest.mark.parametrize("e", [-1042, -1044, -1060])
+def test_smallest_subnormals(sht, N, J, I, F, e):
+    p = sht.Plan(N, J, I, F, "fp64")
+    v = 1.5 * 2.0 ** e
+    got = p.forward(torch.full((F, J, I), v, dtype=torch.float64, device="cuda")).cpu().numpy()
+    assert np.abs(got[0] - v * np.sqrt(2.0)).max() <= (J + 4) * 2.0 ** -1074
+    a = torch.zeros((p.ncoef, F), dtype=torch.complex128, device="cuda")
+    a[0] = v
+    got = p.inverse(a).cpu().numpy()
+    assert np.abs(got - v * np.sqrt(0.5)).max() <= 4 * 2.0 ** -1074
