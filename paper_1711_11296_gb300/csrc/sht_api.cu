@@ -45,9 +45,9 @@ struct DeviceGuard {
     }
 };
 
-bool factor_fft(int L, int F, bool fp64, FftShape& sh) {
+bool factor_fft(int L, int F, int Jh, bool fp64, FftShape& sh) {
     if (!fft_factorable(L)) return false;
-    sh = fft_shape(L, fp64, fft_has_fixed_kernel(L), nullptr, F);
+    sh = fft_shape(L, fp64, fft_has_fixed_kernel(L), nullptr, F, Jh);
     return true;
 }
 
@@ -189,7 +189,7 @@ extern "C" int sht_plan_create_grid(int N, int J, int I, int nfields, int precis
         return SHT_ERR_ARG;
     }
     FftShape shape;
-    if (!factor_fft(I / 2, nfields, precision == SHT_FP64, shape)) {
+    if (!factor_fft(I / 2, nfields, (J + 1) / 2, precision == SHT_FP64, shape)) {
         set_error("I/2 = %d has prime factors other than 2, 3, 5", I / 2);
         return SHT_ERR_ARG;
     }

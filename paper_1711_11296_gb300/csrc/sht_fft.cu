@@ -1,5 +1,7 @@
 // FFT launches: arguments from the plans, the dispatch on the half-length, and
 // the kernels of the compile-time lengths (sht_fft_kernels.h).
+#include <limits.h>
+
 #include <algorithm>
 #include <mutex>
 
@@ -397,7 +399,18 @@ cudaError_t launch_fft_inverse_group(sht_plan_s* const* plans, int n,
 // keep its threads busy (forward / inverse us, L = 288 x 1 field: 12 24
 // 18.3 / 16.4, 3 4 4 6 14.7 / 12.3; L = 900 x 1: 30 30 29.9 / 29.1, 9 10 10
 // 25.1 / 22.2).
-FftShape fft_shape(int L, bool fp64, bool compile_time, float* time, int F) {
+//
+// The kernel that holds all those sizes has 128 registers, two CTAs per SM, and
+// starts about 1.5 us later than the one of the sizes up to kSmallRadix, which
+// has 80 and runs three.  A regular grid of L > 320 takes the latter where the
+// instructions that larger radices save, by the estimate, come to less than 20
+// million over the grid, or to none.  Sums of the forward and inverse FFT in us,
+// all sizes -> up to 10: L = 432 x 4 43.0 -> 28.0, 720 x 1 42.9 -> 27.6, 900 x 2 50.2
+// -> 37.0, 360 x 16 53.4 -> 37.1, 1000 x 16 219 -> 202; kept with all sizes: 675 x 8
+// 85.9 (109 with up to 10), 1080 x 8 138 (161), 1250 x 8 188 (210).  Shorter rows
+// with all sizes take two passes, which is more exact and in grouped launches
+// faster (T63 x 67, L = 96: group pair 66.5 us, with three passes 70.3).
+FftShape fft_shape(int L, bool fp64, bool compile_time, float* time, int F, int Jh) {
     if (time) *time = 0.f;
     if (fp64 || L == 1 || compile_time) return fft_factor(L, fp64);
     struct Size { int r; float work; };   // instructions of the DFT per value
@@ -412,7 +425,7 @@ FftShape fft_shape(int L, bool fp64, bool compile_time, float* time, int F) {
     };
     int best[4], cur[4], nbest = 0;
     float tbest = 0.f;
-    auto search = [&](auto&& self, int rest, int depth, int from, float t) -> void {
+    auto search = [&](auto&& self, int limit, int rest, int depth, int from, float t) -> void {
         if (rest == 1) {
             if (nbest == 0 || t < tbest) {
                 nbest = depth;
@@ -423,14 +436,35 @@ FftShape fft_shape(int L, bool fp64, bool compile_time, float* time, int F) {
         }
         if (depth == 4) return;
         for (int i = from; i < (int)(sizeof(sizes) / sizeof(sizes[0])); ++i) {
-            if (rest % sizes[i].r) continue;
+            if (sizes[i].r > limit || rest % sizes[i].r) continue;
             cur[depth] = sizes[i].r;
-            self(self, rest / sizes[i].r, depth + 1, i, t + cost(sizes[i]));
+            self(self, limit, rest / sizes[i].r, depth + 1, i, t + cost(sizes[i]));
         }
     };
-    search(search, L, 0, 0, 0.f);
+    // instructions per value of the radices found, all threads busy
+    auto instructions = [&]() {
+        float n = 0.f;
+        for (int q = 0; q < nbest; ++q)
+            for (const Size& z : sizes) n += best[q] == z.r ? 14.f + z.work : 0.f;
+        return n;
+    };
+    int small[4], nsmall = 0;
+    float isaved = 0.f;
+    if (Jh > 0 && L > 320) {
+        search(search, kSmallRadix, L, 0, 0, 0.f);
+        nsmall = nbest;
+        for (int q = 0; q < nbest; ++q) small[q] = best[q];
+        isaved = instructions();
+        nbest = 0;
+    }
+    search(search, INT_MAX, L, 0, 0, 0.f);
     if (nbest == 0) return fft_factor(L, true);
     if (time) *time = tbest * (float)L;
+    isaved -= instructions();
+    if (nsmall > 0 && (double)isaved * L * Jh * F < 20e6) {
+        nbest = nsmall;
+        for (int q = 0; q < nsmall; ++q) best[q] = small[q];
+    }
     FftShape sh{};
     sh.L = L;
     sh.npass = nbest;

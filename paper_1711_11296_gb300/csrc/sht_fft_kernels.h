@@ -311,9 +311,10 @@ template <typename T> struct Dft<T, 30> : DftCoprime<T, 5, 6> {};
 template <typename T> struct Dft<T, 32> : DftComposite<T, 8, 4> {};
 template <typename T> struct Dft<T, 40> : DftCoprime<T, 8, 5> {};
 
-// f(integral_constant<int, r>) for a radix known at run time: every register
-// DFT size for FP32, the basic ones for FP64 (Bluestein rows).
-template <typename T, class F>
+// f(integral_constant<int, r>) for a radix known at run time: FP64 (Bluestein
+// rows) 2, 3, 4, 5 and 8, FP32 the register DFT sizes up to kSmallRadix, with
+// ALL every one.
+template <typename T, bool ALL, class F>
 __device__ __forceinline__ void with_radix(int r, F f) {
 #define SHT_RADIX(R) \
     case R: f(std::integral_constant<int, R>{}); return;
@@ -323,9 +324,14 @@ __device__ __forceinline__ void with_radix(int r, F f) {
     }
     if constexpr (sizeof(T) == 4) {
         switch (r) {
-            SHT_RADIX(6) SHT_RADIX(9) SHT_RADIX(10) SHT_RADIX(12) SHT_RADIX(15)
-            SHT_RADIX(16) SHT_RADIX(20) SHT_RADIX(24) SHT_RADIX(25) SHT_RADIX(30)
-            SHT_RADIX(32)
+            SHT_RADIX(6) SHT_RADIX(9) SHT_RADIX(10)
+            default: break;
+        }
+    }
+    if constexpr (sizeof(T) == 4 && ALL) {
+        switch (r) {
+            SHT_RADIX(12) SHT_RADIX(15) SHT_RADIX(16) SHT_RADIX(20) SHT_RADIX(24)
+            SHT_RADIX(25) SHT_RADIX(30) SHT_RADIX(32)
             default: break;
         }
     }
@@ -387,14 +393,14 @@ __device__ __forceinline__ void bfly_fixed(typename Vec2<T>::type* z, int base,
 
 // In-place mixed-radix DIF FFT over `nrows` padded rows (pitch LP), passes
 // p0 .. p1 - 1 of a shape known at run time.
-template <typename T>
+template <typename T, bool ALL>
 __device__ __forceinline__ void passes_runtime(typename Vec2<T>::type* rows, int nrows, int LP,
                                                const FftShape& sh, int p0, int p1,
                                                const typename Vec2<T>::type* twp) {
     for (int p = p0; p < p1; ++p) {
         const int M = sh.span[p];
         const typename Vec2<T>::type* tw = twp + sh.twoff[p];
-        with_radix<T>(sh.radix[p], [&](auto rc) {
+        with_radix<T, ALL>(sh.radix[p], [&](auto rc) {
             constexpr int R = decltype(rc)::value;
             const int nb = sh.L / R, S = R * M;
             for (int idx = threadIdx.x; idx < nrows * nb; idx += NT) {
@@ -460,7 +466,7 @@ __host__ __device__ constexpr bool inverse_stores_from_last_pass() {
 }
 
 // LT > 0: the compile-time shape of that half-length; LT = -1: any shape at
-// run time.
+// run time; LT = -3: any shape of radices up to kSmallRadix.
 template <typename T, int LT>
 __device__ __forceinline__ void run_passes(typename Vec2<T>::type* rows, int nrows, int LP,
                                            const FftShape& sh,
@@ -468,7 +474,7 @@ __device__ __forceinline__ void run_passes(typename Vec2<T>::type* rows, int nro
     if constexpr (LT > 0)
         passes_fixed<T, LT, 0>(rows, nrows, LP, twp);
     else
-        passes_runtime<T>(rows, nrows, LP, sh, 0, sh.npass, twp);
+        passes_runtime<T, LT == -1>(rows, nrows, LP, sh, 0, sh.npass, twp);
 }
 
 // Bluestein's chirp-z DFT of rows of half-length L (any L), for the rows of
@@ -496,8 +502,8 @@ __device__ __noinline__ void bluestein_rows(typename Vec2<T>::type* rows, int nr
     using V = typename Vec2<T>::type;
     using K = C2<T>;
     const int np = sh.npass;
-    passes_runtime<T>(rows, nrows, LP, sh, 0, np - 1, tws);
-    with_radix<T>(sh.radix[np - 1], [&](auto rc) {
+    passes_runtime<T, true>(rows, nrows, LP, sh, 0, np - 1, tws);
+    with_radix<T, true>(sh.radix[np - 1], [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         const int nb = sh.L / R;
         for (int idx = threadIdx.x; idx < nrows * nb; idx += NT) {
@@ -519,7 +525,7 @@ __device__ __noinline__ void bluestein_rows(typename Vec2<T>::type* rows, int nr
     for (int p = np - 2; p >= 0; --p) {
         const int M = sh.span[p];
         const V* tw = tws + sh.twoff[p];
-        with_radix<T>(sh.radix[p], [&](auto rc) {
+        with_radix<T, true>(sh.radix[p], [&](auto rc) {
             constexpr int R = decltype(rc)::value;
             const int nb = sh.L / R, S = R * M;
             for (int idx = threadIdx.x; idx < nrows * nb; idx += NT) {
@@ -624,11 +630,11 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
             __syncthreads();
             passes_fixed<T, LT, 1>(rows, nrows, LP, tws);
         }
-    } else if (LT == -1 && sizeof(T) == 4 && A.shape.npass > 0 && direct) {
+    } else if ((LT == -1 || LT == -3) && sizeof(T) == 4 && A.shape.npass > 0 && direct) {
         // the same with the shape known at run time
         const int M = A.shape.span[0];
         load_twiddles_async(tws, A.twp, A.shape.twtotal);
-        with_radix<T>(A.shape.radix[0], [&](auto rc) {
+        with_radix<T, LT == -1>(A.shape.radix[0], [&](auto rc) {
             constexpr int R = decltype(rc)::value;
             const int total = nrows * M;
             bool waited = false;
@@ -660,7 +666,7 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
             }
         });
         __syncthreads();
-        passes_runtime<T>(rows, nrows, LP, A.shape, 1, A.shape.npass, tws);
+        passes_runtime<T, LT == -1>(rows, nrows, LP, A.shape, 1, A.shape.npass, tws);
     } else if constexpr (LT == -2) {
         load_twiddles_async(tws, A.twp, A.shape.twtotal);
         for (int r = 0; r < nrows; ++r) {
@@ -891,7 +897,7 @@ __device__ __forceinline__ void fwd_body(const FwdArgs<T>& A, int fg, int jh) {
 }
 
 template <typename T, int LT, bool STRIDED>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(NT, LT == -3 ? 3 : sizeof(T) == 4 ? 2 : 1)
     fft_forward_kernel(const __grid_constant__ FwdArgs<T> A) {
     begin_fft(A.follow);
     fwd_body<T, LT, STRIDED>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);
@@ -1116,15 +1122,15 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
         // pass's registers, 64 bytes a row and warp at a time, the products
         // took 1340 us for Tc479 x 64, now 450.
     }
-    if (LT == -1 && sizeof(T) == 4 && A.accumulate == 0 && A.shape.npass > 0) {
+    if ((LT == -1 || LT == -3) && sizeof(T) == 4 && A.accumulate == 0 && A.shape.npass > 0) {
         // the last pass (span 1) straight to the grid rows, as above: the
         // butterfly of the digits k of the passes before it holds the
         // frequencies f + (L / R) k1, f = k_0 + r_0 (k_1 + r_1 (...)), so
         // lanes of consecutive f store consecutive values
         const int np = A.shape.npass;
-        passes_runtime<T>(rows, nrows, LP, A.shape, 0, np - 1, tws);
+        passes_runtime<T, LT == -1>(rows, nrows, LP, A.shape, 0, np - 1, tws);
         const V sgn = K::make(rs, -rs);   // x = conj(z) rs
-        with_radix<T>(A.shape.radix[np - 1], [&](auto rc) {
+        with_radix<T, LT == -1>(A.shape.radix[np - 1], [&](auto rc) {
             constexpr int R = decltype(rc)::value;
             const int nb = L / R;
             for (int idx = tid; idx < nrows * nb; idx += NT) {
@@ -1226,7 +1232,7 @@ __device__ __forceinline__ void inv_body(const InvArgs<T>& A, int fg, int jh) {
 }
 
 template <typename T, int LT, bool PLAIN = false>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(NT, LT == -3 ? 3 : sizeof(T) == 4 ? 2 : 1)
     fft_inverse_kernel(const __grid_constant__ InvArgs<T> A) {
     begin_fft(A.follow);
     inv_body<T, LT, PLAIN>(A, blockIdx.x, A.jh_list ? A.jh_list[blockIdx.y] : blockIdx.y);

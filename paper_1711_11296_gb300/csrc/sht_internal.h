@@ -316,6 +316,9 @@ void ragged_free(RaggedGrid* rg);
 int inverse_scaled(sht_plan_s* p, const void* spec, const InvScale& sc, void* grid,
                    cudaStream_t s);
 
+// Largest radix of the FP32 FFT kernel for regular grids of few values.
+constexpr int kSmallRadix = 10;
+
 // Register DFT sizes Q of the two-pass FP32 FFT (L = Q x 32).
 __host__ __device__ constexpr bool fft_big_radix(int q) {
     return q == 2 || q == 4 || q == 8 || q == 10 || q == 16 || q == 20 || q == 32 ||
@@ -360,8 +363,10 @@ __host__ __device__ constexpr FftShape fft_factor(int L, bool fp64) {
 // of the length will run, else passes of the register DFT sizes that the
 // kernels with run-time shapes hold (2 .. 32).
 // time: the estimate the choice was made by (0 where there was none).
-// F: the plan's fields.
-FftShape fft_shape(int L, bool fp64, bool compile_time, float* time = nullptr, int F = 16);
+// F: the plan's fields; Jh: a regular grid's latitude pairs, where a shape of
+// radices up to kSmallRadix runs in the kernel that holds only those (0: never).
+FftShape fft_shape(int L, bool fp64, bool compile_time, float* time = nullptr, int F = 16,
+                   int Jh = 0);
 
 __host__ __device__ constexpr bool fft_factorable(int L) {
     return L == 1 || fft_factor(L, true).npass > 0;

@@ -120,3 +120,42 @@ def test_restriction_reads_any_alignment(sht, I, k, offset):
     fine = buf[offset:].view(shape)
     ref = p.forward(p.inject_nested(fine, k))
     assert torch.equal(p.restrict_nested(fine, k), ref)
+
+
+# Grids of few values of L > 320 (the cases above) take the kernel of the radices
+# up to 10; these have enough of them for the kernel of all register sizes.
+@pytest.mark.parametrize("L,F", [(96, 200), (100, 201), (150, 200), (240, 100), (288, 100),
+                                 (300, 101), (375, 64), (625, 64), (720, 40), (800, 40),
+                                 (900, 40), (1125, 41), (1536, 40), (1600, 40), (2000, 24),
+                                 (2048, 25)])
+def test_regular_rows_of_many_fields(sht, L, F):
+    J, I = 201, 2 * L
+    p = sht.Plan(N, J, I, F, "bf16x3")
+    x = W.random_grid(F, J, I, seed=2500 + L).astype(np.float32).astype(np.float64)
+    a = W.random_spectrum(N, F, "flat", seed=2600 + L).astype(np.complex64)
+    assert rel_l2(p.forward(to_cuda(x, torch.float32)).cpu().numpy(), O.analysis(x, N)) <= TOL
+    got = p.inverse(torch.from_numpy(a).cuda()).cpu().numpy()
+    assert rel_l2(got, O.synthesis(a.astype(np.complex128), N, J, I)) <= TOL
+    p.status()
+
+
+def test_both_runtime_kernels_agree(sht):
+    # the same fields in a plan of 3 fields (radices up to 10) and of 64 (30 24), forward,
+    # inverse, onto a grid, strided; both within the FFT's rounding
+    J, I, F = 101, 1440, 64
+    gen = torch.Generator("cuda").manual_seed(2800)
+    x = torch.randn(F, J, I, device="cuda", generator=gen)
+    fine = torch.randn(F, 2 * J + 1, 2 * I, device="cuda", generator=gen)
+    a = torch.from_numpy(W.random_spectrum(N, F, "flat", seed=2801).astype(np.complex64)).cuda()
+    p, q = sht.Plan(N, J, I, F, "bf16x3"), sht.Plan(N, J, I, 3, "bf16x3")
+    pick = slice(5, 8)
+    b = a[:, pick].contiguous()
+
+    def close(got, ref):
+        assert rel_l2(got.cpu().numpy(), ref.cpu().numpy()) <= 5e-7
+
+    close(q.forward(x[pick].contiguous()), p.forward(x)[:, pick])
+    close(q.inverse(b), p.inverse(a)[pick])
+    close(q.prolong_spectral(b, N, out=x[pick].clone(), add=True),
+          p.prolong_spectral(a, N, out=x.clone(), add=True)[pick])
+    close(q.restrict_nested(fine[pick].contiguous(), 1), p.restrict_nested(fine, 1)[:, pick])
