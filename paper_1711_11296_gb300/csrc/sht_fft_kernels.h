@@ -318,20 +318,22 @@ template <typename T, bool ALL, class F>
 __device__ __forceinline__ void with_radix(int r, F f) {
 #define SHT_RADIX(R) \
     case R: f(std::integral_constant<int, R>{}); return;
-    switch (r) {
-        SHT_RADIX(2) SHT_RADIX(3) SHT_RADIX(4) SHT_RADIX(5)
-        default: break;
-    }
-    if constexpr (sizeof(T) == 4) {
-        switch (r) {
-            SHT_RADIX(6) SHT_RADIX(9) SHT_RADIX(10)
-            default: break;
-        }
-    }
     if constexpr (sizeof(T) == 4 && ALL) {
         switch (r) {
-            SHT_RADIX(12) SHT_RADIX(15) SHT_RADIX(16) SHT_RADIX(20) SHT_RADIX(24)
-            SHT_RADIX(25) SHT_RADIX(30) SHT_RADIX(32)
+            SHT_RADIX(2) SHT_RADIX(3) SHT_RADIX(4) SHT_RADIX(5) SHT_RADIX(6)
+            SHT_RADIX(9) SHT_RADIX(10) SHT_RADIX(12) SHT_RADIX(15) SHT_RADIX(16)
+            SHT_RADIX(20) SHT_RADIX(24) SHT_RADIX(25) SHT_RADIX(30) SHT_RADIX(32)
+            default: break;
+        }
+    } else if constexpr (sizeof(T) == 4) {
+        switch (r) {
+            SHT_RADIX(2) SHT_RADIX(3) SHT_RADIX(4) SHT_RADIX(5) SHT_RADIX(6)
+            SHT_RADIX(9) SHT_RADIX(10)
+            default: break;
+        }
+    } else {
+        switch (r) {
+            SHT_RADIX(2) SHT_RADIX(3) SHT_RADIX(4) SHT_RADIX(5)
             default: break;
         }
     }
