@@ -509,12 +509,24 @@ size_t fft_smem_bytes(int I, int G, bool fp64) {
 // fields 369 / 449).  Small grids (T31 x 32 bf16x3): 16 fields, 66 CTAs
 // 10.0 / 11.4, 4 fields, 264 CTAs 8.4 / 8.0; FP64 T63 x 16: 8 fields, 130
 // CTAs 18.0 / 22.4, 2 fields, 520 CTAs 15.1 / 14.2.
+// A few FP32 fields leave a power of two's last CTA of each latitude with little
+// to do.  Up to 5 fields stay together where the latitudes alone fill the grid,
+// and up to 12 that make two CTAs are halved (sum of both FFTs, us: T255 x 3, 2
+// fields 24.9, 3 20.6; T511 x 3 49.3, 40.4; T255 x 5, 4 fields 27.9, 5 22.9; T199 x
+// 9, 8 fields 49.7, 5 37.2; T255 x 12, 8 fields 36.7, 6 35.6; T319 x 12 the other
+// way, 52.0 and 54.6).
 int fft_default_fields(int I, int Jh, int F, bool fp64, int ctas) {
     const size_t budget = (fp64 ? 55 : 112) * 1024;
     int g = 16;
     while (g > 1 && (g > F || fft_smem_bytes(I, g, fp64) > budget ||
                      (long)Jh * ((F + g - 1) / g) < ctas))
         g /= 2;
+    if (!fp64) {
+        if (F <= 5 && Jh >= ctas && fft_smem_bytes(I, F, false) <= budget)
+            g = F;
+        else if (F <= 12 && (F + g - 1) / g == 2)
+            g = (F + 1) / 2;
+    }
     return fft_smem_bytes(I, g, fp64) <= 227 * 1024 ? g : 0;
 }
 

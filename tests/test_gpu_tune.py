@@ -110,3 +110,17 @@ def test_tuning_arguments_and_groups(sht):
     q.set_tuning(tile_width=64)
     with pytest.raises(sht.SHTError):
         grp.forward(x)
+
+
+@pytest.mark.parametrize("N,F,G", [(255, 3, 3), (255, 5, 5), (255, 12, 6), (199, 9, 5), (63, 12, 2),
+                                   (255, 8, 8), (255, 13, 8)])
+def test_default_fields_of_a_few(sht, N, F, G):
+    # few fields share a CTA, or two of equal size, whatever their number; results
+    # do not depend on it
+    J, I = 2 * N + 3, 4 * (N + 1)
+    p = sht.Plan(N, J, I, F, "bf16x3")
+    assert p.tuning["fields_per_cta"] == G
+    x = torch.randn(F, J, I, device="cuda", generator=torch.Generator("cuda").manual_seed(1340))
+    spec, grid = p.forward(x), p.inverse(p.forward(x))
+    p.set_tuning(fields_per_cta=1)
+    assert torch.equal(p.forward(x), spec) and torch.equal(p.inverse(spec), grid)
