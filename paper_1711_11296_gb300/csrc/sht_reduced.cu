@@ -207,9 +207,14 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
     rg->blue_count = (int)jh_all.size() - rg->blue_off;
     if (rg->blue_count > 0) {
         // fields per CTA of the Bluestein launch: a power of two that leaves
-        // room for two CTAs per SM, or one field
+        // room for two CTAs per SM; FP64, whose CTAs the FP64 pipe bounds, also
+        // one that keeps the launch at 256 CTAs (octahedral T63 x 8, forward /
+        // inverse us: 8 fields a CTA 217 / 227, 2 fields 61 / 55; FP32 T127 x 4 the
+        // other way, 4 fields 32 / 33, 2 fields 36 / 40)
         int G = 16;
-        while (G > 1 && (G > p->F || bluestein_smem_bytes(L2max, G, fp64) > 112 * 1024)) G /= 2;
+        while (G > 1 && (G > p->F || bluestein_smem_bytes(L2max, G, fp64) > 112 * 1024 ||
+                         (fp64 && (long)rg->blue_count * ((p->F + G - 1) / G) < 256)))
+            G /= 2;
         rg->blue_G = G;
         rg->blue_smem = bluestein_smem_bytes(L2max, G, fp64);
         if (rg->blue_smem > 227 * 1024) {

@@ -115,3 +115,18 @@ def test_shift_is_a_rotation_of_the_row(sht):
     g1 = p.inverse(to_cuda(a, torch.complex128)).cpu().numpy()
     g2 = q.inverse(to_cuda(rot, torch.complex128)).cpu().numpy()
     assert_fp64_close(g1, g2)
+
+
+@pytest.mark.parametrize("F", [1, 5, 16, 33, 200])
+def test_fp64_bluestein_rows_of_many_fields(sht, F):
+    # one to sixteen fields per CTA of the Bluestein rows, partial groups among them
+    N, J = 15, 33
+    pts = O.octahedral_sizes(J).tolist()
+    p = sht.Plan(N, J, max(pts), F, "fp64", grid="reduced", lat_points=pts)
+    x = np.random.default_rng(2900 + F).standard_normal((F, sum(pts)))
+    a = W.random_spectrum(N, F, "flat", seed=2910)
+    assert_fp64_close(p.forward(to_cuda(x, torch.float64)).cpu().numpy(),
+                      O.analysis_reduced(x, N, J, pts))
+    assert_fp64_close(p.inverse(to_cuda(a, torch.complex128)).cpu().numpy(),
+                      O.synthesis_reduced(a, N, J, pts))
+    p.status()
