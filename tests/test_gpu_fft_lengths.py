@@ -159,3 +159,22 @@ def test_both_runtime_kernels_agree(sht):
     close(q.prolong_spectral(b, N, out=x[pick].clone(), add=True),
           p.prolong_spectral(a, N, out=x.clone(), add=True)[pick])
     close(q.restrict_nested(fine[pick].contiguous(), 1), p.restrict_nested(fine, 1)[:, pick])
+
+
+@pytest.mark.parametrize("L", [384, 480, 768, 960])
+@pytest.mark.parametrize("prec,tol", [("bf16x3", TOL), ("fp64", 1e-12)])
+def test_shifted_and_plain_rows_of_later_compile_time_lengths(sht, L, prec, tol):
+    # shifted rows go to the run-time kernel, plain ones beside them to the
+    # compile-time one (FP64: the run-time one)
+    pts, shift = [2 * L] * J, [j % 2 for j in range((J + 1) // 2)]
+    shift = shift + shift[-2::-1]
+    p = sht.Plan(N, J, 2 * L, 3, prec, grid="reduced", lat_points=pts, half_shift=shift)
+    x = np.random.default_rng(L).standard_normal((3, sum(pts))).astype(np.float32)
+    x = x.astype(np.float64)
+    a = W.random_spectrum(N, 3, "flat", seed=2900 + L).astype(np.complex64).astype(np.complex128)
+    spacings = [0.5 * v for v in shift]
+    got = p.forward(to_cuda(x, p.real_dtype)).cpu().numpy()
+    assert rel_l2(got, O.analysis_reduced(x, N, J, pts, shifts=spacings)) <= tol
+    got = p.inverse(to_cuda(a, p.complex_dtype)).cpu().numpy()
+    assert rel_l2(got, O.synthesis_reduced(a, N, J, pts, shifts=spacings)) <= tol
+    p.status()

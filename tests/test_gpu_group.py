@@ -114,3 +114,40 @@ def test_ensemble_group_full_size_and_graph(sht):
     torch.cuda.synchronize()
     for s, b in zip(s_out, back):
         assert torch.equal(s, b)
+
+
+def test_fp64_group_of_sliced_and_small_plans(sht):
+    # contractions on the tensor cores (slices and GEMM, a launch each per plan) and
+    # with a thread per output, one after another in the group's stream: the
+    # single plans' results bit for bit, eager and from a CUDA graph
+    cfg = [(63, 129, 256, 64), (31, 65, 128, 3), (127, 257, 512, 9), (340, 701, 720, 3)]
+    plans = [sht.Plan(N, J, I, F, "fp64") for N, J, I, F in cfg]
+    assert [p.tensor_tables["on"] for p in plans] == [True, False, True, True]
+    grp = sht.Group(plans)
+    a = [to_cuda(W.random_spectrum(N, F, seed=100 + k), torch.complex128)
+         for k, (N, J, I, F) in enumerate(cfg)]
+    ref_g = [p.inverse(x) for p, x in zip(plans, a)]
+    ref_s = [p.forward(g) for p, g in zip(plans, ref_g)]
+    grids, specs = [p.empty_grid() for p in plans], [p.empty_spec() for p in plans]
+
+    def pair():
+        grp.inverse(a, out=grids)
+        grp.forward(grids, out=specs)
+
+    def check():
+        torch.cuda.synchronize()
+        for got, ref in zip(grids + specs, ref_g + ref_s):
+            assert torch.equal(got, ref)
+            got.zero_()
+
+    for _ in range(5):
+        pair()
+        check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pair()
+    for _ in range(5):
+        graph.replay()
+        check()
+    for p in plans:
+        p.status()
