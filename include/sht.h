@@ -44,13 +44,26 @@ extern "C" {
 typedef struct sht_plan_s* sht_plan_t;
 
 typedef enum {
-    SHT_FP64 = 0,   /* FP64 FFT and FP64 Legendre contraction            */
+    SHT_FP64 = 0,   /* FP64 data, errors at the FP64 rounding (below)    */
     SHT_BF16X2 = 1, /* FP32 FFT; Legendre as 2-term BF16 split products  */
     SHT_BF16X3 = 2, /* FP32 FFT; Legendre as 3-term BF16 split products  */
     SHT_FP16X2 = 3, /* FP32 FFT; Legendre as 2-term FP16 split products  */
     SHT_FP16X3 = 4  /* FP32 FFT; Legendre as 3-term FP16 split products  */
 } sht_precision;
-/* FP16 splits scale each row of the P~ table (at plan time) and each real
+/* FP64: the FFTs run in 64-bit fixed point, scaled per field and latitude pair,
+ * and contractions from 1.5e7 flops up as exact sums of 8-bit slices, scaled per
+ * row of the P~ table and per real column of the data (smaller ones, and plans of
+ * one field, on the FP64 pipe).  Rounding is therefore relative to the largest
+ * value of the latitude pair, row or column, below that of FP64 sums, and not to
+ * each element: what is 2^-k of the largest keeps 53 to 55 - k bits.  An infinity
+ * or NaN makes every result it enters NaN.
+ *
+ * Results of a field depend, within the rounding, on the plan's nfields: FP64
+ * contractions as above, and FP32 rows of lengths without a compile-time FFT
+ * kernel, whose radices are chosen with it.  They never depend on the other
+ * fields' values.
+ *
+ * FP16 splits scale each row of the P~ table (at plan time) and each real
  * column of the FP32 operand (per call, from its largest magnitude) by a
  * power of two into [-1, 1), so that the narrow FP16 exponent range holds
  * the operands; x = x_1 + 2^-11 (x_2 [+ x_3]).  FP16x2 keeps ~22 bits of
@@ -243,8 +256,8 @@ int sht_forward_noalloc(int N, int J, int I, int nfields, const double* grid,
 
 /* Groups: several plans (for example uneven truncations of an ensemble, or
  * the levels of a multigrid ladder) transformed by one launch per kernel
- * stage, so that a batch is four launches per transform pair and fits in
- * one CUDA graph.  The paper has no counterpart; the per-plan results are
+ * stage (FP64 contractions: a launch or two per plan), so that a batch is a
+ * few launches per transform pair and fits in one CUDA graph.  The paper has no counterpart; the per-plan results are
  * those of sht_forward / sht_inverse on each plan.
  *   plans: 1..8 live plans of one precision on one device, each at most
  *   once (their workspaces are used).  The group refers to the plans; they
@@ -305,7 +318,7 @@ int sht_plan_autotune(sht_plan_t plan, int reps, void* stream, int* fields_per_c
  * 1e-16 are dropped in whole 16-node K tiles of the forward contraction and
  * whole 128-node row tiles of the inverse one (those rows are written as
  * zero).  FP64 plans drop whole 16-node K chunks of the forward sums and
- * whole 32-node row tiles of the inverse ones the same way.  on = 0
+ * whole row tiles of the inverse ones (32 to 128 nodes) the same way.  on = 0
  * restores the full sums.  Synchronises the device and rebuilds the plan's problem
  * and tile lists; groups that hold the plan keep working and follow the
  * setting, since the set of tiles does not change. */
@@ -322,7 +335,7 @@ int sht_plan_set_reduced(sht_plan_t plan, int on);
  * m with some |P~_n^m(mu_j)| >= 1e-16, and I_lat[j] = the smallest count
  * >= 4 M_j + 1 allowed by `rule`, capped at the plan's I.  SHT_REDUCED_SMOOTH
  * allows every even count whose half has no prime factor above 5 (fewest
- * points); SHT_REDUCED_FAST allows the counts 2 L whose half-length L has a
+ * points); SHT_REDUCED_FAST allows eight counts 2 L whose half-length L has a
  * compile-time FFT kernel (128, 256, 512, 640, 1024, 1280, 2048, 2560):
  * a few more points, far faster FFTs.  I_lat: host array of J ints,
  * written.  SHT_ERR_ARG for an unknown rule.  Synchronous.

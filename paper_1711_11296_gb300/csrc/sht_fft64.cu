@@ -24,7 +24,9 @@
 // Rounding (L = 1280, relative L2 error of the complex DFT, FP64 -> fixed
 // point): white noise 2.9e-16 -> 2.2e-16, a zonal flow with 1.5 % noise 1.7e-16
 // -> 0.8e-16 (the noise part alone 9.0e-16 -> 4.3e-16), a smooth row 1.8e-16
-// -> 1.0e-16, a single point 1.5e-16 -> 1.0e-16.
+// -> 1.0e-16, a single point 1.5e-16 -> 1.0e-16.  That is relative to the
+// latitude pair's largest value: what lies 2^-k below it keeps SH - k bits,
+// where FP64 keeps 53 of each input (and of a sum, those of its largest term).
 //
 // Rows with an infinity or a NaN give NaN throughout (the FP64 transform's
 // sums give NaN or an infinity).

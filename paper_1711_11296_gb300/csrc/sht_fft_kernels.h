@@ -31,7 +31,7 @@
 // the launch order, so their partial-sector writes of the same workspace
 // rows meet in L2.
 //
-// The half-lengths of the standard grids (64 ... 1280) have kernels
+// The half-lengths of the standard grids (fft_has_fixed_kernel) have kernels
 // specialised at compile time: radices, spans, twiddle offsets and the
 // digit reversal are constants, so the index arithmetic needs no integer
 // division by a runtime value.  Other lengths use the same code with the
@@ -41,7 +41,8 @@
 // 4, 2, 3, 5 through shared memory took 1.2 to 1.8 times as long (forward /
 // inverse us for 64 fields: T399, L = 800, 281 / 329 -> 207 / 207; T179, L = 360,
 // 81 / 82 -> 53 / 50; T119, L = 240, 51 / 46 -> 30 / 29).
-// Grouped launches branch per CTA to the body of their plan's length, and a
+// Grouped launches branch per CTA to the body of their plan's length (64, 128,
+// 256, 320, 512, 640, 1024, 1280; the run-time body for the others), and a
 // reduced grid launches the compile-time kernel once per row length it
 // contains, over a list of latitude pairs.
 #pragma once

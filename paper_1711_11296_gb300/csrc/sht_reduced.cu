@@ -7,7 +7,7 @@
 // every |P~_n^m(mu_j)| is below 1e-16.  sht_reduced_grid_sizes applies it
 // to a plan's P~ table: M_j = the largest m with some |P~_n^m(mu_j)| >=
 // 1e-16, and I_j = the smallest even count >= 4 M_j + 1 whose half has no
-// prime factor above 5 (SHT_REDUCED_SMOOTH), or whose half is one of the
+// prime factor above 5 (SHT_REDUCED_SMOOTH), or whose half is one of eight
 // lengths with a compile-time FFT kernel (SHT_REDUCED_FAST: fewer distinct
 // lengths, a few more points), capped at the plan's I.
 //
@@ -135,8 +135,8 @@ int attach_ragged(sht_plan_s* p, const int* I_lat, const int* shift) {
     rg->npts = acc;
     // Distinct (half-length, route) pairs, in order of first appearance from
     // the pole.  Unshifted rows whose half-length has a compile-time kernel
-    // go to that kernel; other 2-3-5-smooth rows to the generic kernel with
-    // radices up to 8; the rest to the Bluestein kernel.
+    // go to that kernel; other 2-3-5-smooth rows to the run-time kernel (FP32
+    // radices up to 32, FP64 2, 3, 4, 5 and 8); the rest to the Bluestein kernel.
     std::map<std::pair<int, int>, int> id;
     std::vector<RShape> shapes;
     std::vector<int> shape_of(p->Jh), shift_of(p->Jh), route_of;

@@ -296,7 +296,8 @@ class Plan:
 
 
 class Group:
-    """Several plans transformed by one launch per kernel stage.
+    """Several plans transformed by one launch per kernel stage (FP64
+    contractions: a launch or two per plan).
 
     ``forward(grids)`` / ``inverse(specs)`` take and return lists with one
     tensor per plan (each plan's own layouts).  The plans must outlive the
