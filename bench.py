@@ -438,8 +438,8 @@ def roofline_for(name, tot_ms, n, w, F, prec, pk, pk_src, npts=None, grid="cc"):
             roof = {"kernel": name + "_f64", "bound": "alu",
                     "achieved": b / per_launch_s / 1e9, "peak": None,
                     "unit": "GB/s", "traffic": None,
-                    "peak_source": "integer pipes (64-bit fixed point); HBM "
-                                   "figure for context"}
+                    "peak_source": "64-bit fixed point, bound by its phases' latency; "
+                                   "HBM figure for context"}
         else:
             roof = {"kernel": name + "_f32", "bound": "hbm",
                     "achieved": b / per_launch_s / 1e9, "peak": pk["hbm_gbs"],
