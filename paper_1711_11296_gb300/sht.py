@@ -255,7 +255,8 @@ class Plan:
 
     def set_tensor_tables(self, on=True):
         """Free those tables (the contractions then run on the FP64 pipe), or
-        build them whatever memory they take."""
+        build them whatever memory they take.  CUDA graphs captured before
+        must be captured again."""
         with torch.cuda.device(self.device):
             check(lib.sht_plan_set_tensor_tables(self._h, 1 if on else 0))
 
