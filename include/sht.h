@@ -135,8 +135,10 @@ int sht_plan_destroy(sht_plan_t plan);
  * sht_plan_get_tensor_tables writes whether the plan has them (*on = 1 or 0)
  * and their bytes; either pointer may be NULL.  sht_plan_set_tensor_tables frees
  * them (on = 0), or builds them whatever they take (on != 0; SHT_ERR_ALLOC leaves
- * the plan without).  Synchronises the device; groups that hold the plan follow, CUDA
- * graphs captured before must be captured again.  SHT_ERR_UNSUPPORTED for split plans and for plans outside the range above. */
+ * the plan without).  Synchronises the device; groups that hold the plan follow,
+ * CUDA graphs captured before must be captured again.  SHT_ERR_UNSUPPORTED for
+ * split plans and for plans outside the range above.
+ */
 int sht_plan_set_tensor_tables(sht_plan_t plan, int on);
 int sht_plan_get_tensor_tables(sht_plan_t plan, int* on, size_t* bytes);
 
