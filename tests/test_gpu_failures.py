@@ -12,7 +12,7 @@ import torch
 
 import oracle as O
 from paper_1711_11296_gb300 import workloads as W
-from sht_testutil import assert_fp64_close, built_lib, rel_l2, to_cuda
+from sht_testutil import built_lib, rel_l2, to_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -60,6 +60,9 @@ def test_injected_allocation_failure(sht):
     x = W.random_grid(2, 65, 128, seed=1702)
     assert rel_l2(p.forward(to_cuda(x, torch.float64)).cpu().numpy(), O.analysis(x, 31)) < 1e-12
 
+
+# ---- the FP64 plans' tensor-core tables ----
+from sht_testutil import assert_fp64_close  # noqa: E402
 
 # Plans whose contractions are sliced; the last one's columns and nodes fill no tile.
 SLICED = [(63, 129, 256, 64), (40, 71, 96, 321), (62, 131, 128, 65)]
